@@ -433,13 +433,13 @@ def mgt_remesh(pos, rho, r_max, max_level, n_side, stream=None):
     rho = np.ascontiguousarray(rho, np.float64)
     n = pos.shape[0]
     k = _i64(0)
-    _check(load().mgt_remesh(n, _ptr(pos), _ptr(rho), float(r_max), int(max_level), int(n_side), None, None, 0,
-                             ctypes.byref(k), _stream(stream)), "mgt_remesh")
-    out = np.zeros((k.value, 3), np.float64)
-    flags = np.zeros(k.value, np.uint8)
+    # one call: at most one box per point, and the surface nodes of the lattice
+    cap = n + max(0, 6 * int(n_side) ** 2 - 12 * int(n_side) + 8)
+    out = np.empty((cap, 3), np.float64)
+    flags = np.empty(cap, np.uint8)
     _check(load().mgt_remesh(n, _ptr(pos), _ptr(rho), float(r_max), int(max_level), int(n_side), _ptr(out),
-                             _ptr(flags), k.value, ctypes.byref(k), _stream(stream)), "mgt_remesh")
-    return out, flags
+                             _ptr(flags), cap, ctypes.byref(k), _stream(stream)), "mgt_remesh")
+    return out[:k.value].copy(), flags[:k.value].copy()
 
 
 def _check_noalloc_tensors(iterates, prediction):

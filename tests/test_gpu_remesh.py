@@ -53,3 +53,21 @@ def test_remesh_rejects_bad_input(mgt):
         mgt.mgt_remesh(pos, np.array([1.0, 2.0, -1.0, 1.0]), 0.4, 5, 3)
     with pytest.raises(mgt.MgtError):
         mgt.mgt_remesh(pos, np.ones(4), 0.4, 5, 1)
+
+
+@pytest.mark.parametrize("n", [1, 31, 511, 512, 513, 1025, 20000])
+def test_remesh_unit_edges(mgt, n):
+    # boxes of one point, of less and more than a warp, and on both sides of
+    # the 512 points of one warp's unit; clustered positions (boxes of very
+    # different sizes on one level) and coordinates of both signs with exact
+    # zeros.  Bounds, midpoints and counts are exact: equality, no tolerance
+    rng = np.random.default_rng(100 + n)
+    pos = np.concatenate([rng.normal(size=(n - n // 2, 3)) * 1e-3, rng.uniform(-1, 1, size=(n // 2, 3))])
+    pos[::7] = 0.0
+    pos[::11] *= -1.0
+    rho = np.exp(rng.normal(size=n))
+    out, flags = mgt.mgt_remesh(pos, rho, 0.3, 9, 3)
+    ref, rflags, _ = O.remesh(pos, rho, 0.3, 9, 3)
+    assert out.shape == ref.shape and np.array_equal(flags, rflags)
+    assert np.array_equal(_sorted(out[flags == 0]), _sorted(ref[rflags == 0]))
+    assert np.array_equal(out[flags == 1], ref[rflags == 1])
