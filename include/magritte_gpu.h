@@ -189,7 +189,7 @@ mgt_status mgt_set_solve_opts(mgt_model *m, const mgt_solve_opts *opts);
  * prove the FP64 predicates agree; the others are evaluated in FP64.
  * Stores the ray geometry on the device.  `stats` (host, may be NULL) is
  * filled after a stream synchronisation.  The walk's working memory (one
- * record slot per walk and step, a few GB for 10^5 points and 48 rays) comes
+ * index slot per walk, a few GB for 10^5 points and 48 rays) comes
  * from a memory pool of this library, one per device, that keeps it reserved
  * for the next trace of any model; the reserve is returned to the driver when
  * the last model on that device is destroyed.  The model's ray buffer (16 B

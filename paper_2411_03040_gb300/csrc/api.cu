@@ -334,7 +334,7 @@ static mgt_status validate(const mgt_model_desc *d)
 
 static void free_model(mgt_model *m)
 {
-    void *ptrs[] = {m->d_dir_map, m->d_batch_pairs, m->d_nbr_pos, m->d_ent, m->d_ent_off, m->d_pos_hl, m->d_vel_hl, m->d_dirs32, m->d_order, m->d_pos, m->d_vel, m->d_temp, m->d_vturb2, m->d_ncoll, m->d_nspec, m->d_w64, m->d_w32, m->d_dxmax,
+    void *ptrs[] = {m->d_dir_map, m->d_batch_pairs, m->d_nbr_pos, m->d_ent, m->d_ent_row, m->d_pos_hl, m->d_vel_hl, m->d_dirs32, m->d_order, m->d_pos, m->d_vel, m->d_temp, m->d_vturb2, m->d_ncoll, m->d_nspec, m->d_w64, m->d_w32, m->d_dxmax,
                     m->d_nbr_off, m->d_nbrs, m->d_bnd, m->d_dirs, m->d_pairs, m->d_xq, m->d_wq, m->d_line_tab,
                     m->d_line_ul, m->d_level_tab, m->d_coll_tab, m->d_coll_ul, m->d_entry, m->d_pops,
                     m->d_pops_prev, m->d_line32, m->d_line64, m->d_J, m->d_Lst, m->d_err, m->d_range_bad, m->d_count,
@@ -515,21 +515,20 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
         m->pos_scale = std::ldexp(1.0, -ex);
         // |xs - (hi + lo)| <= 2^-24 |lo| <= 2^-48 |xs| <= 2^-48; four times that, for both endpoints
         m->pos_slack = (float)std::ldexp(1.0, -46);
-        // packed walk rows: every point's neighbours in CSR order, the last one
-        // flagged; an empty row holds one kEntEmpty entry; 16 pad entries
-        std::vector<int32_t> eoff(N);
-        int64_t ne = 0;
+        // packed walk rows: every point's neighbours in CSR order, in whole
+        // chunks of kWalkRow entries (at least one); nnz + N < 2^31, so the
+        // chunk numbers fit 32 bits
+        std::vector<int32_t> row(N);
+        int64_t nc = 0;
         for (int64_t i = 0; i < N; ++i) {
-            eoff[i] = (int32_t)ne;
+            row[i] = (int32_t)nc;
             const int64_t deg = d->nbr_offsets[i + 1] - d->nbr_offsets[i];
-            ne += deg > 0 ? deg : 1;
+            nc += deg > 0 ? (deg + kWalkRow - 1) / kWalkRow : 1;
         }
-        // the packed entries carry their rows' offsets as 32-bit integers
-        if (ne + 16 > (int64_t)0x7fffffff) return set_error(MGT_ERR_ARG, "more than 2^31 - 1 neighbour entries");
-        m->n_ent = ne + 16;
-        MGT_TRY(dalloc(&m->d_ent, 2 * (size_t)m->n_ent));
-        MGT_TRY(dalloc(&m->d_ent_off, (size_t)N));
-        MGT_TRY(upload(m->d_ent_off, eoff.data(), (size_t)N, s));
+        m->n_chunks = (int32_t)nc;
+        MGT_TRY(dalloc(&m->d_ent, 2 * kWalkRow * (size_t)nc));
+        MGT_TRY(dalloc(&m->d_ent_row, (size_t)N));
+        MGT_TRY(upload(m->d_ent_row, row.data(), (size_t)N, s));
         std::vector<float4> d32(m->R);
         for (int r = 0; r < m->R; ++r)
             d32[r] = make_float4((float)d->dirs[3 * r], (float)d->dirs[3 * r + 1], (float)d->dirs[3 * r + 2], 0.0f);

@@ -39,7 +39,7 @@ mgt_status launch_widths(mgt_model *m, cudaStream_t s)
 // positions, velocities, neighbour lists and boundary mask):
 //  * positions times pos_scale and v/c, each split into float hi + lo;
 //  * the FP64 position of every neighbour entry;
-//  * the packed neighbour rows (see WalkEntry in mgt_common.cuh);
+//  * the packed neighbour rows (see kWalkRow in mgt_common.cuh);
 //  * the Morton (Z-curve) visiting order of the points: 21 bits per axis of
 //    the point's place in the bounding box, sorted with ties to the lower
 //    index.
@@ -82,29 +82,26 @@ __device__ __forceinline__ void put_entry(float4 *ent, int64_t e, const float *p
     ent[2 * e + 1] = make_float4(v[4], v[5], __uint_as_float(word), __int_as_float(noff));
 }
 
-// One thread per point (rows of ~15 entries), then the 16 pad entries.
-__global__ void k_pack_rows(int64_t N, int64_t ne, const int32_t *__restrict__ off, const int32_t *__restrict__ nb,
+// One thread per point (rows of ~15 entries).  A row is padded with empty
+// entries to whole chunks of kWalkRow entries (one 128-byte line), and every
+// entry of a row's last chunk carries the last-of-row flag.
+__global__ void k_pack_rows(int64_t N, const int32_t *__restrict__ off, const int32_t *__restrict__ nb,
                             const uint8_t *__restrict__ bnd, const float *__restrict__ phl,
-                            const int32_t *__restrict__ eoff, float4 *__restrict__ ent)
+                            const int32_t *__restrict__ row, float4 *__restrict__ ent)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= N + 16) return;
-    if (i >= N) {
-        put_entry(ent, ne + (i - N), phl, -1, kEntEmpty | kEntLast, 0);
-        return;
-    }
-    const int32_t k0 = off[i], k1 = off[i + 1];
-    const int64_t e0 = eoff[i];
-    if (k1 == k0) {
-        put_entry(ent, e0, phl, -1, kEntEmpty | kEntLast, 0);
-        return;
-    }
-    for (int32_t k = k0; k < k1; ++k) {
-        const int32_t mpt = nb[k];
-        uint32_t word = (uint32_t)mpt;
-        if (k == k1 - 1) word |= kEntLast;
-        if (bnd[mpt]) word |= kEntBnd;
-        put_entry(ent, e0 + (k - k0), phl, mpt, word, eoff[mpt]);
+    if (i >= N) return;
+    const int32_t k0 = off[i], deg = off[i + 1] - k0;
+    const int64_t e0 = (int64_t)row[i] * kWalkRow;
+    const int32_t n = max(1, (deg + kWalkRow - 1) / kWalkRow) * kWalkRow;
+    for (int32_t k = 0; k < n; ++k) {
+        const uint32_t last = k >= n - kWalkRow ? kEntLast : 0u;
+        if (k >= deg) {
+            put_entry(ent, e0 + k, phl, -1, kEntEmpty | last, 0);
+            continue;
+        }
+        const int32_t mpt = nb[k0 + k];
+        put_entry(ent, e0 + k, phl, mpt, (uint32_t)mpt | last | (bnd[mpt] ? kEntBnd : 0u), row[mpt]);
     }
 }
 
@@ -172,8 +169,8 @@ mgt_status build_walk_tables(mgt_model *m, const double lo[3], const double hi[3
         k_nbr_pos<<<ceil_div(3 * m->nnz, 256), 256, 0, s>>>(m->nnz, m->d_nbrs, m->d_pos, m->d_nbr_pos);
         MGT_LAUNCH_CHECK("k_nbr_pos");
     }
-    k_pack_rows<<<ceil_div(N + 16, 128), 128, 0, s>>>(N, m->n_ent - 16, m->d_nbr_off, m->d_nbrs, m->d_bnd,
-                                                      m->d_pos_hl, m->d_ent_off, m->d_ent);
+    k_pack_rows<<<ceil_div(N, 128), 128, 0, s>>>(N, m->d_nbr_off, m->d_nbrs, m->d_bnd, m->d_pos_hl, m->d_ent_row,
+                                                 m->d_ent);
     MGT_LAUNCH_CHECK("k_pack_rows");
     // Morton order: keys, then a stable radix sort of (key, index)
     uint64_t *keys = nullptr;
@@ -429,15 +426,14 @@ struct WalkArgs {
     double pos_scale;         // power of two near 1 / (largest coordinate): exact scaling
     const uint8_t *bnd;
     const double *dirs;
-    const float4 *ent;        // packed neighbour entries, two float4 each (WalkEntry layout)
-    const int32_t *ent_off;   // [N] first packed entry of each point's row
+    const float4 *ent;        // packed neighbour entries, two float4 each (see kWalkRow)
+    const int32_t *ent_row;   // [N] first chunk of each point's row of packed entries
     const float *pos_hl;      // [N][6] positions times pos_scale, split into float hi + lo
     const float4 *dirs32;     // [R] directions in FP32
     const int32_t *order;     // walks of one direction are visited in this point order
     float pos_slack;          // bound on |x - (hi + lo)| over all coordinates
     unsigned long long *n_exact;   // steps decided by the FP64 predicates
-    int32_t max_row_chunks;   // bound on the 16-entry chunks of one row scan (packed entries / 16 + 2)
-    int64_t n_ent;            // packed entries (index bound)
+    int32_t n_chunks;         // chunks of packed entries (index bound)
     const int32_t *dir_map;   // walk direction r -> model direction (NULL: the same); R counts walk directions
 };
 
@@ -463,33 +459,56 @@ __device__ __forceinline__ double dot3_exact(double ax, double ay, double az, do
     return __dadd_rn(__dadd_rn(__dmul_rn(ax, bx), __dmul_rn(ay, by)), __dmul_rn(az, bz));
 }
 
-// Next point of the walk from c in FP64, the defining arithmetic, or -1.
-// Writes the winner's Z and its neighbour-entry index.
-__device__ __noinline__ int64_t walk_next_exact(const WalkArgs &a, int64_t c, double xo, double yo, double zo, double n0,
-                                                double n1, double n2, double Zc, double *Znext)
+// Next point of the walk from c in FP64, the defining arithmetic, or -1, found
+// by the whole warp (every argument the same in every lane): one candidate per
+// lane, the least (squared distance, index) over the lanes.  Returned with the
+// winner's Z in every lane.  One lane alone took ~15 times the FP64 warp
+// instructions, and an instruction costs this GPU's FP64 pipe the same 16
+// cycles for one lane as for 32.
+__device__ __noinline__ int walk_next_exact(const int32_t *__restrict__ off, const int32_t *__restrict__ nb,
+                                            const double *__restrict__ nb_pos, int c, double xo, double yo, double zo,
+                                            double n0, double n1, double n2, double Zc, double *Znext)
 {
-    int64_t best = -1;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int32_t k0 = off[c], k1 = off[c + 1];
+    int best = 0x7fffffff;
     double bestd = 0.0, bestZ = 0.0;
-    const int32_t k1 = a.off[c + 1];
-    for (int32_t k = a.off[c]; k < k1; ++k) {
-        int64_t mm = a.nb[k];
-        double dx = __dsub_rn(a.nb_pos[3 * (int64_t)k], xo);
-        double dy = __dsub_rn(a.nb_pos[3 * (int64_t)k + 1], yo);
-        double dz = __dsub_rn(a.nb_pos[3 * (int64_t)k + 2], zo);
-        double Z = dot3_exact(dx, dy, dz, n0, n1, n2);
+    bool have = false;
+    for (int32_t kb = k0; kb < k1; kb += 32) {
+        const int32_t k = kb + lane;
+        if (k >= k1) continue;
+        const int mm = nb[k];
+        const double dx = __dsub_rn(nb_pos[3 * (int64_t)k], xo);
+        const double dy = __dsub_rn(nb_pos[3 * (int64_t)k + 1], yo);
+        const double dz = __dsub_rn(nb_pos[3 * (int64_t)k + 2], zo);
+        const double Z = dot3_exact(dx, dy, dz, n0, n1, n2);
         if (!(Z > Zc)) continue;
-        double px = __dsub_rn(dx, __dmul_rn(Z, n0));
-        double py = __dsub_rn(dy, __dmul_rn(Z, n1));
-        double pz = __dsub_rn(dz, __dmul_rn(Z, n2));
-        double d2 = dot3_exact(px, py, pz, px, py, pz);
-        if (best < 0 || d2 < bestd || (d2 == bestd && mm < best)) {
+        const double px = __dsub_rn(dx, __dmul_rn(Z, n0));
+        const double py = __dsub_rn(dy, __dmul_rn(Z, n1));
+        const double pz = __dsub_rn(dz, __dmul_rn(Z, n2));
+        const double d2 = dot3_exact(px, py, pz, px, py, pz);
+        if (!have || d2 < bestd || (d2 == bestd && mm < best)) {
+            have = true;
             best = mm;
             bestd = d2;
             bestZ = Z;
         }
     }
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool oh = __shfl_xor_sync(full, have, o);
+        const int ob = __shfl_xor_sync(full, best, o);
+        const double od = __shfl_xor_sync(full, bestd, o), oz = __shfl_xor_sync(full, bestZ, o);
+        if (oh && (!have || od < bestd || (od == bestd && ob < best))) {
+            have = true;
+            best = ob;
+            bestd = od;
+            bestZ = oz;
+        }
+    }
     *Znext = bestZ;
-    return best;
+    return have ? best : -1;
 }
 
 // Per-walk constants, all FP32 (GB300's FP64 pipe is far too narrow for
@@ -518,59 +537,36 @@ __device__ __forceinline__ WalkFrame make_frame(const WalkArgs &a, int64_t o, in
 }
 
 
-// Step records of `cnt` consecutive steps, one per lane of a 16-lane group
-// (the whole warp calls; cnt = 0 in a group with nothing to write): lane j < cnt writes the record of the step
-// ending at its point my_pt, the step starting at the previous lane's point
-// (prev_last for lane 0).  All in FP32: dx from the hi + lo scaled positions,
-// beta = n.(v_c - v_o)/c and dbeta = n.(v_c - v_prev)/c from hi + lo values
-// of v/c (relative error about 1e-7 of |v_c - v_o|/c), the averaged width of
-// the segment.
-__device__ __forceinline__ void write_step_records(const WalkArgs &a, int64_t o, int r, int64_t prev_last,
-                                                   int32_t my_pt, int cnt, const float *__restrict__ vel_hl,
-                                                   const float2 *__restrict__ w32, float inv_Lunit, int width_mode,
-                                                   Step32 *__restrict__ out, int sl)
+// 32 bytes at a 32-byte aligned address of read-only memory, in one load.
+struct Vec8 {
+    float4 a, b;
+};
+
+__device__ __forceinline__ Vec8 load32(const void *p)
 {
-    int64_t prev = __shfl_up_sync(0xffffffffu, my_pt, 1, 16);
-    if (sl == 0) prev = prev_last;
-    if (sl >= cnt) return;
-    const int64_t c = my_pt;
-    const float *pc = a.pos_hl + 6 * c, *pp = a.pos_hl + 6 * prev;
-    const float *vc = vel_hl + 6 * c, *vp = vel_hl + 6 * prev, *vo = vel_hl + 6 * o;
-    const float4 n = a.dirs32[r];
-    float e[3], db[3], dp[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        e[d] = (pc[d] - pp[d]) + (pc[3 + d] - pp[3 + d]);
-        db[d] = (vc[d] - vo[d]) + (vc[3 + d] - vo[3 + d]);
-        dp[d] = (vc[d] - vp[d]) + (vc[3 + d] - vp[3 + d]);
-    }
-    const float dxs = sqrtf(fmaf(e[2], e[2], fmaf(e[1], e[1], e[0] * e[0]))) * inv_Lunit;
-    const float beta = fmaf(n.z, db[2], fmaf(n.y, db[1], n.x * db[0]));
-    const float dbeta = fmaf(n.z, dp[2], fmaf(n.y, dp[1], n.x * dp[0]));
-    const float wc = w32[c].x, wp = w32[prev].x;
-    const float wbar = width_mode == 0 ? sqrtf(0.5f * (wc * wc + wp * wp)) : 0.5f * (wc + wp);
-    out[sl] = make_int4((int)c, __float_as_int(dxs), __float_as_int(beta), __float_as_int(dbeta / wbar));
+    Vec8 v;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z), "=f"(v.b.w)
+        : "l"(p));
+    return v;
 }
 
-// Minimum over the calling lane's 16-lane group of a non-negative float: two
-// whole-warp integer min-reductions (non-negative floats order like their bit
-// patterns), each lane keeping its own group's.  One reduction instruction per
-// group instead of four dependent shuffle-and-min steps.
-__device__ __forceinline__ float group16_min_nonneg(float v, int grp)
+// Minimum over the calling lane's walk (a group of G lanes).
+template <int G> __device__ __forceinline__ float group_min(float v)
 {
-    const unsigned k = __float_as_uint(v);
-    const unsigned k0 = __reduce_min_sync(0xffffffffu, grp == 0 ? k : 0xffffffffu);
-    const unsigned k1 = __reduce_min_sync(0xffffffffu, grp == 1 ? k : 0xffffffffu);
-    return __uint_as_float(grp ? k1 : k0);
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
 // ---------------------------------------------------------------------------
-// Two walks per warp, one per 16-lane group.  Each step reads the current
-// point's row of packed neighbour entries (WalkEntry: the neighbour's scaled
-// position as float hi + lo, its index with its boundary flag and a
-// last-of-row flag, and the offset of its own row), 16 entries per load, so
-// the next step's row offset, the winner's index and its boundary flag arrive
-// with the candidates: one dependent L2 round trip per step.
+// One walk per group of G lanes: eight walks per warp (G = kWalkRow = 4), or two
+// (G = 16) in launches of few walks, see walk_wide.  Each step reads
+// the current point's row of packed neighbour entries (the neighbour's scaled
+// position as float hi + lo, its index with its boundary flag and a last-chunk
+// flag, and its own row), G / 4 chunks (128-byte lines) per load and group, so
+// the next step's row, the winner's index and its boundary flag arrive with
+// the candidates: one dependent L2 round trip per load.
 //
 // The lanes evaluate the candidates with FP32 arithmetic and error bounds that
 // cover both the FP32 and the FP64 rounding (generous multiples of the
@@ -586,16 +582,16 @@ __device__ __forceinline__ float group16_min_nonneg(float v, int grp)
 // lane) is accepted only if its upper d2 bound is below every other
 // candidate's lower bound, so near-ties never decide.  Undecided steps run
 // walk_next_exact, the FP64 predicates themselves (exact Z_c recomputed by
-// the same expression), on lane 0 of the group.  The point lists are
-// therefore those of the FP64 rule.
+// the same expression), one walk of the warp after the other.  The point lists
+// are therefore those of the FP64 rule.
 //
-// Two modes share the walk:
+// Four modes share the walk:
 //  * kWalkFused: every walk of the grid.  Writes the half-ray length, counts
-//    stalls, and writes the step records (see Step32), 16 at a time, into a
-//    fixed-stride scratch area (K records per walk); records of steps >= K are
-//    not kept (such walks are redone by the list mode).
-//  * kWalkList: the walks named in `list` only, records written to their final
-//    place (ray offsets known).
+//    stalls, and writes the point indices into a fixed-stride scratch area
+//    (K per walk); those of steps >= K are not kept (such walks are redone by
+//    the list mode).  k_walk_compact makes the step records from them.
+//  * kWalkList: the walks named in `list` only, point indices written into
+//    the records at their final place (ray offsets known).
 //  * kWalkImgCount / kWalkImgFill: the two half-rays of every image pixel
 //    (walk 2q + h: h = 0 along -n, h = 1 along +n, n toward the observer),
 //    from the pixel's anchor point, distances to the pixel line, Z measured
@@ -614,49 +610,61 @@ struct ImgWalkArgs {
     double n[3];              // unit direction toward the observer
 };
 
-// Blocks of 128 threads, eight per SM (registers capped at 64): the walk is
-// bound by dependent latency (L2 row loads, shuffle chains), and 32 resident
-// warps per SM beat the spill-free 93-register build at 16 (workload 2 trace:
-// 91 -> 73 ms; 128-thread blocks instead of 256 a further 3 %).  Every launch
-// uses kWalkThreads.
-constexpr int kWalkThreads = 128;
-template <int MODE>
-__global__ void __launch_bounds__(kWalkThreads, 8) k_walk(WalkArgs a, int64_t *__restrict__ lens, const int64_t *__restrict__ ray_off,
-                                              const int64_t *__restrict__ list, int64_t n_list, int32_t K,
-                                              unsigned long long *__restrict__ n_stall,
-                                              const float *__restrict__ vel_hl, const float2 *__restrict__ w32,
-                                              float inv_Lunit, int width_mode, Step32 *__restrict__ steps,
-                                              int *__restrict__ err, ImgWalkArgs im)
+// What bounds it: instruction issue (about 75 warp instructions per step at
+// 100k shell points) and the L2 round trips of the rows.  Four lanes per walk
+// read a row (15.5 entries on average) in its own 128-byte lines with few lanes
+// past its end; the decision's shuffles and the loop serve eight walks at once;
+// and walks of neighbouring origins step together, so their rows coincide in
+// L1.  Walk kernel, 100k shell points x 48 directions (1.9e8 steps): 36.9 ms
+// with 16 lanes per walk, records made inside, 64 registers; 16.0 ms with 4
+// lanes and the records left to k_walk_compact; 14.9 ms at 48 registers (ten
+// blocks of 128 threads per SM; 16.0 at eight, 18.8 at six, 17.5 at fourteen);
+// 14.4 ms with 256-bit loads.  8 lanes per walk: 18.7 ms, 2 lanes: 16.2 ms.
+// Not kept: loading the next chunk ahead (16.8 ms, a quarter of the loads
+// wasted), and giving a finished group the warp's next walk (16.7 ms: the
+// walks of a warp no longer pass the same rows together).
+// Every launch goes through launch_walk.
+constexpr int kWalkThreads = 128, kWalkBlocks = 10;
+
+template <int MODE, int G>
+__global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, int64_t *__restrict__ lens,
+                                                          const int64_t *__restrict__ ray_off,
+                                                          const int64_t *__restrict__ list, int64_t n_list, int32_t K,
+                                                          unsigned long long *__restrict__ n_stall,
+                                                          int32_t *__restrict__ scratch, Step32 *__restrict__ steps,
+                                                          int *__restrict__ err, ImgWalkArgs im)
 {
     constexpr bool IMG = MODE == kWalkImgCount || MODE == kWalkImgFill;
+    static_assert(G % kWalkRow == 0 && 32 % G == 0, "whole chunks per group, whole groups per warp");
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, sl = lane & 15, grp = lane >> 4;
-    const unsigned gmask = 0xffffu << (16 * grp);
-    const int64_t wg = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;   // walk slot
+    const int lane = threadIdx.x & 31, sl = lane & (G - 1), first = lane & ~(G - 1);
+    const unsigned gmask = ((1u << G) - 1u) << first;
+    const int64_t wg = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;   // walk slot
     const int64_t W = MODE == kWalkFused ? (int64_t)a.R * a.N : IMG ? 2 * im.npix : n_list;
-    if ((wg & ~(int64_t)1) >= W) return;                       // both walks of the warp absent
+    if (wg - first / G >= W) return;                           // every walk of the warp absent
     bool live = wg < W;
     int r = 0;
-    int64_t o = 0;
+    int64_t o64 = 0;
     if (live) {
         if (MODE == kWalkFused) {
             r = (int)(wg / a.N);
-            o = a.order[wg - (int64_t)r * a.N];
+            o64 = a.order[wg - (int64_t)r * a.N];
         } else if (IMG) {
             r = (int)(wg & 1);
-            o = im.anchor[wg >> 1];
+            o64 = im.anchor[wg >> 1];
         } else {
             const int64_t t = list[wg];
             r = (int)(t / a.N);
-            o = t - (int64_t)r * a.N;
+            o64 = t - (int64_t)r * a.N;
         }
     }
-    if (o < 0 || o >= a.N || r < 0 || r >= (IMG ? 2 : a.R)) {   // index check: record and skip
-        walk_give_up(err, 13, wg, o);
-        o = 0;
+    if (o64 < 0 || o64 >= a.N || r < 0 || r >= (IMG ? 2 : a.R)) {   // index check: record and skip
+        walk_give_up(err, 13, wg, o64);
+        o64 = 0;
         r = 0;
         live = false;
     }
+    const int o = (int)o64;
     const int64_t wi = (int64_t)r * a.N + o;
     const int rg = (!IMG && a.dir_map) ? a.dir_map[r] : r;   // the model's direction index
     // the walk's frame: origin o and direction r, or for image walks the pixel's
@@ -665,7 +673,7 @@ __global__ void __launch_bounds__(kWalkThreads, 8) k_walk(WalkArgs a, int64_t *_
     double img_Z0 = 0.0;                        // image walks: Z of the anchor
     if (IMG) {
         const double sg = r == 0 ? -1.0 : 1.0;
-        const double *pr = im.ref + 3 * (wg >> 1);
+        const double *pr = im.ref + 3 * (live ? wg >> 1 : 0);
         const double sx = pr[0] * a.pos_scale, sy = pr[1] * a.pos_scale, sz = pr[2] * a.pos_scale;
         f.ohx = (float)sx;
         f.ohy = (float)sy;
@@ -676,46 +684,47 @@ __global__ void __launch_bounds__(kWalkThreads, 8) k_walk(WalkArgs a, int64_t *_
         f.f0 = (float)(sg * im.n[0]);
         f.f1 = (float)(sg * im.n[1]);
         f.f2 = (float)(sg * im.n[2]);
-        const double *q = a.pos + 3 * o;
+        const double *q = a.pos + 3 * (int64_t)o;
         img_Z0 = dot3_exact(__dsub_rn(q[0], pr[0]), __dsub_rn(q[1], pr[1]), __dsub_rn(q[2], pr[2]), sg * im.n[0],
                             sg * im.n[1], sg * im.n[2]);
     } else {
         f = make_frame(a, o, rg);
     }
-    // records go to out[0 .. cap): the walk's scratch slot, or its final place
-    int64_t cap = K;
-    Step32 *out = steps + wi * (int64_t)K;
-    if (MODE == kWalkList && live) {
-        out = steps + ray_off[wi];
-        cap = ray_off[wi + 1] - ray_off[wi];
-    }
-    if (IMG) cap = a.N;
-    int64_t img_nfar = 0, img_base = 0;         // fill: far-half length and the pixel's ray offset
-    if (MODE == kWalkImgFill && live) {
-        img_nfar = lens[wg & ~(int64_t)1];
-        img_base = im.off[wg >> 1];
-        cap = lens[wg];
-    }
-    // step records are built 16 at a time: lane j of the group keeps the point
-    // of step (chunk start + j); prev_last is the point before the chunk
-    int32_t my_pt = 0;
-    int64_t prev_last = o;
-    int64_t c = o, n = 0;
-    int32_t c_off = live ? a.ent_off[o] : 0;   // the current point's row of packed entries
+    int c = o, n = 0;                           // current point, steps taken
+    int c_row = live ? a.ent_row[o] : 0;        // the current point's row of packed entries
     float Zc = 0.0f, eZc = 0.0f;                // Z of o is exactly 0 (image walks: the anchor's Z)
     if (IMG) {
         Zc = (float)(img_Z0 * a.pos_scale);     // the filter works in scaled units (exact factor)
         eZc = 1e-7f * fabsf(Zc) + 1e-30f;
     }
-    bool done = !live;
+    // where point index k goes (lane sl keeps the index of step k = sl mod G
+    // until the group's G indices are written together)
+    auto put = [&](int k, int32_t pt) {
+        if (MODE == kWalkFused) {
+            if (k < K) scratch[wi * (int64_t)K + k] = pt;
+        } else if (MODE == kWalkList) {
+            const int64_t at = ray_off[wi] + k;
+            if (at < ray_off[wi + 1])
+                steps[at].x = pt;
+            else
+                atomicCAS(err, 0, (int)kDevBounds);    // cannot happen: deterministic walk
+        } else if (MODE == kWalkImgFill) {
+            const int nfar = (int)lens[wg & ~(int64_t)1];
+            if (k < (int)lens[wg])
+                im.pts[im.off[wg >> 1] + (r == 0 ? nfar - 1 - k : nfar + 1 + k)] = pt;
+            else
+                atomicCAS(err, 0, (int)kDevBounds);
+        }
+    };
+    int32_t my_pt = 0;
+    bool done = !live, gave_up = false;
     // every loop below is bounded: the walk by the point count and a 2 s
-    // clock, a row scan by the number of packed entries; running out records
-    // the site and returns
+    // clock, a row scan by the number of chunks; running out records the site
+    // and returns.  All live walks of the warp have taken `it` steps.
     const uint64_t t_start = walk_clock_ns();
-    bool gave_up = false;
-    uint32_t iter = 0;                          // the same in every lane (the loop test is a warp vote)
-    while (!__all_sync(full, done)) {
-        if ((++iter & 15u) == 0u && __any_sync(full, walk_clock_ns() - t_start > 2000000000ull)) {
+    int it = 0;
+    for (; __any_sync(full, !done); ++it) {
+        if ((it & 15) == 15 && __any_sync(full, walk_clock_ns() - t_start > 2000000000ull)) {
             if (sl == 0 && !done) walk_give_up(err, 1, wg, n);
             gave_up = true;
             break;
@@ -725,128 +734,132 @@ __global__ void __launch_bounds__(kWalkThreads, 8) k_walk(WalkArgs a, int64_t *_
         // of its other candidates; the group decides once per step
         float bd2 = 3.0e38f, bU = 0.0f, bLo = 3.0e38f, bZ = 0.0f, beZ = 0.0f, lo2 = 3.0e38f;
         uint32_t bword = 0u;
-        int32_t boff = 0;
-        bool und_lane = false, row_open = !done;
-        int32_t chunks = 0;
-        for (int32_t kb = c_off; __any_sync(full, row_open); kb += 16) {
-            if (++chunks > a.max_row_chunks) {
-                if (sl == 0 && row_open) walk_give_up(err, 2, wg, n);
-                gave_up = true;
-                break;
-            }
-            bool last = false;
-            uint32_t word = 0u;
-            int32_t eoff = 0;
-            float4 e0 = make_float4(0.f, 0.f, 0.f, 0.f), e1 = e0;
-            if (row_open && (kb + sl < 0 || kb + sl >= a.n_ent)) {   // index check: record and skip
-                walk_give_up(err, 10, wg, kb + sl);
-                row_open = false;
-            }
-            if (row_open) {
-                const float4 *ep = reinterpret_cast<const float4 *>(a.ent + 2 * (int64_t)(kb + sl));
-                e0 = ep[0];
-                e1 = ep[1];
-                word = __float_as_uint(e1.z);
-                eoff = __float_as_int(e1.w);
-                last = (word & kEntLast) != 0u;
-            }
-            // entries up to the group's first last-of-row flag belong to the row
-            const unsigned lastbits = (__ballot_sync(full, last) & gmask) >> (16 * grp);
-            const bool inrow = row_open && (lastbits & ((1u << sl) - 1u)) == 0u;
-            if (inrow && (word & kEntIdx) != kEntEmpty) {
-                const float dx = (e0.x - f.ohx) + (e0.w - f.olx);
-                const float dy = (e0.y - f.ohy) + (e1.x - f.oly);
-                const float dz = (e0.z - f.ohz) + (e1.y - f.olz);
-                const float adx = fabsf(dx), ady = fabsf(dy), adz = fabsf(dz);
-                const float ed = 2e-6f * (fmaxf(adx, fmaxf(ady, adz)) + a.pos_slack);
-                const float Z = fmaf(dz, f.f2, fmaf(dy, f.f1, dx * f.f0));
-                const float eZ = 2e-6f * (adx + ady + adz) + 2.0f * ed;
-                if (Z - eZ > Zc + eZc) {
-                    const float px = fmaf(-Z, f.f0, dx), py = fmaf(-Z, f.f1, dy), pz = fmaf(-Z, f.f2, dz);
-                    const float d2 = fmaf(pz, pz, fmaf(py, py, px * px));
-                    const float ep = ed + eZ + 2e-7f * (fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))) + fabsf(Z));
-                    // |p32| from the approximate square root, raised by 2^-10
-                    // (far above its error) so that the bound stays an upper one
-                    float rp;
-                    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(d2));
-                    const float e2 = 4.0f * (rp * 1.0009765625f) * ep + 4.0f * ep * ep + 1e-6f * d2;
-                    const float U = d2 + e2, Lo = d2 - e2;
-                    if (d2 < bd2) {
-                        lo2 = fminf(lo2, bLo);
-                        bd2 = d2;
-                        bU = U;
-                        bLo = Lo;
-                        bZ = Z;
-                        beZ = eZ;
-                        bword = word;
-                        boff = eoff;
-                    } else {
-                        lo2 = fminf(lo2, Lo);
-                    }
-                } else if (!(Z + eZ <= Zc - eZc)) {
-                    und_lane = true;
+        int brow = 0;
+        bool und = false;
+        const float Zhi = Zc + eZc, Zlo = Zc - eZc;
+        auto candidate = [&](const float4 &e0, const float4 &e1) {
+            const uint32_t word = __float_as_uint(e1.z);
+            if ((word & kEntIdx) == kEntEmpty) return;
+            const float dx = (e0.x - f.ohx) + (e0.w - f.olx);
+            const float dy = (e0.y - f.ohy) + (e1.x - f.oly);
+            const float dz = (e0.z - f.ohz) + (e1.y - f.olz);
+            const float adx = fabsf(dx), ady = fabsf(dy), adz = fabsf(dz);
+            const float ed = 2e-6f * (fmaxf(adx, fmaxf(ady, adz)) + a.pos_slack);
+            const float Z = fmaf(dz, f.f2, fmaf(dy, f.f1, dx * f.f0));
+            const float eZ = 2e-6f * (adx + ady + adz) + 2.0f * ed;
+            if (Z - eZ > Zhi) {
+                const float px = fmaf(-Z, f.f0, dx), py = fmaf(-Z, f.f1, dy), pz = fmaf(-Z, f.f2, dz);
+                const float d2 = fmaf(pz, pz, fmaf(py, py, px * px));
+                const float ep_ = ed + eZ + 2e-7f * (fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))) + fabsf(Z));
+                // |p32| from the approximate square root, raised by 2^-10
+                // (far above its error) so that the bound stays an upper one
+                float rp;
+                asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(d2));
+                const float e2 = 4.0f * (rp * 1.0009765625f) * ep_ + 4.0f * ep_ * ep_ + 1e-6f * d2;
+                const float Lo = d2 - e2;
+                if (d2 < bd2) {
+                    lo2 = fminf(lo2, bLo);
+                    bd2 = d2;
+                    bU = d2 + e2;
+                    bLo = Lo;
+                    bZ = Z;
+                    beZ = eZ;
+                    bword = word;
+                    brow = __float_as_int(e1.w);
+                } else {
+                    lo2 = fminf(lo2, Lo);
                 }
+            } else if (!(Z + eZ <= Zlo)) {
+                und = true;
             }
-            row_open = row_open && lastbits == 0u;
+        };
+        if constexpr (G == kWalkRow) {
+            for (int kb = done ? -1 : c_row; kb != -1;) {
+                if ((unsigned)kb >= (unsigned)a.n_chunks) {    // index check: record and end the row
+                    walk_give_up(err, 10, wg, kb);
+                    break;
+                }
+                const Vec8 e = load32(a.ent + 2 * ((int64_t)kb * kWalkRow + sl));
+                // (the same in every lane of the group)
+                kb = (__float_as_uint(e.b.z) & kEntLast) ? -1 : kb + 1;
+                candidate(e.a, e.b);
+            }
+        } else {
+            bool open = !done;
+            for (int kb = c_row; __any_sync(full, open); kb += G / kWalkRow) {
+                if (open && (unsigned)kb >= (unsigned)a.n_chunks) {
+                    walk_give_up(err, 10, wg, kb);
+                    open = false;
+                }
+                const int chunk = kb + sl / kWalkRow;
+                const bool in = open && chunk < a.n_chunks;
+                Vec8 e{};
+                if (in) e = load32(a.ent + 2 * ((int64_t)chunk * kWalkRow + sl % kWalkRow));
+                // chunks up to the group's first one with the last-chunk flag belong to the row
+                const unsigned last = __ballot_sync(full, in && (__float_as_uint(e.b.z) & kEntLast)) & gmask;
+                if (in && (last & ((1u << (lane & ~(kWalkRow - 1))) - 1u)) == 0u) candidate(e.a, e.b);
+                open = open && last == 0u;
+            }
         }
-        if (gave_up) break;
-        // The decision runs in both groups in lockstep (a finished group only
-        // predicates itself off), so every warp intrinsic below names the
-        // whole warp.  The FP32 winner is the group's smallest d2 (lowest lane
-        // on ties); it is accepted only if every other candidate's lower bound
-        // lies above its upper bound (a negative lower bound always fails,
-        // since upper bounds are >= 0), so a tie never decides.
-        const bool undecided = (__ballot_sync(full, und_lane) & gmask) != 0u;
-        const float m = group16_min_nonneg(bd2, grp);
-        const bool have = m < 3.0e38f;
-        const unsigned wins = (__ballot_sync(full, have && bd2 == m) & gmask) >> (16 * grp);
-        const int wl = wins ? __ffs(wins) - 1 : sl;
-        const int src = 16 * grp + wl;
+        __syncwarp();
+        // The FP32 winner is the group's smallest d2 (lowest lane on ties); it
+        // is accepted only if every other candidate's lower bound lies above
+        // its upper bound (a negative lower bound always fails, since upper
+        // bounds are >= 0), so a tie never decides.
+        const float dmin = group_min<G>(bd2);
+        const bool have = dmin < 3.0e38f;
+        const unsigned wins = __ballot_sync(full, have && bd2 == dmin) & gmask;
+        const int src = wins ? __ffs(wins) - 1 : lane;
         bU = __shfl_sync(full, bU, src);
         bZ = __shfl_sync(full, bZ, src);
         beZ = __shfl_sync(full, beZ, src);
         bword = __shfl_sync(full, bword, src);
-        boff = __shfl_sync(full, boff, src);
-        const float lo_other = sl == wl ? lo2 : fminf(bLo, lo2);
-        const bool close = (__ballot_sync(full, have && lo_other <= bU) & gmask) != 0u;
-        const bool exact = !done && (undecided || close);
-        int64_t v = -1;
+        brow = __shfl_sync(full, brow, src);
+        const float lo_other = lane == src ? lo2 : fminf(bLo, lo2);
+        // (every warp intrinsic runs in all lanes: none behind a short circuit)
+        const bool close = (__ballot_sync(full, und || (have && lo_other <= bU)) & gmask) != 0u;
+        const bool exact = !done && close;
+        int v = -1;
         double Zn = 0.0;
-        if (exact && sl == 0) {
-            // FP64 predicates, evaluated by lane 0 of the group
-            if (!IMG) atomicAdd(a.n_exact, 1ULL);
+        // (rare) the FP64 predicates, for one undecided walk after the other
+        for (unsigned todo = __ballot_sync(full, exact && sl == 0); todo; todo &= todo - 1u) {
+            const int w = __ffs(todo) - 1;
+            const int wo = __shfl_sync(full, o, w), wc = __shfl_sync(full, c, w), wr = __shfl_sync(full, rg, w);
+            if (!IMG && lane == 0) atomicAdd(a.n_exact, 1ULL);
             double xo, yo, zo, n0, n1, n2;
-            if (IMG) {
-                const double *pr = im.ref + 3 * (wg >> 1);
-                const double sg = r == 0 ? -1.0 : 1.0;
-                xo = pr[0];
-                yo = pr[1];
-                zo = pr[2];
+            if constexpr (IMG) {
+                const double *po = im.ref + 3 * (__shfl_sync(full, wg, w) >> 1);
+                const double sg = wr == 0 ? -1.0 : 1.0;
+                xo = po[0];
+                yo = po[1];
+                zo = po[2];
                 n0 = sg * im.n[0];
                 n1 = sg * im.n[1];
                 n2 = sg * im.n[2];
             } else {
-                xo = a.pos[3 * o];
-                yo = a.pos[3 * o + 1];
-                zo = a.pos[3 * o + 2];
-                n0 = a.dirs[3 * rg];
-                n1 = a.dirs[3 * rg + 1];
-                n2 = a.dirs[3 * rg + 2];
+                const double *po = a.pos + 3 * (int64_t)wo, *pn = a.dirs + 3 * wr;
+                xo = po[0];
+                yo = po[1];
+                zo = po[2];
+                n0 = pn[0];
+                n1 = pn[1];
+                n2 = pn[2];
             }
             double Zc64 = 0.0;
-            if (c != o || IMG) {
-                const double *q = a.pos + 3 * c;
+            if (wc != wo || IMG) {
+                const double *q = a.pos + 3 * (int64_t)wc;
                 Zc64 = dot3_exact(__dsub_rn(q[0], xo), __dsub_rn(q[1], yo), __dsub_rn(q[2], zo), n0, n1, n2);
             }
-            v = walk_next_exact(a, c, xo, yo, zo, n0, n1, n2, Zc64, &Zn);
+            double z;
+            const int nv = walk_next_exact(a.off, a.nb, a.nb_pos, wc, xo, yo, zo, n0, n1, n2, Zc64, &z);
+            if (first == w) {
+                v = nv;
+                Zn = z;
+            }
         }
-        if (__any_sync(full, exact)) {          // (rare) the FP64 result of lane 0 to its group
-            v = __shfl_sync(full, v, 16 * grp);
-            Zn = __shfl_sync(full, Zn, 16 * grp);
-        }
-        int64_t nx = -1;
-        bool nx_bnd = false;
         if (!done) {
+            int nx = -1;
+            bool nx_bnd = false;
             if (exact) {
                 nx = v;
                 if (nx >= a.N) {
@@ -855,76 +868,84 @@ __global__ void __launch_bounds__(kWalkThreads, 8) k_walk(WalkArgs a, int64_t *_
                 }
                 Zc = (float)(Zn * a.pos_scale);      // the filter works in scaled units (exact factor)
                 eZc = 1e-7f * fabsf(Zc) + 1e-30f;
-                nx_bnd = nx >= 0 && a.bnd[nx] != 0;
-                if (nx >= 0) c_off = a.ent_off[nx];
+                if (nx >= 0) {
+                    nx_bnd = a.bnd[nx] != 0;
+                    c_row = a.ent_row[nx];
+                }
             } else if (have) {
-                nx = (int64_t)(bword & kEntIdx);
-                if (nx >= a.N || boff < 0 || boff >= a.n_ent) {
+                nx = (int)(bword & kEntIdx);
+                if (nx >= a.N) {
                     walk_give_up(err, 12, wg, nx);
                     nx = -1;
                 }
                 nx_bnd = (bword & kEntBnd) != 0u;
-                c_off = boff;
+                c_row = brow;
                 Zc = bZ;
                 eZc = beZ;
             }
-        }
-        bool flush_full = false, flush_last = false;   // a full chunk of 16 records / the walk's tail
-        if (!done) {
             if (nx < 0) {
                 if (MODE == kWalkFused && sl == 0 && !(c == o && a.bnd[o])) atomicAdd(n_stall, 1ULL);
                 done = true;
-                flush_last = (n & 15) != 0;
-            } else if ((MODE == kWalkList || MODE == kWalkImgFill) && n >= cap) {   // cannot happen: deterministic walk
-                if (sl == 0) atomicCAS(err, 0, (int)kDevBounds);
-                done = true;
             } else {
-                if (sl == (int)(n & 15)) my_pt = (int32_t)nx;
-                flush_full = (n & 15) == 15;
+                if (sl == (it & (G - 1))) my_pt = nx;
                 ++n;
                 c = nx;
-                if (nx_bnd || n >= a.N) {
-                    done = true;
-                    flush_last = (n & 15) != 0;
-                }
+                done = nx_bnd || n >= a.N;
             }
         }
-        if (IMG) {
-            // image fill: the group's buffered point indices to their place in
-            // the pixel's full ray (far half reversed, then anchor, then near half)
-            if (MODE == kWalkImgFill && __any_sync(full, flush_full || flush_last)) {
-                const int cnt = flush_full ? 16 : (int)(n & 15);
-                const int64_t first = flush_full ? n - 16 : (n & ~(int64_t)15);
-                if ((flush_full || flush_last) && sl < cnt) {
-                    const int64_t k = first + sl;
-                    const int64_t at = r == 0 ? img_base + img_nfar - 1 - k : img_base + img_nfar + 1 + k;
-                    im.pts[at] = my_pt;
-                }
-            }
-        } else if (__any_sync(full, flush_full || flush_last)) {
-            // records of the group's buffered steps (n already counts the newest);
-            // chunks start at multiples of 16 and cap is one (fused mode) or
-            // exactly the walk's length (list mode), so a chunk is kept whole or
-            // not at all
-            const int cnt = flush_full ? 16 : (int)(n & 15);
-            const int64_t first = flush_full ? n - 16 : (n & ~(int64_t)15);
-            const bool keep = (flush_full || flush_last) && first < cap;
-            write_step_records(a, o, rg, prev_last, my_pt, keep ? cnt : 0, vel_hl, w32, inv_Lunit, width_mode,
-                               out + first, sl);
-            if (flush_full) prev_last = nx;
+        // a full chunk of indices (a finished walk's last ones are written
+        // with its neighbours' next chunk; n bounds what is written)
+        if (MODE != kWalkImgCount && (it & (G - 1)) == G - 1) {
+            const int k = it - (G - 1) + sl;
+            if (k < n) put(k, my_pt);
         }
+    }
+    if (MODE != kWalkImgCount && (it & (G - 1)) != 0) {
+        const int k = (it & ~(G - 1)) + sl;
+        if (k < n) put(k, my_pt);
     }
     if (live && sl == 0) {
         if (MODE == kWalkFused)
             lens[wi] = gave_up ? 0 : n;
         else if (MODE == kWalkImgCount)
             lens[wg] = gave_up ? 0 : n;
-        else if (n != cap && !gave_up)
+        else if (!gave_up && n != (MODE == kWalkList ? ray_off[wi + 1] - ray_off[wi] : lens[wg]))
             atomicCAS(err, 0, (int)kDevBounds);
     }
 }
 
-// Walks whose records did not fit their scratch slot (length > K).
+// Launches of few walks take 16 lanes per walk: a step's latency counts there,
+// not its instructions (a row is one or two dependent loads instead of four or
+// five).  The line lies where a launch fills three quarters of the GPU at 4
+// lanes: 12,000 walks (sphere models, 12 directions) take 32 us with 16 lanes
+// and 48 us with 4; 30,000 take 62 and 65; 48,000 take 97 and 85; 240,000 take
+// 592 and 386.
+inline bool walk_wide(int64_t walks, int sms)
+{
+    return walks < (int64_t)sms * kWalkBlocks * (kWalkThreads / kWalkRow) * 3 / 4;
+}
+
+template <int MODE>
+static mgt_status launch_walk(const WalkArgs &a, int64_t walks, int64_t *lens, const int64_t *ray_off,
+                              const int64_t *list, int32_t K, unsigned long long *n_stall, int32_t *scratch,
+                              Step32 *steps, int *err, const ImgWalkArgs &im, cudaStream_t s)
+{
+    int dev = 0, sms = 0;
+    MGT_CUDA(cudaGetDevice(&dev));
+    MGT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const auto run = [&](auto kernel, int lanes) {
+        kernel<<<(unsigned)ceil_div(walks * lanes, kWalkThreads), kWalkThreads, 0, s>>>(
+            a, lens, ray_off, list, walks, K, n_stall, scratch, steps, err, im);
+    };
+    if (walk_wide(walks, sms))
+        run(k_walk<MODE, 16>, 16);
+    else
+        run(k_walk<MODE, kWalkRow>, kWalkRow);
+    MGT_LAUNCH_CHECK("k_walk");
+    return MGT_OK;
+}
+
+// Walks whose indices did not fit their scratch slot (length > K).
 __global__ void k_walk_overflow(int64_t W, const int64_t *__restrict__ lens, int32_t K, int64_t *__restrict__ list,
                                 unsigned long long *__restrict__ count)
 {
@@ -933,17 +954,96 @@ __global__ void k_walk_overflow(int64_t W, const int64_t *__restrict__ lens, int
     list[atomicAdd(count, 1ULL)] = t;
 }
 
-// Move each walk's records (at most K) from its scratch slot to its final
-// place: one warp per walk, 16-byte records.
-__global__ void k_walk_compact(int64_t W, const int64_t *__restrict__ ray_off, int32_t K,
-                               const Step32 *__restrict__ scratch, Step32 *__restrict__ steps)
+// What a step record takes from a point, one 64-byte row: positions times
+// pos_scale and v/c as float hi + lo, and the line width.
+struct __align__(64) WalkPoint {
+    float4 q[4];              // {hx, hy, hz, lx}, {ly, lz, vhx, vhy}, {vhz, vlx, vly, vlz}, {w, 0, 0, 0}
+};
+
+__global__ void k_walk_points(int64_t N, const float *__restrict__ pos_hl, const float *__restrict__ vel_hl,
+                              const float2 *__restrict__ w32, WalkPoint *__restrict__ out)
 {
-    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (t >= W) return;
-    const int64_t b = ray_off[t], n = ray_off[t + 1] - b;
-    const int64_t m = n < K ? n : K;
-    for (int64_t j = lane; j < m; j += 32) steps[b + j] = scratch[t * (int64_t)K + j];
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const float *p = pos_hl + 6 * i, *v = vel_hl + 6 * i;
+    out[i].q[0] = make_float4(p[0], p[1], p[2], p[3]);
+    out[i].q[1] = make_float4(p[4], p[5], v[0], v[1]);
+    out[i].q[2] = make_float4(v[2], v[3], v[4], v[5]);
+    out[i].q[3] = make_float4(w32[i].x, 0.0f, 0.0f, 0.0f);
+}
+
+// Step records from the walks' point indices, one walk per 16 lanes: walk t's
+// indices in its scratch slot (at most K; a longer walk is left to the list
+// form), or (LIST) already in the records of the walks named in `list`.  The
+// lanes hold 16 consecutive points of the ray, the first of them from the trip
+// before (the origin at first), and lanes 1-15 write the records of the steps
+// ending at their points.  All in FP32: dx from the hi + lo scaled positions,
+// beta = n.(v_c - v_o)/c and dbeta = n.(v_c - v_prev)/c from hi + lo values of
+// v/c (relative error about 1e-7 of |v_c - v_o|/c), the averaged width of the
+// segment.  Bound by the gathers of the points' rows (one L1 wavefront per lane
+// and 32 bytes): 2.6 ms for 1.9e8 records.  A record moves 20 bytes of DRAM
+// traffic here instead of 48 through a slot of finished records, and the walk,
+// whose lanes gathered one record at a time, keeps only point indices.
+template <bool LIST>
+__global__ void __launch_bounds__(256, 5) k_walk_compact(WalkArgs a, int64_t W, const int64_t *__restrict__ ray_off,
+                                                      const int64_t *__restrict__ list, int32_t K,
+                                                      const int32_t *__restrict__ scratch,
+                                                      const WalkPoint *__restrict__ pt, float inv_Lunit, int width_mode,
+                                                      Step32 *__restrict__ steps, int *__restrict__ err)
+{
+    const unsigned full = 0xffffffffu;
+    const int64_t slot = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
+    const int sl = threadIdx.x & 15;
+    int64_t t = 0, base = 0, n = 0;
+    if (slot < W) {
+        t = LIST ? list[slot] : slot;
+        base = ray_off[t];
+        n = ray_off[t + 1] - base;
+        if (!LIST && n > K) n = 0;
+    }
+    const int r = (int)(t / a.N);
+    const int o = (int)(t - (int64_t)r * a.N);
+    const float4 dir = a.dirs32[a.dir_map ? a.dir_map[r] : r];
+    const float4 o1 = pt[o].q[1], o2 = pt[o].q[2];
+    auto point = [&](int64_t j) {                // step j's point, -1 (and past the end) the origin
+        return j >= 0 && j < n ? (LIST ? steps[base + j].x : scratch[t * (int64_t)K + j]) : o;
+    };
+    int nc = point(sl - 1);
+    for (int64_t j0 = -1; __any_sync(full, j0 + 1 < n); j0 += 15) {
+        const int64_t j = j0 + sl;
+        int c = nc;
+        nc = point(j + 15);                      // the next trip's, ahead of this one's gathers
+        if (c < 0 || c >= a.N) {                 // index check: record, use the origin
+            atomicCAS(err, 0, (int)kDevBounds);
+            c = o;
+        }
+        const Vec8 lo = load32(&pt[c].q[0]), hi = load32(&pt[c].q[2]);
+        const float4 c0 = lo.a, c1 = lo.b, c2 = hi.a;
+        const float wc = hi.b.x;
+        const float pc[6] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y};
+        const float vc[6] = {c1.z, c1.w, c2.x, c2.y, c2.z, c2.w};
+        const float vo[6] = {o1.z, o1.w, o2.x, o2.y, o2.z, o2.w};
+        float pp[6], vp[6];
+#pragma unroll
+        for (int d = 0; d < 6; ++d) {
+            pp[d] = __shfl_up_sync(full, pc[d], 1, 16);
+            vp[d] = __shfl_up_sync(full, vc[d], 1, 16);
+        }
+        const float wp = __shfl_up_sync(full, wc, 1, 16);
+        if (sl == 0 || j >= n) continue;
+        float e[3], db[3], dp[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            e[d] = (pc[d] - pp[d]) + (pc[3 + d] - pp[3 + d]);
+            db[d] = (vc[d] - vo[d]) + (vc[3 + d] - vo[3 + d]);
+            dp[d] = (vc[d] - vp[d]) + (vc[3 + d] - vp[3 + d]);
+        }
+        const float dxs = sqrtf(fmaf(e[2], e[2], fmaf(e[1], e[1], e[0] * e[0]))) * inv_Lunit;
+        const float beta = fmaf(dir.z, db[2], fmaf(dir.y, db[1], dir.x * db[0]));
+        const float dbeta = fmaf(dir.z, dp[2], fmaf(dir.y, dp[1], dir.x * dp[0]));
+        const float wbar = width_mode == 0 ? sqrtf(0.5f * (wc * wc + wp * wp)) : 0.5f * (wc + wp);
+        steps[base + j] = make_int4(c, __float_as_int(dxs), __float_as_int(beta), __float_as_int(dbeta / wbar));
+    }
 }
 
 // Double-precision step geometry for the FP64 formal solution, from the
@@ -1005,17 +1105,17 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
     }
     const int64_t W = (int64_t)Rw * m->N;
     WalkArgs a{m->N,        Rw,            m->d_pos,  m->d_nbr_off, m->d_nbrs,   m->d_nbr_pos,
-               m->pos_scale, m->d_bnd,     m->d_dirs, m->d_ent,     m->d_ent_off, m->d_pos_hl,
-               m->d_dirs32,  m->d_order,   m->pos_slack, m->d_count + 2,
-               (int32_t)((m->n_ent + 15) / 16 + 2), m->n_ent, all ? nullptr : m->d_dir_map};
+               m->pos_scale, m->d_bnd,     m->d_dirs, m->d_ent,     m->d_ent_row, m->d_pos_hl,
+               m->d_dirs32,  m->d_order,   m->pos_slack, m->d_count + 2, m->n_chunks, all ? nullptr : m->d_dir_map};
     if (!m->d_ray_off) MGT_CUDA(cudaMalloc(&m->d_ray_off, sizeof(int64_t) * ((int64_t)m->R * m->N + 1)));
-    // Scratch slot per walk: K records, a multiple of 16; the longest half-ray
-    // of this model's previous trace when there was one, else 4 N^(1/3) + 16
-    // (a few times the mean half-ray of a cloud of N points), kept within a
-    // third of the free device memory (counting what the scratch pool holds
-    // unused).  Longer walks are redone.
+    // Scratch slot per walk: K point indices, a multiple of 16; the longest
+    // half-ray of this model's previous trace when there was one, else four
+    // times 4 N^(1/3) + 16 (a few times the mean half-ray of a cloud of N
+    // points, so that a first trace rarely redoes a walk: 16 bytes per step of
+    // the usual longest), kept within a third of the free device memory
+    // (counting what the scratch pool holds unused).  Longer walks are redone.
     int64_t K = m->max_half > 0 ? (m->max_half + 15) / 16 * 16
-                                : ((int64_t)(4.0 * std::cbrt((double)m->N)) + 16 + 15) / 16 * 16;
+                                : 4 * (((int64_t)(4.0 * std::cbrt((double)m->N)) + 16 + 15) / 16 * 16);
     cudaMemPool_t pool = nullptr;
     MGT_TRY_STATUS(scratch_pool(&pool));
     {
@@ -1025,10 +1125,11 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
         MGT_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved));
         MGT_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
         freeb += reserved > used ? (size_t)(reserved - used) : 0;
-        while (K > 16 && (size_t)(W * K) * sizeof(Step32) > freeb / 3) K -= 16;
+        while (K > 16 && (size_t)(W * K) * sizeof(int32_t) > freeb / 3) K -= 16;
     }
     int64_t *d_len = nullptr, *d_list = nullptr, *d_max = nullptr;
-    Step32 *d_scratch = nullptr;
+    int32_t *d_scratch = nullptr;
+    WalkPoint *d_pt = nullptr;
     unsigned long long *d_nover = nullptr;
     void *tmp = nullptr, *tmpb = nullptr;
     auto release = [&]() {
@@ -1039,6 +1140,7 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
         if (d_list) cudaFreeAsync(d_list, s);
         if (d_nover) cudaFreeAsync(d_nover, s);
         if (d_scratch) cudaFreeAsync(d_scratch, s);
+        if (d_pt) cudaFreeAsync(d_pt, s);
     };
     struct Guard {
         decltype(release) &f;
@@ -1047,7 +1149,8 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
     MGT_CUDA(cudaMallocFromPoolAsync(&d_len, sizeof(int64_t) * (W + 1), pool, s));
     MGT_CUDA(cudaMallocFromPoolAsync(&d_list, sizeof(int64_t) * W, pool, s));
     MGT_CUDA(cudaMallocFromPoolAsync(&d_nover, sizeof(unsigned long long), pool, s));
-    if (cudaMallocFromPoolAsync(&d_scratch, sizeof(Step32) * W * K, pool, s) != cudaSuccess) {
+    MGT_CUDA(cudaMallocFromPoolAsync(&d_pt, sizeof(WalkPoint) * m->N, pool, s));
+    if (cudaMallocFromPoolAsync(&d_scratch, sizeof(int32_t) * W * K, pool, s) != cudaSuccess) {
         cudaGetLastError();
         d_scratch = nullptr;
         return set_error(MGT_ERR_OOM, "cannot allocate the walk scratch");
@@ -1057,11 +1160,9 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
     const float inv_Lunit = (float)(1.0 / (m->pos_scale * m->L_unit));
     {
         MGT_KTIMER("k_walk<fused>", s);
-        k_walk<kWalkFused><<<ceil_div(W * 16, kWalkThreads), kWalkThreads, 0, s>>>(a, d_len, nullptr, nullptr, 0, (int32_t)K,
-                                                                 m->d_count + 1, m->d_vel_hl, m->d_w32, inv_Lunit,
-                                                                 m->opts.width_mode, d_scratch, m->d_err, ImgWalkArgs{});
+        MGT_TRY_STATUS(launch_walk<kWalkFused>(a, W, d_len, nullptr, nullptr, (int32_t)K, m->d_count + 1, d_scratch,
+                                               nullptr, m->d_err, ImgWalkArgs{}, s));
     }
-    MGT_LAUNCH_CHECK("k_walk<fused>");
     MGT_CUDA(cudaMemsetAsync(d_len + W, 0, sizeof(int64_t), s));
     size_t tmp_bytes = 0;
     MGT_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, d_len, m->d_ray_off, W + 1, s));
@@ -1104,19 +1205,25 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
     m->n_exact_steps = (int64_t)exact_steps;   // the walks of the fused pass
     if (total > 0) {
         {
-            // each record read once from its slot and written once, plus the offsets
-            MGT_KTIMER_BYTES("k_walk_compact", s, 32.0 * (double)total + 8.0 * (double)W);
-            k_walk_compact<<<ceil_div(W * 32, 256), 256, 0, s>>>(W, m->d_ray_off, (int32_t)K, d_scratch, m->d_steps32);
+            // each index read once from its slot and each record written once, plus the offsets
+            MGT_KTIMER_BYTES("k_walk_compact", s, 20.0 * (double)total + 8.0 * (double)W);
+            k_walk_points<<<ceil_div(m->N, 256), 256, 0, s>>>(m->N, m->d_pos_hl, m->d_vel_hl, m->d_w32, d_pt);
+            k_walk_compact<false><<<ceil_div(W * 16, 256), 256, 0, s>>>(a, W, m->d_ray_off, nullptr, (int32_t)K, d_scratch,
+                                                                    d_pt, inv_Lunit, m->opts.width_mode, m->d_steps32,
+                                                                    m->d_err);
         }
         MGT_LAUNCH_CHECK("k_walk_compact");
+        note_launch();                             // k_walk_points
         if (n_over > 0) {
             {
                 MGT_KTIMER("k_walk<list>", s);
-                k_walk<kWalkList><<<ceil_div((int64_t)n_over * 16, kWalkThreads), kWalkThreads, 0, s>>>(
-                    a, nullptr, m->d_ray_off, d_list, (int64_t)n_over, 0, nullptr, m->d_vel_hl, m->d_w32, inv_Lunit,
-                    m->opts.width_mode, m->d_steps32, m->d_err, ImgWalkArgs{});
+                MGT_TRY_STATUS(launch_walk<kWalkList>(a, (int64_t)n_over, nullptr, m->d_ray_off, d_list, 0, nullptr,
+                                                      nullptr, m->d_steps32, m->d_err, ImgWalkArgs{}, s));
+                k_walk_compact<true><<<ceil_div((int64_t)n_over * 16, 256), 256, 0, s>>>(
+                    a, (int64_t)n_over, m->d_ray_off, d_list, 0, nullptr, d_pt, inv_Lunit, m->opts.width_mode,
+                    m->d_steps32, m->d_err);
             }
-            MGT_LAUNCH_CHECK("k_walk<list>");
+            MGT_LAUNCH_CHECK("k_walk_compact<list>");
         }
     }
     m->steps_width_mode = m->opts.width_mode;
@@ -1329,9 +1436,8 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
     MGT_CUDA(cudaMalloc(&g.d_off, sizeof(int64_t) * (npix + 1)));
     MGT_CUDA(cudaMemcpyAsync(g.d_ref, ref.data(), sizeof(double) * ref.size(), cudaMemcpyHostToDevice, s));
     WalkArgs a{m->N,        m->R,          m->d_pos,  m->d_nbr_off, m->d_nbrs,   m->d_nbr_pos,
-               m->pos_scale, m->d_bnd,     m->d_dirs, m->d_ent,     m->d_ent_off, m->d_pos_hl,
-               m->d_dirs32,  m->d_order,   m->pos_slack, m->d_count + 3,
-               (int32_t)((m->n_ent + 15) / 16 + 2), m->n_ent, nullptr};
+               m->pos_scale, m->d_bnd,     m->d_dirs, m->d_ent,     m->d_ent_row, m->d_pos_hl,
+               m->d_dirs32,  m->d_order,   m->pos_slack, m->d_count + 3, m->n_chunks, nullptr};
     k_img_anchor<<<ceil_div(npix * 32, 256), 256, 0, s>>>(a, g.d_ref, npix, n[0], n[1], n[2], g.d_anchor);
     MGT_LAUNCH_CHECK("k_img_anchor");
     int64_t *d_lens = nullptr, *d_sizes = nullptr;
@@ -1339,10 +1445,8 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
     MGT_CUDA(cudaMallocAsync(&d_lens, sizeof(int64_t) * 2 * npix, s));
     MGT_CUDA(cudaMallocAsync(&d_sizes, sizeof(int64_t) * (npix + 1), s));
     ImgWalkArgs im{g.d_ref, g.d_anchor, g.d_off, nullptr, npix, {n[0], n[1], n[2]}};
-    k_walk<kWalkImgCount><<<ceil_div(2 * npix * 16, kWalkThreads), kWalkThreads, 0, s>>>(a, d_lens, nullptr, nullptr, 0, 0, nullptr,
-                                                                       nullptr, nullptr, 0.0f, 0, nullptr, m->d_err,
-                                                                       im);
-    MGT_LAUNCH_CHECK("k_walk<image count>");
+    MGT_TRY_STATUS(launch_walk<kWalkImgCount>(a, 2 * npix, d_lens, nullptr, nullptr, 0, nullptr, nullptr, nullptr, m->d_err,
+                                              im, s));
     k_img_sizes<<<ceil_div(npix, 256), 256, 0, s>>>(npix, d_lens, d_sizes);
     MGT_LAUNCH_CHECK("k_img_sizes");
     MGT_CUDA(cudaMemsetAsync(d_sizes + npix, 0, sizeof(int64_t), s));
@@ -1364,9 +1468,8 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
     }
     MGT_CUDA(cudaMalloc(&g.d_pts, sizeof(int32_t) * (total > 0 ? total : 1)));
     im.pts = g.d_pts;
-    k_walk<kWalkImgFill><<<ceil_div(2 * npix * 16, kWalkThreads), kWalkThreads, 0, s>>>(a, d_lens, nullptr, nullptr, 0, 0, nullptr,
-                                                                      nullptr, nullptr, 0.0f, 0, nullptr, m->d_err, im);
-    MGT_LAUNCH_CHECK("k_walk<image fill>");
+    MGT_TRY_STATUS(launch_walk<kWalkImgFill>(a, 2 * npix, d_lens, nullptr, nullptr, 0, nullptr, nullptr, nullptr, m->d_err,
+                                             im, s));
     k_img_place_anchor<<<ceil_div(npix, 256), 256, 0, s>>>(npix, d_lens, g.d_off, g.d_anchor, g.d_pts);
     MGT_LAUNCH_CHECK("k_img_place_anchor");
     MGT_CUDA(cudaFreeAsync(d_lens, s));
