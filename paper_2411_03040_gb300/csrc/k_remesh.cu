@@ -41,21 +41,9 @@ struct __align__(32) RmPoint {
     double x, y, z, rho;
 };
 
-// Doubles as unsigned integers of the same order (no NaN, zeros canonical).
-__device__ __forceinline__ uint64_t ord(double v)
-{
-    const long long b = __double_as_longlong(v);
-    return (uint64_t)(b ^ ((b >> 63) | (long long)0x8000000000000000ull));
-}
-
-__device__ __forceinline__ double unord(uint64_t u)
-{
-    return __longlong_as_double((long long)(u & 0x8000000000000000ull ? u ^ 0x8000000000000000ull : ~u));
-}
-
 __device__ __forceinline__ double no_negative_zero(double v) { return v == 0.0 ? 0.0 : v; }
 
-__device__ __forceinline__ uint64_t ord_mid(double v) { return ord(no_negative_zero(v)); }
+__device__ __forceinline__ uint64_t ord_mid(double v) { return order_key(no_negative_zero(v)); }
 
 // A box's bounds and tracer range as ordered integers: lo[3], hi[3], rmin, rmax.
 struct RmBox {
@@ -113,7 +101,7 @@ __device__ __forceinline__ RmPoint load_point(const RmPoint *p)
 
 __device__ __forceinline__ int octant(const RmPoint &p, const uint64_t *mid)
 {
-    return (ord(p.x) >= mid[0] ? 1 : 0) | (ord(p.y) >= mid[1] ? 2 : 0) | (ord(p.z) >= mid[2] ? 4 : 0);
+    return (order_key(p.x) >= mid[0] ? 1 : 0) | (order_key(p.y) >= mid[1] ? 2 : 0) | (order_key(p.z) >= mid[2] ? 4 : 0);
 }
 
 // Lanes of the warp whose active point lies in octant `oct`.
@@ -142,7 +130,7 @@ __global__ void __launch_bounds__(kRmThreads) k_rm_stats(RmUnits u, const RmPoin
     empty_box(s);
     for (int i = lane; i < n; i += 32) {
         const RmPoint p = load_point(pts + p0 + i);
-        const uint64_t c[4] = {ord(p.x), ord(p.y), ord(p.z), ord(p.rho)};
+        const uint64_t c[4] = {order_key(p.x), order_key(p.y), order_key(p.z), order_key(p.rho)};
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
             uint64_t &lo = s.v[d < 3 ? d : 6], &hi = s.v[d < 3 ? 3 + d : 7];
@@ -177,11 +165,11 @@ __global__ void k_rm_decide(int64_t nb, const RmBox *__restrict__ box, double r_
     const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (b >= nb) return;
     const RmBox s = box[b];
-    const double rmin = unord(s.v[6]), rmax = unord(s.v[7]);
+    const double rmin = order_value(s.v[6]), rmax = order_value(s.v[7]);
     const double var = 2.0 * ((rmax - rmin) / (rmax + rmin));
     divide[b] = may_divide && var > r_max ? 1 : 0;
     for (int d = 0; d < 3; ++d) {
-        const double lo = unord(s.v[d]), hi = unord(s.v[3 + d]);
+        const double lo = order_value(s.v[d]), hi = order_value(s.v[3 + d]);
         mids[3 * b + d] = (lo + hi) * 0.5;
         if (root) {
             root[d] = lo;

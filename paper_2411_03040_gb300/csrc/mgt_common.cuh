@@ -66,6 +66,9 @@ struct ImageGeom {
     int32_t *d_anchor = nullptr;        // [npix]
     int64_t *d_off = nullptr;           // [npix+1]
     int32_t *d_pts = nullptr;           // [total] far end first
+    int64_t npix_cap = 0, pts_cap = 0;  // what the buffers hold (from the library's pool)
+    cudaStream_t stream = nullptr;      // the stream they were filled on
+    bool shared = false;                // read on another stream too
 };
 
 // What a started Ng step still has to do (see ng_step).
@@ -214,8 +217,6 @@ mgt_status build_steps64(mgt_model *m, cudaStream_t s);
 
 mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy, cudaStream_t s);
 void image_free(mgt_model *m);
-void image_frame(const double *pos, int64_t N, const double n[3], int32_t npx, int32_t npy, double e1[3],
-                 double e2[3], std::vector<double> &ref);
 
 // rays of every pair held and current for the model's options (api.cu)
 mgt_status ensure_rays(mgt_model *m, mgt_precision p, cudaStream_t s);
@@ -270,6 +271,19 @@ mgt_status ng_begin(mgt_model *m, const mgt_ng_opts *o, cudaStream_t s);
 mgt_status ng_after_push(mgt_model *m, cudaStream_t s);
 mgt_status ng_after_predict(mgt_model *m, cudaStream_t s);
 void ng_free(mgt_model *m);
+
+// Doubles as unsigned integers of the same order (no NaN), so that minima and
+// maxima run on the integer pipes and in integer atomics.
+__device__ __forceinline__ uint64_t order_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return (uint64_t)(b ^ ((b >> 63) | (long long)0x8000000000000000ull));
+}
+
+__device__ __forceinline__ double order_value(uint64_t u)
+{
+    return __longlong_as_double((long long)(u & 0x8000000000000000ull ? u ^ 0x8000000000000000ull : ~u));
+}
 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 

@@ -202,3 +202,58 @@ def test_adjoint_matches_gpu_finite_differences_and_autograd(mgt):
     assert np.allclose(lt.grad.cpu().numpy(), gT, rtol=1e-9, atol=0)
     assert np.allclose(ln.grad.cpu().numpy(), gn, rtol=1e-9, atol=0)
     assert np.allclose(vv.grad.cpu().numpy(), gv, rtol=1e-9, atol=0)
+
+
+@pytest.mark.parametrize("n,npx,npy,shape", [(1, 3, 2, "ball"), (7, 5, 5, "ball"), (400, 33, 7, "ball"),
+                                             (400, 9, 9, "line"), (400, 9, 9, "plane"), (5000, 40, 40, "clumps"),
+                                             (5000, 12, 12, "far")])
+def test_pixel_rays_of_awkward_clouds(mgt, n, npx, npy, shape):
+    # anchors found through the search grid: one cell only, every projection on
+    # one place or on a line, empty corners, thousands of points in one cell
+    # and coincident points (ties), a cloud far from the origin (bounds wider
+    # than a cell).  Rays are decided by FP64 predicates: equality
+    rng = np.random.default_rng(n + npx)
+    pos = rng.normal(size=(n, 3))
+    d = np.array([0.0, 0.0, 1.0])
+    if shape == "line":
+        pos[:, :2] = 0.25
+    elif shape == "plane":
+        pos[:, 0] = 0.0
+    elif shape == "clumps":
+        pos[: n // 2] = np.round(pos[: n // 2] * 1e-3, 4)
+        pos[::50] *= 30.0
+        d = DIR
+    elif shape == "far":
+        pos = pos * 1e-4 + np.array([1.0, -2.0, 0.5])
+        d = DIR
+    nb = [rng.choice(n, size=min(n, 8), replace=False) for _ in range(n)]
+    off = np.concatenate([[0], np.cumsum([len(v) for v in nb])]).astype(np.int64)
+    m = synth.Model("cloud", pos * 1e11, np.zeros((n, 3)), np.full(n, 50.0), np.full(n, 1e4), np.full(n, 1e10),
+                    np.full(n, 1e5), off, np.concatenate([np.sort(v) for v in nb]).astype(np.int32),
+                    np.arange(0, n, 10, dtype=np.int32), synth.healpix_directions(1), 3, synth.linear_rotor(3, rng))
+    h = mgt.mgt_model_create(m)
+    for direction in (d, -d):                  # the second view reuses the first one's buffers
+        anchor, roff, pts = mgt.mgt_image_rays(h, direction, npx, npy)
+        r = O.image_rays(m, direction, npx, npy)
+        assert np.array_equal(anchor, r.anchor)
+        assert np.array_equal(roff, r.off) and np.array_equal(pts, r.pts)
+
+
+def test_pixel_rays_longer_than_their_slots(mgt):
+    # a chain along the line of sight: half-rays of up to 1,500 points, beyond
+    # the scratch slot (8 n^(1/3) + 16), are walked again into their place
+    n = 1500
+    x = np.linspace(-1, 1, n)
+    pos = np.stack([0.05 * x ** 2, 0.01 * np.sin(3 * x), x], axis=1)
+    nb = [[j for j in (i - 1, i + 1) if 0 <= j < n] for i in range(n)]
+    off = np.concatenate([[0], np.cumsum([len(v) for v in nb])]).astype(np.int64)
+    rng = np.random.default_rng(3)
+    m = synth.Model("chain", pos * 1e11, np.zeros((n, 3)), np.full(n, 50.0), np.full(n, 1e4), np.full(n, 1e10),
+                    np.full(n, 1e5), off, np.concatenate(nb).astype(np.int32), np.array([0, n - 1], np.int32),
+                    synth.healpix_directions(1), 3, synth.linear_rotor(3, rng))
+    d = np.array([0.0, 0.0, 1.0])
+    h = mgt.mgt_model_create(m)
+    anchor, roff, pts = mgt.mgt_image_rays(h, d, 4, 3)
+    r = O.image_rays(m, d, 4, 3)
+    assert np.max(np.diff(roff)) > 1000
+    assert np.array_equal(anchor, r.anchor) and np.array_equal(roff, r.off) and np.array_equal(pts, r.pts)
