@@ -336,7 +336,7 @@ static void free_model(mgt_model *m)
 {
     void *ptrs[] = {m->d_dir_map, m->d_batch_pairs, m->d_nbr_pos, m->d_ent, m->d_ent_row, m->d_pos_hl, m->d_vel_hl, m->d_dirs32, m->d_order, m->d_pos, m->d_vel, m->d_temp, m->d_vturb2, m->d_ncoll, m->d_nspec, m->d_w64, m->d_w32, m->d_dxmax,
                     m->d_nbr_off, m->d_nbrs, m->d_bnd, m->d_dirs, m->d_pairs, m->d_xq, m->d_wq, m->d_line_tab,
-                    m->d_line_ul, m->d_level_tab, m->d_coll_tab, m->d_coll_ul, m->d_entry, m->d_pops,
+                    m->d_line_ul, m->d_level_tab, m->d_coll_tab, m->d_coll_ul, m->d_pops,
                     m->d_pops_prev, m->d_line32, m->d_line64, m->d_J, m->d_Lst, m->d_err, m->d_range_bad, m->d_count,
                     m->d_ray_off, m->d_steps64};
     for (void *p : ptrs)
@@ -433,15 +433,8 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
         lev[i] = m->energy[i];
         lev[L + i] = m->g[i];
     }
-    std::vector<int16_t> entry(3 * (size_t)L * L, (int16_t)-1);
-    for (int k = 0; k < m->M; ++k) {
-        entry[m->up[k] * L + m->lo[k]] = (int16_t)k;              // down
-        entry[(size_t)L * L + m->lo[k] * L + m->up[k]] = (int16_t)k; // up
-    }
     std::vector<int32_t> cul(2 * (size_t)std::max(K, 1), 0);
     for (int k = 0; k < K; ++k) {
-        entry[2 * (size_t)L * L + m->cup[k] * L + m->clo[k]] = (int16_t)k;
-        entry[2 * (size_t)L * L + m->clo[k] * L + m->cup[k]] = (int16_t)k;
         cul[k] = m->cup[k];
         cul[K + k] = m->clo[k];
     }
@@ -478,7 +471,6 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
     MGT_TRY(dalloc(&m->d_level_tab, lev.size()));
     MGT_TRY(dalloc(&m->d_coll_tab, std::max(K, 1)));
     MGT_TRY(dalloc(&m->d_coll_ul, cul.size()));
-    MGT_TRY(dalloc(&m->d_entry, entry.size()));
     MGT_TRY(dalloc(&m->d_pops, N * L));
     MGT_TRY(dalloc(&m->d_pops_prev, N * L));
     MGT_TRY(dalloc(&m->d_line32, N * row_stride32(Mp)));
@@ -549,7 +541,6 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
     MGT_TRY(upload(m->d_level_tab, lev.data(), lev.size(), s));
     if (K > 0) MGT_TRY(upload(m->d_coll_tab, m->Kul.data(), K, s));
     MGT_TRY(upload(m->d_coll_ul, cul.data(), cul.size(), s));
-    MGT_TRY(upload(m->d_entry, entry.data(), entry.size(), s));
     MGT_CUDA(cudaMemsetAsync(m->d_err, 0, sizeof(int) * 4, s));
     MGT_CUDA(cudaMemsetAsync(m->d_count, 0, sizeof(unsigned long long) * 4, s));
     MGT_TRY(launch_widths(m, s));
@@ -610,8 +601,7 @@ static mgt_status formal_solve_device(mgt_model *m, mgt_precision p, cudaStream_
 static mgt_status stat_eq_device(mgt_model *m, cudaStream_t s)
 {
     if (!m->have_J) return set_error(MGT_ERR_STATE, "mgt_formal_solve must be called first");
-    MGT_CUDA(cudaMemcpyAsync(m->d_pops_prev, m->d_pops, sizeof(double) * m->N * m->L, cudaMemcpyDeviceToDevice, s));
-    MGT_TRY(launch_stat_eq(m, s));
+    MGT_TRY(launch_stat_eq(m, s));       // keeps the previous populations in d_pops_prev
     m->line_dirty = true;
     return MGT_OK;
 }

@@ -1,4 +1,4 @@
-// Statistical equilibrium: one warp per point, FP64, state reduction.
+// Statistical equilibrium: FP64, state reduction, G lanes per point.
 //
 // Rates i -> j per point (s^-1):
 //   radiative, preconditioned by the diagonal approximate Lambda operator
@@ -12,8 +12,18 @@
 // R_ij += R_in R_nj / S_n with S_n = sum_{j<n} R_nj; then n_0 = 1,
 // n_k = sum_{i<k} n_i R_ik / S_k and normalise.  Only non-negative numbers are
 // added, so populations many decades below the ground level keep full
-// relative accuracy.  All warp reductions run in a fixed lane order, so the
-// result is bitwise reproducible.
+// relative accuracy.  All reductions run in a fixed lane order, so the result
+// is bitwise reproducible.
+//
+// What bounds it: the FP64 pipe, 16 cycles per warp instruction and SM whatever
+// the number of active lanes (two lanes per cycle).  The elimination of 41
+// levels is 22,140 multiply-adds, 692 full warp instructions; with one warp per
+// point another 1,440 went into work that fills few lanes: the sum and the
+// reciprocal of every pivot, rates assembled from all L^2 entries, the back
+// substitution.  So a warp takes 32 / G points and every such instruction
+// serves all of them, and the rates are filled in from the lists of lines and
+// collisions.  100k points: 41 levels 11.8 -> 7.5 ms, 21 levels 3.34 -> 1.47,
+// 11 levels 1.49 -> 0.44, 5 levels 0.76 -> 0.17.
 #include <algorithm>
 #include <cstring>
 
@@ -34,49 +44,78 @@ struct SEArgs {
     const double *level_tab;  // [2][L]: E, g
     const double *Kul;        // [K]
     const int32_t *coll_ul;   // [2][K]
-    const int16_t *entry;     // [3][L*L]
-    double *pops_out;         // [N][L] (may be pops_old: each warp reads its row before writing it)
-    double *pops_prev;        // [N][L] copy of pops_old, or NULL
-    int wpb;                  // warps (points) per block
+    double *pops_out;         // [N][L] (may be pops_old: each point's row is read before it is written)
+    double *pops_prev;        // [N][L] copy of pops_old
+    int wpb;                  // warps of a CTA that take points (what its shared memory holds)
 };
 
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Sum over the warp when only lanes below n hold nonzero values: the xor
-// butterfly stops at the smallest power of two >= n, and every lane below n
-// ends with the total (fewer FP64 additions on GB300's narrow FP64 pipe).
-__device__ __forceinline__ double warp_sum_first(double v, int n)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        if (o < n) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 constexpr int kMaxWarpsPerBlock = 4;
+constexpr size_t kSEMaxSmem = 227 * 1024;
 
-// Point p, solved by one warp in its shared-memory slice sm (LL + 3L + 2 Mpad doubles).
-__device__ __forceinline__ void se_point(const SEArgs &a, int64_t p, double *sm, int lane)
+// A point's working memory in doubles: the rates, the reciprocals 1/bz (later
+// the unnormalised populations), and the lines' rates (later the pivots'
+// reciprocals).
+__host__ __device__ inline int se_point_doubles(int L, int M) { return L * L + L + (L > 2 * M ? L : 2 * M); }
+
+// Lanes per point: enough points per warp to fill the FP64 instructions, enough
+// warps to hide their latency.  41 levels: 16 lanes 8.1 ms per 100k points, 8
+// lanes (16 points of 14.4 KB fill an SM's shared memory, so one warp per
+// scheduler) 10.4; 21 levels: 8 lanes 1.6, 4 lanes 2.1, 16 lanes 2.3; 11 levels:
+// 4 lanes 0.48, 8 lanes 0.72.
+__host__ __device__ inline int se_lanes(int L) { return L > 32 ? 16 : L > 16 ? 8 : 4; }
+
+// Sum of v[0 .. n-1] (n <= 64) over the point's lanes, in the order of a warp
+// that holds v[l] + v[l + 32] in lane l and adds lanes 16, 8, 4, 2 and 1 apart,
+// whatever G is: accelerated iterations amplify a changed rounding.  Additions
+// of what lies past n are skipped.  Every lane ends with the sum.
+template <int G> __device__ __forceinline__ double point_sum(const double *v, int n, int t)
+{
+    double s[32 / G];
+#pragma unroll
+    for (int q = 0; q < 32 / G; ++q) {
+        const int l = t + q * G;
+        s[q] = l < n ? v[l] : 0.0;
+        if (n > 32 + q * G) s[q] += l + 32 < n ? v[l + 32] : 0.0;
+    }
+#pragma unroll
+    for (int o = 16; o >= G; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < o / G; ++q)
+            if (n > o + q * G) s[q] += s[q + o / G];
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1)
+        if (n > o) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o, G);
+    return __shfl_sync(0xffffffffu, s[0], 0, G);
+}
+
+constexpr int kLevelsPerLane = 4;                 // G lanes hold up to 4 G levels
+static_assert(kMaxLevels <= 16 * kLevelsPerLane, "levels per lane");
+
+// v > 0 for a sum of non-negative numbers (false for NaN), by its bits: a
+// comparison on the FP64 pipe costs as much as a multiply-add.
+__device__ __forceinline__ bool positive_bits(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+
+// Point p, solved by the G lanes t = 0 .. G - 1 of its group in their
+// shared-memory slice sm; `write` false: a group past the last point, which
+// repeats that point (same warp) and writes nothing.
+template <int G> __device__ __forceinline__ void se_point(const SEArgs &a, int64_t p, double *sm, int t, bool write)
 {
     const int L = a.L, LL = L * L;
-    double *R = sm;                       // R[i*L + j]: rate i -> j
-    double *Sn = R + LL;                  // [L] reciprocals of the pivots
-    double *xx = Sn + L;                  // [L] unnormalised populations
-    double *bz = xx + L;                  // [L] Boltzmann factors g_i exp(-(E_i - E_0)/kT)
-    double *rdown = bz + L;               // [Mpad] radiative u -> l rate per line
-    double *rup = rdown + a.Mpad;         // [Mpad] radiative l -> u rate per line
+    double *R = sm;                       // R[i*L + j]: rate i -> j; diagonal: bz_i = g_i exp(-(E_i - E_0)/kT)
+    double *xx = R + LL;                  // [L] 1/bz, later the unnormalised populations
+    double *Sn = xx + L;                  // [L] reciprocals of the pivots
+    double *rdown = Sn, *rup = Sn + a.M;  // [M] each, before the pivots: radiative u -> l, l -> u rate per line
 
     const double *po = a.pops_old + p * L;
-    if (a.pops_prev)
-        for (int i = lane; i < L; i += 32) a.pops_prev[p * L + i] = po[i];
+    if (write)
+        for (int i = t; i < L; i += G) a.pops_prev[p * L + i] = po[i];
     const double Tp = a.T[p], nc = a.ncoll[p];
     // per-line preconditioned radiative rates
-    for (int k = lane; k < a.M; k += 32) {
+    for (int k = t; k < a.M; k += G) {
         const int u = a.line_ul[k], l = a.line_ul[a.Mpad + k];
         const double A = a.line_tab[a.Mpad + k], Bul = a.line_tab[2 * a.Mpad + k], Blu = a.line_tab[3 * a.Mpad + k];
         const double x_l = po[l] * Blu, x_u = po[u] * Bul;
@@ -89,102 +128,143 @@ __device__ __forceinline__ void se_point(const SEArgs &a, int64_t p, double *sm,
         rdown[k] = fmax(A * (1.0 - Ls) + Bul * Jeff, 0.0);
         rup[k] = fmax(Blu * Jeff, 0.0);
     }
+    for (int e = t; e < LL; e += G) R[e] = 0.0;
+    __syncwarp();
+    for (int k = t; k < a.M; k += G) R[a.line_ul[a.Mpad + k] * L + a.line_ul[k]] = rup[k];
     const double *E = a.level_tab, *g = a.level_tab + L;
     const double ikT = 1.0 / (kKB * Tp);
     // one exponential per level instead of one per collisional pair: the
     // upward rate C_lu = C_ul (g_u/g_l) exp(-(E_u - E_l)/kT) = C_ul bz_u / bz_l,
-    // formed with 1/bz_l from one division per level (kept in xx until the
-    // populations need it; FP64 division is a long sequence on this GPU's
-    // narrow FP64 pipe, and there are L^2/2 upward pairs)
-    for (int i = lane; i < L; i += 32) {
+    // formed with 1/bz_l from one division per level (FP64 division is a long
+    // sequence, and there are L^2/2 upward pairs)
+    for (int i = t; i < L; i += G) {
         const double b = g[i] * exp(-(E[i] - E[0]) * ikT);
-        bz[i] = b;
+        R[i * L + i] = b;
         xx[i] = b > 1e-290 ? 1.0 / b : 0.0;
     }
     __syncwarp();
-    for (int e = lane; e < LL; e += 32) {
-        const int i = e / L, j = e - i * L;
-        double v = 0.0;
-        if (i != j) {
-            const int kd = a.entry[e], ku = a.entry[LL + e], kc = a.entry[2 * LL + e];
-            if (kd >= 0) v += rdown[kd];
-            if (ku >= 0) v += rup[ku];
-            if (kc >= 0) {
-                const int cu = a.coll_ul[kc], cl = a.coll_ul[a.K + kc];
-                const double Cul = nc * a.Kul[kc];
-                if (i == cu)
-                    v += Cul;
-                else if (bz[cl] > 1e-290 && bz[cu] > 1e-290)
-                    v += Cul * bz[cu] * xx[cl];
-                else   // a factor near the bottom of the FP64 range: the pair's own exponential
-                    v += Cul * g[cu] / g[cl] * exp(-(E[cu] - E[cl]) * ikT);
-            }
-        }
-        R[e] = v;
+    for (int k = t; k < a.K; k += G) {
+        const int u = a.coll_ul[k], l = a.coll_ul[a.K + k];
+        const double Cul = __dmul_rn(nc, a.Kul[k]);
+        const double bu = R[u * L + u], ru = xx[u], rl = xx[l];
+        double &up = R[l * L + u];
+        R[u * L + l] = Cul;
+        // (1/bz is zero where the factor is near the bottom of the FP64 range:
+        // then the pair's own exponential)
+        if (__double2hiint(rl) != 0 && __double2hiint(ru) != 0)
+            up = __fma_rn(__dmul_rn(Cul, bu), rl, up);
+        else
+            up = __fma_rn(Cul * g[u] / g[l], exp(-(E[u] - E[l]) * ikT), up);
+    }
+    __syncwarp();
+    for (int k = t; k < a.M; k += G) {
+        double &down = R[a.line_ul[k] * L + a.line_ul[a.Mpad + k]];
+        down = __dadd_rn(rdown[k], down);
     }
     __syncwarp();
     // state reduction, highest level first
     for (int n = L - 1; n >= 1; --n) {
-        double part = 0.0;
-        for (int j = lane; j < n; j += 32) part += R[n * L + j];
-        double s = warp_sum_first(part, n);
-        s = s > 0.0 ? s : 1e-300;
-        // one lane divides (the division is a long FP64 sequence), all read it
-        double rs = 0.0;
-        if (lane == 0) {
-            rs = 1.0 / s;
-            Sn[n] = rs;
-        }
-        rs = __shfl_sync(0xffffffffu, rs, 0);
-        for (int j = lane; j < n; j += 32) R[n * L + j] *= rs;
+        double s = point_sum<G>(R + n * L, n, t);
+        s = positive_bits(s) ? s : 1e-300;
+        const double rs = 1.0 / s;
+        if (t == 0) Sn[n] = rs;
+        for (int j = t; j < n; j += G) R[n * L + j] *= rs;
         __syncwarp();
-        const int nn = n * n;
-        for (int e = lane; e < nn; e += 32) {
-            const int i = e / n, j = e - i * n;
-            R[i * L + j] += R[i * L + n] * R[n * L + j];
+        // rows i, columns j < n: entry e = i n + j, the stride advances (i, j)
+        // by (di, dj); with few warps per scheduler two entries at a time,
+        // loads before stores, so that their latencies overlap
+        constexpr int kUpdate = G == 16 ? 2 : 1;
+        const int di = G / n, dj = G - di * n;
+        int i = t / n, j = t - i * n;
+        for (int e = t; e < n * n; e += kUpdate * G) {
+            double *at[kUpdate];
+            double r[kUpdate], x[kUpdate], y[kUpdate];
+#pragma unroll
+            for (int q = 0; q < kUpdate; ++q) {
+                const bool in = e + q * G < n * n;
+                at[q] = R + (in ? i * L + j : 0);
+                r[q] = *at[q];
+                x[q] = R[in ? i * L + n : 0];
+                y[q] = R[n * L + (in ? j : 0)];
+                i += di;
+                j += dj;
+                if (j >= n) {
+                    j -= n;
+                    ++i;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kUpdate; ++q) r[q] += x[q] * y[q];
+#pragma unroll
+            for (int q = 0; q < kUpdate; ++q)
+                if (e + q * G < n * n) *at[q] = r[q];
         }
         __syncwarp();
     }
     // back substitution n_k = sum_{i<k} n_i R_ik / S_k, column by column: lane
-    // j keeps the running sums of levels j and j + 32, and once n_{k-1} is
+    // t keeps the running sums of levels t, t + G, ..., and once n_{k-1} is
     // known every lane adds its term to the levels above it (one FP64
-    // multiply-add per lane and level instead of a warp sum per level)
-    double acc0 = 0.0, acc1 = 0.0;
-    if (lane == 0) xx[0] = 1.0;
+    // multiply-add per lane and level instead of a sum over lanes per level)
+    double acc[kLevelsPerLane];
+#pragma unroll
+    for (int q = 0; q < kLevelsPerLane; ++q) acc[q] = 0.0;
+    if (t == 0) xx[0] = 1.0;
     double xprev = 1.0;                   // n_0
     for (int k = 1; k < L; ++k) {
         const int i = k - 1;              // n_i is known: add n_i R_ij to every level j > i
-        if (lane > i && lane < L) acc0 += xprev * R[i * L + lane];
-        if (lane + 32 > i && lane + 32 < L) acc1 += xprev * R[i * L + lane + 32];
-        // n_k = acc[k] / S_k from the lane that holds level k
-        const double a = k < 32 ? acc0 : acc1;
+        double ak = 0.0;
+#pragma unroll
+        for (int q = 0; q < kLevelsPerLane; ++q) {
+            const int j = t + q * G;
+            if (j > i && j < L) acc[q] += xprev * R[i * L + j];
+            if (q == k / G) ak = acc[q];
+        }
+        // n_k = acc / S_k from the lane that holds level k
         double nk = 0.0;
-        if ((k & 31) == lane) {
-            nk = a * Sn[k];
+        if (k % G == t) {
+            nk = ak * Sn[k];
             xx[k] = nk;
         }
-        xprev = __shfl_sync(0xffffffffu, nk, k & 31);
+        xprev = __shfl_sync(0xffffffffu, nk, k % G, G);
     }
     __syncwarp();
-    double part = 0.0;
-    for (int i = lane; i < L; i += 32) part += xx[i];
-    const double tot = warp_sum(part);
-    const double f = a.nspec[p] / tot;
-    for (int i = lane; i < L; i += 32) a.pops_out[p * L + i] = xx[i] * f;
+    const double f = a.nspec[p] / point_sum<G>(xx, L, t);
+    if (write)
+        for (int i = t; i < L; i += G) a.pops_out[p * L + i] = xx[i] * f;
+}
+
+// The calling warp's points of one model (32 / G of them, from first_warp on).
+template <int G> __device__ __forceinline__ void se_warp(const SEArgs &a, int64_t warp, double *sm)
+{
+    const int lane = threadIdx.x & 31, grp = lane / G;
+    const int64_t p = warp * (32 / G) + grp;
+    if (p - grp >= a.N) return;           // whole warp
+    se_point<G>(a, min(p, a.N - 1), sm + grp * se_point_doubles(a.L, a.M), lane - grp * G, p < a.N);
+}
+
+__device__ __forceinline__ void se_block(const SEArgs &a, int64_t block, double *sm)
+{
+    const int w = threadIdx.x >> 5;
+    if (w >= a.wpb) return;               // whole warp
+    const int G = se_lanes(a.L);
+    const int64_t warp = block * a.wpb + w;
+    sm += (int64_t)w * (32 / G) * se_point_doubles(a.L, a.M);
+    if (G == 16)
+        se_warp<16>(a, warp, sm);
+    else if (G == 8)
+        se_warp<8>(a, warp, sm);
+    else
+        se_warp<4>(a, warp, sm);
 }
 
 __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock) k_se(SEArgs a)
 {
     extern __shared__ __align__(16) double sm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per_warp = a.L * a.L + 3 * a.L + 2 * a.Mpad;
-    const int64_t p = (int64_t)blockIdx.x * a.wpb + warp;
-    if (p >= a.N) return;                 // whole warp leaves together
-    se_point(a, p, sm + warp * per_warp, lane);
+    se_block(a, blockIdx.x, sm);
 }
 
-// Many models in one launch, kMaxWarpsPerBlock points of one model per CTA:
-// blk_end[i] is one past the last CTA of model i.
+// Many models in one launch, one model per CTA: blk_end[i] is one past the last
+// CTA of model i.
 __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock) k_se_batch(const SEArgs *__restrict__ args,
                                                                      const int64_t *__restrict__ blk_end, int n_models)
 {
@@ -202,11 +282,7 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock) k_se_batch(const SEArg
         s_first = lo > 0 ? blk_end[lo - 1] : 0;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per_warp = sa.L * sa.L + 3 * sa.L + 2 * sa.Mpad;
-    const int64_t p = ((int64_t)blockIdx.x - s_first) * kMaxWarpsPerBlock + warp;
-    if (p >= sa.N) return;
-    se_point(sa, p, sm + warp * per_warp, lane);
+    se_block(sa, (int64_t)blockIdx.x - s_first, sm);
 }
 
 SEArgs fill_se_args(const mgt_model *m)
@@ -217,7 +293,7 @@ SEArgs fill_se_args(const mgt_model *m)
     a.M = m->M;
     a.Mpad = m->Mpad;
     a.K = m->K;
-    a.pops_old = m->d_pops_prev;
+    a.pops_old = m->d_pops;
     a.J = m->d_J;
     a.Lst = m->d_Lst;
     a.T = m->d_temp;
@@ -228,47 +304,51 @@ SEArgs fill_se_args(const mgt_model *m)
     a.level_tab = m->d_level_tab;
     a.Kul = m->d_coll_tab;
     a.coll_ul = m->d_coll_ul;
-    a.entry = m->d_entry;
     a.pops_out = m->d_pops;
+    a.pops_prev = m->d_pops_prev;
     return a;
 }
 
-size_t se_warp_bytes(const mgt_model *m) { return sizeof(double) * ((size_t)m->L * m->L + 3 * m->L + 2 * m->Mpad); }
+// Warps per CTA, CTAs and a CTA's shared memory; false if no warp's points fit.
+bool se_layout(const mgt_model *m, int *wpb, int64_t *blocks, size_t *smem)
+{
+    const int points = 32 / se_lanes(m->L);
+    const size_t per_warp = sizeof(double) * points * (size_t)se_point_doubles(m->L, m->M);
+    *wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, kSEMaxSmem / per_warp);
+    if (*wpb < 1) return false;
+    *blocks = ceil_div(m->N, (int64_t)*wpb * points);
+    *smem = per_warp * *wpb;
+    return true;
+}
 
 }  // namespace
 
 mgt_status launch_stat_eq(mgt_model *m, cudaStream_t s)
 {
     SEArgs a = fill_se_args(m);
-    const size_t per_warp = sizeof(double) * ((size_t)m->L * m->L + 3 * m->L + 2 * m->Mpad);
-    const size_t max_smem = 227 * 1024;
-    int wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, max_smem / per_warp);
-    if (wpb < 1) return set_error(MGT_ERR_ARG, "statistical equilibrium: too many levels/lines for shared memory");
-    a.wpb = wpb;
-    const size_t smem = per_warp * wpb;
+    int64_t blocks = 0;
+    size_t smem = 0;
+    if (!se_layout(m, &a.wpb, &blocks, &smem))
+        return set_error(MGT_ERR_ARG, "statistical equilibrium: too many levels/lines for shared memory");
     MGT_TRY_STATUS(raise_smem_limit((const void *)k_se, smem));
     {
         MGT_KTIMER("k_se", s);
-        k_se<<<ceil_div(m->N, wpb), 32 * wpb, smem, s>>>(a);
+        k_se<<<(unsigned)blocks, 32 * a.wpb, smem, s>>>(a);
     }
     MGT_LAUNCH_CHECK("k_se");
     return MGT_OK;
 }
 
-// Batched statistical equilibrium: the model's arguments with the previous
-// populations read from and written back to d_pops (the copy for Ng made by
-// the same warp into d_pops_prev).
 size_t se_args_bytes() { return sizeof(SEArgs); }
 
 mgt_status se_batch_args(const mgt_model *m, void *args, int64_t *blocks, size_t *smem)
 {
     SEArgs a = fill_se_args(m);
-    a.pops_old = m->d_pops;
-    a.pops_prev = m->d_pops_prev;
-    a.wpb = kMaxWarpsPerBlock;
-    *smem = se_warp_bytes(m) * kMaxWarpsPerBlock;
-    if (*smem > 227 * 1024) return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
-    *blocks = (m->N + kMaxWarpsPerBlock - 1) / kMaxWarpsPerBlock;
+    // the batch's documented limit
+    if (4 * sizeof(double) * ((size_t)m->L * m->L + 3 * m->L + 2 * m->Mpad) > kSEMaxSmem)
+        return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
+    if (!se_layout(m, &a.wpb, blocks, smem))
+        return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
     std::memcpy(args, &a, sizeof a);
     return MGT_OK;
 }

@@ -140,7 +140,6 @@ struct mgt_model {
     double *d_level_tab = nullptr;             // [2][L]: energy, g
     double *d_coll_tab = nullptr;              // [K]: K_ul
     int32_t *d_coll_ul = nullptr;              // [2][K]
-    int16_t *d_entry = nullptr;                // [3][L*L]: radiative-down line, radiative-up line, collision
     // device: state
     double *d_pops = nullptr, *d_pops_prev = nullptr;   // [N][L]
     float *d_line32 = nullptr;                 // [N][row_stride32] chi~', S', w, 1/w, 0, 0

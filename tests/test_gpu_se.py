@@ -1,0 +1,52 @@
+"""Statistical equilibrium at the edges of its lane and point groups, through
+the C-ABI against the oracle on the model's own J-bar and Lambda*.
+
+Tolerance 1e-8 relative, element by element, as in the parity tests: the state
+reduction keeps populations to about 2 L^3 rounding units (6e-11 at 64 levels),
+and the preconditioned rates lose digits where J-bar - Lambda* S cancels.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2411_03040_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mgt():
+    from paper_2411_03040_gb300 import build, mgt as binding
+    build.build()
+    binding.load()
+    return binding
+
+
+# lanes per point change above 16 and 32 levels; point counts leave the last
+# warp with one, some and all of its points
+@pytest.mark.parametrize("levels,n", [(2, 31), (3, 64), (15, 33), (16, 40), (17, 41), (31, 37), (32, 30), (33, 31),
+                                      (63, 29), (64, 32)])
+@pytest.mark.parametrize("batched", [False, True])
+def test_level_and_point_edges(mgt, levels, n, batched):
+    m = synth.sphere_model(n, levels, 1, 3, seed=50 + levels)
+    m.n_coll = m.n_coll * 1e-4
+    h = mgt.mgt_model_create(m)
+    mgt.mgt_trace_rays(h)
+    if batched:
+        other = synth.sphere_model(60, 5, 1, 3, seed=7)
+        ho = mgt.mgt_model_create(other)
+        mgt.mgt_trace_rays(ho)
+        b = mgt.mgt_batch_create([ho, h])
+        mgt.mgt_batch_formal_solve(b)
+        mgt.mgt_batch_stat_equilibrium(b)
+        got = mgt.mgt_get_populations(h)
+    else:
+        mgt.mgt_formal_solve(h, want=False)
+        got = mgt.mgt_stat_equilibrium(h)
+    J, L = mgt.mgt_get_jbar(h)
+    p0 = O.lte_populations(m.temp, m.n_spec, m.lines.energy_J, m.lines.g)
+    ref = O.stat_equilibrium(p0, J.T, L.T, m.temp, m.n_coll, m.n_spec, m.lines)
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-8
+    # the previous populations are kept for the change that Ng reports
+    _, change = mgt.mgt_ng_accelerate(h)
+    assert change == pytest.approx(np.max(np.abs(got - p0) / p0), rel=1e-9)
