@@ -9,10 +9,10 @@
 //
 // Three kernels:
 //  * k_fs_staged: one CTA per origin.  Each half-ray is cut into chunks of CH
-//    steps; warp 0 moves the next chunk's step records and point rows (line
-//    data + width) into shared memory with bulk asynchronous copies
-//    (cp.async.bulk, completion on an mbarrier) while the CTA eliminates the
-//    current chunk from shared memory.
+//    steps; the next chunk's point rows (line data + width) and the step
+//    records of the chunk after it move into shared memory by bulk
+//    asynchronous copies (cp.async.bulk, completion on an mbarrier) while the
+//    CTA eliminates the current chunk from shared memory.
 //  * k_fs_gather: several origins per CTA (small bin x line counts); every
 //    thread gathers its rows straight from global memory.
 //  * k_fs_batch: the staged body for the items (model, origin, line block) of
@@ -35,13 +35,12 @@
 // q = 1/(1 + beta G), Pi <- G q, Y <- (S h + Y) q -- eight FP32 operations
 // and one reciprocal per line and step, from Pi = 2, alpha = 0 at the far end.
 //
-// Staged kernel, per chunk of a half-ray: first the CTA's threads (in a CTA of
-// 128 threads or more all but warp 0, which issues the copies) compute
-// line-independent segment coefficients for a share of the chunk's (bin,
-// step) pairs (Gaussian at both ends, trapezoid/erf switch, erf difference)
-// into shared memory, then each thread eliminates its lines reading one
-// coefficient pair per step, two steps per trip.  The line groups of a bin
-// do not repeat the coefficient work.
+// Staged kernel, per chunk of a half-ray: first the CTA's threads compute
+// line-independent segment coefficients for a share of the chunk's (bin, step)
+// pairs (Gaussian at both ends, trapezoid/erf switch, erf difference) into
+// shared memory, then each thread eliminates its lines reading one coefficient
+// pair per step, two steps per trip.  The line groups of a bin do not repeat
+// the coefficient work.
 #include <algorithm>
 #include <cstring>
 
@@ -799,38 +798,56 @@ __device__ __forceinline__ bool next_chunk(const longlong2 *ext, int P, const Ch
     return cur.h == 0 ? first_chunk_from(ext, P, cur.p, 1, CH, nx) : first_chunk_from(ext, P, cur.p + 1, 0, CH, nx);
 }
 
-// Issue the copies of chunk c into one buffer (warp 0).  Point slot j holds
-// c_{k_lo-1+j} (c_0 = o); step slot j holds the record of step k_lo-1+j
-// (slot 0 unused when k_lo = 1).
+// Bytes and source of the step records of chunk c: slot j of its buffer holds
+// the record of step k_lo - 1 + j (slot 0 unused when k_lo = 1).
+template <typename T> __device__ __forceinline__ uint32_t step_bytes(const Chunk &c)
+{
+    return (uint32_t)((c.k_hi - max(1, c.k_lo - 1) + 1) * (sizeof(T) == 4 ? 16 : 32));
+}
+
 template <typename T>
-__device__ __forceinline__ void issue_chunk(const FSArgs &a, int64_t o, const Chunk &c, unsigned char *steps_buf,
-                                            unsigned char *rows_buf, uint64_t *bar, int rowB, int lane)
+__device__ __forceinline__ void copy_steps(const FSArgs &a, const Chunk &c, unsigned char *steps_buf, uint64_t *bar)
 {
     constexpr int SB = sizeof(T) == 4 ? 16 : 32;
-    const int npts = c.k_hi - c.k_lo + 2;
     const int kf = max(1, c.k_lo - 1);
-    const int nsteps = c.k_hi - kf + 1;
-    const uint32_t bytes = (uint32_t)(npts * rowB + nsteps * SB);
-    const unsigned char *lines = reinterpret_cast<const unsigned char *>(a.line);
-    if (lane == 0) mbar_expect_tx(bar, bytes);
+    const void *src = sizeof(T) == 4 ? (const void *)(a.s32 + c.s0 + kf - 1) : (const void *)(a.s64 + c.s0 + kf - 1);
+    bulk_g2s(steps_buf + (kf - (c.k_lo - 1)) * SB, src, step_bytes<T>(c), bar);
+}
+
+// Copy point pt's row (an index out of range: record, copy row 0).
+__device__ __forceinline__ void copy_row(const FSArgs &a, int64_t o, int64_t pt, unsigned char *dst, uint64_t *bar,
+                                         int rowB)
+{
+    if (pt < 0 || pt >= a.N) {
+        if (atomicCAS(a.err, 0, (int)kDevBounds) == 0) {
+            a.err[1] = 20;
+            a.err[2] = (int)o;
+            a.err[3] = (int)pt;
+        }
+        pt = 0;
+    }
+    bulk_g2s(dst, static_cast<const unsigned char *>(a.line) + pt * (int64_t)rowB, (uint32_t)rowB, bar);
+}
+
+// Issue the copies of chunk c into one buffer by warp 0 alone, with the point
+// indices read from global memory: point slot j holds the row of c_{k_lo-1+j}
+// (c_0 = o).  With `ahead` also the step records of the chunk after, c2.
+template <typename T>
+__device__ __forceinline__ void issue_chunk(const FSArgs &a, int64_t o, const Chunk &c, unsigned char *steps_buf,
+                                            bool ahead, const Chunk &c2, unsigned char *ahead_buf,
+                                            unsigned char *rows_buf, uint64_t *bar, int rowB, int lane)
+{
+    const int npts = c.k_hi - c.k_lo + 2;
+    if (lane == 0) mbar_expect_tx(bar, (uint32_t)(npts * rowB) + step_bytes<T>(c) + (ahead ? step_bytes<T>(c2) : 0u));
     __syncwarp();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (lane < npts) {
         const int k = c.k_lo - 1 + lane;
-        int64_t pt = k == 0 ? o : (int64_t)__ldg(&a.s32[c.s0 + k - 1].x);
-        if (pt < 0 || pt >= a.N) {   // a point index from the ray records out of range: record, copy row 0
-            if (atomicCAS(a.err, 0, (int)kDevBounds) == 0) {
-                a.err[1] = 20;
-                a.err[2] = (int)o;
-                a.err[3] = (int)pt;
-            }
-            pt = 0;
-        }
-        bulk_g2s(rows_buf + lane * rowB, lines + pt * (int64_t)rowB, (uint32_t)rowB, bar);
+        copy_row(a, o, k == 0 ? o : (int64_t)__ldg(&a.s32[c.s0 + k - 1].x), rows_buf + lane * rowB, bar, rowB);
     }
     if (lane == 0) {
-        const void *src = sizeof(T) == 4 ? (const void *)(a.s32 + c.s0 + kf - 1) : (const void *)(a.s64 + c.s0 + kf - 1);
-        bulk_g2s(steps_buf + (kf - (c.k_lo - 1)) * SB, src, (uint32_t)(nsteps * SB), bar);
+        copy_steps<T>(a, c, steps_buf, bar);
+        if (ahead) copy_steps<T>(a, c2, ahead_buf, bar);
     }
 }
 
@@ -840,7 +857,14 @@ struct StagedLayout {
     int stage, coef, ibg, sab, acc, half0, ext, total;
 };
 
-// Staging buffers [2] and coefficient buffers [2] are contiguous; the final
+// Bins rounded up to whole pairs.
+__host__ __device__ inline int bins_even(int Q) { return (Q + 1) & ~1; }
+
+// Buffers of step records: the chunk in work, the next, and the one after,
+// whose records are on their way.
+constexpr int kStepBufs = 3;
+
+// Staging buffers and coefficient buffers [2] are contiguous; the final
 // FP64 reduction area aliases them once the last chunk is done.
 template <typename T, int LPT, int CH>
 __host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int bd, int P, bool fused)
@@ -850,7 +874,7 @@ __host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int
     auto up = [](int x) { return (x + 15) & ~15; };
     StagedLayout L;
     const int rowB = RS * (int)sizeof(T);
-    const int stage_bytes = 2 * NPT * (SB + rowB);
+    const int stage_bytes = NPT * (kStepBufs * SB + 2 * rowB);
     const int coef_bytes = fused ? 0 : 2 * (CH + 1) * Q * 2 * (int)sizeof(T);
     const int red_bytes = 2 * Mb * Q * (int)sizeof(double);
     L.stage = 128;
@@ -858,7 +882,7 @@ __host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int
     const int pipe_end = L.coef + up(coef_bytes);
     L.ibg = pipe_end > L.stage + up(red_bytes) ? pipe_end : L.stage + up(red_bytes);
     L.sab = L.ibg + up(Mb * Q * (int)sizeof(T));
-    L.acc = L.sab + up(2 * Q * (int)sizeof(T));
+    L.acc = L.sab + up(2 * bins_even(Q) * (int)sizeof(T));
     L.half0 = L.acc + up(3 * LPT * bd * (int)sizeof(T));
     L.ext = L.half0 + up(3 * LPT * bd * (int)sizeof(T));
     L.total = L.ext + 2 * P * 16;
@@ -901,45 +925,36 @@ __device__ __forceinline__ typename Prec<T>::V2 segment_item(const FSArgs &a, in
     return V2{cf, cn};
 }
 
-// Two items of the FP32 pre-pass at once on packed FP32 (one lane per item),
-// lane for lane the arithmetic of segment_item / segment_coefs, so the
-// coefficients are bit-identical.  An item's inputs:
-struct PairIn {
-    float dx, z_f, z_n, du, w_f, w_n, rw_f, rw_n;
-    bool trap, band;
-};
-
 __device__ __forceinline__ float2 f2(float x, float y) { return make_float2(x, y); }
 __device__ __forceinline__ float2 f2s(float x) { return make_float2(x, x); }
 
-// Both items on the same branch (neither near the switch): their halved
-// {cf, cn} in c0, c1.
-__device__ __forceinline__ void segment_pair(const PairIn &i0, const PairIn &i1, int width_mode, float2 &c0,
-                                             float2 &c1)
+// What a step's segment coefficients take from its two points, whatever the bin.
+struct StepPts {
+    float dx, w_f, w_n, rw_f, rw_n;
+};
+
+// The halved {cf, cn} of one step for two bins at once on packed FP32 (one lane
+// per bin), both on the same branch and not near the switch: lane for lane the
+// arithmetic of segment_item / segment_coefs, so the coefficients are
+// bit-identical.
+__device__ __forceinline__ void segment_pair(const StepPts &st, float2 z_f, float2 z_n, float2 du, bool trap,
+                                             int width_mode, float2 &cf, float2 &cn)
 {
-    const float2 dx = f2(i0.dx, i1.dx), wf = f2(i0.w_f, i1.w_f), wn = f2(i0.w_n, i1.w_n);
-    float2 cf, cn;
-    if (i0.trap) {
+    if (trap) {
         // Gaussians of the far and near points (point_gauss on each lane)
-        const float2 uf = __fmul2_rn(f2(i0.z_f, i1.z_f), f2(i0.rw_f, i1.rw_f));
-        const float2 un = __fmul2_rn(f2(i0.z_n, i1.z_n), f2(i0.rw_n, i1.rw_n));
+        const float2 uf = __fmul2_rn(z_f, f2s(st.rw_f)), un = __fmul2_rn(z_n, f2s(st.rw_n));
         const float2 yf = __fmul2_rn(__fmul2_rn(uf, uf), f2s(-kLog2E));
         const float2 yn = __fmul2_rn(__fmul2_rn(un, un), f2s(-kLog2E));
         const float2 gf = f2(ex2_mufu(yf.x), ex2_mufu(yf.y)), gn = f2(ex2_mufu(yn.x), ex2_mufu(yn.y));
-        const float2 q = __fmul2_rn(f2s(0.25f), dx);
+        const float2 q = f2s(__fmul_rn(0.25f, st.dx));
         cf = __fmul2_rn(q, gf);
         cn = __fmul2_rn(q, gn);
     } else {
-        float2 iw;
-        if (width_mode == 0) {
-            const float2 h = __fmul2_rn(f2s(0.5f), __ffma2_rn(wf, wf, __fmul2_rn(wn, wn)));
-            iw = f2(rsqrtf(h.x), rsqrtf(h.y));
-        } else {
-            const float2 h = __fmul2_rn(f2s(0.5f), __fadd2_rn(wf, wn));
-            iw = f2(Prec<float>::rcp(h.x), Prec<float>::rcp(h.y));
-        }
-        const float2 du = f2(i0.du, i1.du);
-        float2 a = __fmul2_rn(f2(i0.z_f, i1.z_f), iw);
+        const float iw =
+            width_mode == 0
+                ? rsqrtf(__fmul_rn(0.5f, __fmaf_rn(st.w_f, st.w_f, __fmul_rn(st.w_n, st.w_n))))
+                : Prec<float>::rcp(__fmul_rn(0.5f, __fadd_rn(st.w_f, st.w_n)));
+        float2 a = __fmul2_rn(z_f, f2s(iw));
         float2 b = __fadd2_rn(a, du);
         const float2 sab = __fadd2_rn(a, b);
         if (sab.x < 0.0f) {
@@ -955,13 +970,11 @@ __device__ __forceinline__ void segment_pair(const PairIn &i0, const PairIn &i1,
         const float2 ea = erfc_fit2(a.x, a.y), eb = erfc_fit2(b.x, b.y);
         const float2 E = __fadd2_rn(ea, f2(-eb.x, -eb.y));
         const float2 rdu = f2(Prec<float>::rcp(du.x), Prec<float>::rcp(du.y));
-        const float2 kk =
-            __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(dx, f2s(float(0.125 * kSqrtPi))), E), iw), rdu);
-        cf = __fmul2_rn(kk, wf);
-        cn = __fmul2_rn(kk, wn);
+        const float2 kk = __fmul2_rn(
+            __fmul2_rn(__fmul2_rn(f2s(__fmul_rn(st.dx, float(0.125 * kSqrtPi))), E), f2s(iw)), rdu);
+        cf = __fmul2_rn(kk, f2s(st.w_f));
+        cn = __fmul2_rn(kk, f2s(st.w_n));
     }
-    c0 = f2(cf.x, cn.x);
-    c1 = f2(cf.y, cn.y);
 }
 
 // Line-independent coefficients of every (bin, step) of one chunk, shared by
@@ -969,14 +982,21 @@ __device__ __forceinline__ void segment_pair(const PairIn &i0, const PairIn &i1,
 // for bin q.  Each bin's steps are contiguous, so the elimination steps its
 // pointer by a constant; the row stride cs = CH + 1 is odd, so the threads of
 // consecutive bins read different banks.
-// Two ways to share the items among the CTA's threads:
-//  * strided (CARRY false): item kk * Q + q to thread (kk * Q + q) mod bd;
-//  * runs (CARRY true): thread t takes bin t mod Q and a run of consecutive
-//    steps; the near point of a step is the far point of the step before, so
-//    its Gaussian is carried instead of recomputed.  This pays where the
-//    pre-pass dominates (few lines per origin, 4 lines per thread), while with
-//    many lines the extra live registers cost more than the saved exponentials.
-template <typename T, bool CARRY>
+// The items are shared among all threads of the CTA:
+//  * FP32 (the switch rule): a thread keeps one pair of adjacent bins and takes
+//    every nslots-th step, so the bins' offsets stay in registers, a step's
+//    record and widths are read and its mean width formed once for both bins,
+//    and a warp's lanes are on few different steps (one branch).  With
+//    pairs of items dealt out one by one, each reading its own step, the
+//    launch of 100k shell points (40 lines x 50 bins, 48 rays) took 150.8 ms,
+//    now 143.6 with the rows asked for by all warps (see fs_staged_item; 145.7
+//    with warp 0 asking alone and taking no items, 152.1 with it taking its
+//    share); 10-line models 3.35 -> 2.72 ms, 20-line ones 5.03 -> 4.16.
+//  * FP64: thread t takes bin t mod Q and a run of consecutive steps; the near
+//    point of a step is the far point of the step before, so its Gaussian is
+//    carried instead of recomputed.
+//  * the subdivided reference: item kk Q + q to thread (kk Q + q) mod bd.
+template <typename T>
 __device__ __forceinline__ void chunk_coefs(const FSArgs &a, int64_t o, int r, int k_lo, int k_hi,
                                             const unsigned char *Sb, const T *Rb, const T *sA, const T *sB,
                                             typename Prec<T>::V2 *coef, int cs, int tid, int bd)
@@ -988,121 +1008,68 @@ __device__ __forceinline__ void chunk_coefs(const FSArgs &a, int64_t o, int r, i
     auto one = [&](int kk, int q, T Aq, T Bq, const StepG<T> &sf, T z_f, auto gpair) {
         coef[q * cs + kk] = segment_item<T>(a, o, r, k_lo + kk, q, Sb, Rb, kk + 1, Aq, Bq, sf, z_f, gpair);
     };
-    if constexpr (CARRY) {
-        const int nseg = bd / a.Q;                     // Q <= bd: bins x line groups fit the CTA
-        const int seg = tid / a.Q, q = tid - seg * a.Q;
-        const int sps = (nst + nseg - 1) / nseg;
-        const int kk0 = seg * sps, kk1 = min(nst, kk0 + sps);
-        if (seg >= nseg || kk0 >= kk1) return;
-        const T Aq = sA[q], Bq = sB[q];
-        T g_n = point_gauss<T>(bin_z<T>(Aq, Bq, k_lo + kk0 > 1 ? step_from<T>(Sb + kk0 * SB).beta : T(0)),
-                               Rb[kk0 * a.RS + 2 * a.Mpad + 1]);
+    if constexpr (sizeof(T) == 8) {
+        if (a.subdiv == 0) {
+            const int nseg = bd / a.Q;                     // Q <= bd: bins x line groups fit the CTA
+            const int seg = tid / a.Q, q = tid - seg * a.Q;
+            const int sps = (nst + nseg - 1) / nseg;
+            const int kk0 = seg * sps, kk1 = min(nst, kk0 + sps);
+            if (seg >= nseg || kk0 >= kk1) return;
+            const T Aq = sA[q], Bq = sB[q];
+            T g_n = point_gauss<T>(bin_z<T>(Aq, Bq, k_lo + kk0 > 1 ? step_from<T>(Sb + kk0 * SB).beta : T(0)),
+                                   Rb[kk0 * a.RS + 2 * a.Mpad + 1]);
 #pragma unroll 1
-        for (int kk = kk0; kk < kk1; ++kk) {
-            const StepG<T> sf = step_from<T>(Sb + (kk + 1) * SB);
-            const T z_f = bin_z<T>(Aq, Bq, sf.beta);
-            const T g_f = point_gauss<T>(z_f, Rb[(kk + 1) * a.RS + 2 * a.Mpad + 1]);
-            one(kk, q, Aq, Bq, sf, z_f, [&] { return V2{g_f, g_n}; });
-            g_n = g_f;
+            for (int kk = kk0; kk < kk1; ++kk) {
+                const StepG<T> sf = step_from<T>(Sb + (kk + 1) * SB);
+                const T z_f = bin_z<T>(Aq, Bq, sf.beta);
+                const T g_f = point_gauss<T>(z_f, Rb[(kk + 1) * a.RS + 2 * a.Mpad + 1]);
+                one(kk, q, Aq, Bq, sf, z_f, [&] { return V2{g_f, g_n}; });
+                g_n = g_f;
+            }
+            return;
         }
     } else {
-        // warp 0 issues the bulk copies after the barrier: in a wide CTA it
-        // takes no items, and the last threads take the extra items of an
-        // uneven split
-        // item it = kk Q + q; the stride advances (kk, q) by (dk, dq)
-        // without a division per item
-        const int items = a.Q * nst;
-        const int pw = bd >= 128 ? 32 : 0;
-        const int stride = bd - pw;
-        const int dk = stride / a.Q, dq = stride - dk * a.Q;
-        const int it0 = tid >= pw ? bd - 1 - tid : items;
-        int kk = it0 / a.Q, q = it0 - kk * a.Q;
-        if constexpr (sizeof(T) == 4) {
-            if (a.subdiv == 0) {
-                // two adjacent items per trip (bins q and q + 1 of one step,
-                // or the last bin of a step and the first of the next), on
-                // packed FP32 when both take the same branch away from the
-                // switch
-                auto item_in = [&](int kk_, int q_, PairIn &in, StepG<T> &sf, T &Aq, T &Bq, T &beta_n) {
-                    const int k = k_lo + kk_, jf = kk_ + 1;
-                    sf = step_from<T>(Sb + jf * SB);
-                    beta_n = k > 1 ? step_from<T>(Sb + kk_ * SB).beta : T(0);
-                    Aq = sA[q_];
-                    Bq = sB[q_];
-                    in.dx = sf.dx;
-                    in.z_f = bin_z<T>(Aq, Bq, sf.beta);
-                    in.z_n = bin_z<T>(Aq, Bq, beta_n);
-                    in.w_f = Rb[jf * a.RS + 2 * a.Mpad];
-                    in.w_n = Rb[kk_ * a.RS + 2 * a.Mpad];
-                    in.rw_f = Rb[jf * a.RS + 2 * a.Mpad + 1];
-                    in.rw_n = Rb[kk_ * a.RS + 2 * a.Mpad + 1];
-                    in.du = -Prec<T>::mul(Bq, sf.dbw);
-                    in.trap = fabs(in.du) < (T)a.thr;
-                    in.band = fabs(fabs(in.du) - (T)a.thr) < T(kSwitchBand) * (T)a.thr;
-                };
-                auto single = [&](int kk_, int q_, const StepG<T> &sf, T Aq, T Bq, const PairIn &in) {
-                    one(kk_, q_, Aq, Bq, sf, in.z_f, [&] {
-                        return V2{point_gauss<T>(in.z_f, in.rw_f), point_gauss<T>(in.z_n, in.rw_n)};
-                    });
-                };
-                const int npairs = (items + 1) >> 1;
-                const int pstride2 = 2 * stride;
-                const int dk2 = pstride2 / a.Q, dq2 = pstride2 - dk2 * a.Q;
-                const int p0 = tid >= pw ? bd - 1 - tid : npairs;
-                int kk0 = (2 * p0) / a.Q, q0 = 2 * p0 - kk0 * a.Q;
+        if (a.subdiv == 0) {
+            const int np = bins_even(a.Q) >> 1, nslots = bd / np;
+            const int slot = tid / np, q = 2 * (tid - slot * np);
+            if (slot >= nslots) return;
+            const float2 A = *reinterpret_cast<const float2 *>(sA + q), B = *reinterpret_cast<const float2 *>(sB + q);
+            const bool two = q + 1 < a.Q;                  // an odd last bin has no partner
+            const float thr = (float)a.thr, band = kSwitchBand * thr;
 #pragma unroll 1
-                for (int pi = p0; pi < npairs; pi += stride) {
-                    int kk1 = kk0, q1 = q0 + 1;
-                    if (q1 >= a.Q) {
-                        q1 = 0;
-                        ++kk1;
-                    }
-                    PairIn in0, in1;
-                    StepG<T> sf0, sf1;
-                    T A0, B0, bn0, A1, B1, bn1;
-                    item_in(kk0, q0, in0, sf0, A0, B0, bn0);
-                    if (2 * pi + 1 < items) {
-                        item_in(kk1, q1, in1, sf1, A1, B1, bn1);
-                        if (!in0.band && !in1.band && in0.trap == in1.trap) {
-                            float2 c0, c1;
-                            segment_pair(in0, in1, a.width_mode, c0, c1);
-                            coef[q0 * cs + kk0] = c0;
-                            coef[q1 * cs + kk1] = c1;
-                        } else {
-                            single(kk0, q0, sf0, A0, B0, in0);
-                            single(kk1, q1, sf1, A1, B1, in1);
-                        }
-                    } else {
-                        single(kk0, q0, sf0, A0, B0, in0);
-                    }
-                    kk0 += dk2;
-                    q0 += dq2;
-                    if (q0 >= a.Q) {
-                        q0 -= a.Q;
-                        ++kk0;
-                    }
+            for (int kk = slot; kk < nst; kk += nslots) {
+                const StepG<float> sf = step_from<float>(Sb + (kk + 1) * SB);
+                const float beta_n = k_lo + kk > 1 ? step_from<float>(Sb + kk * SB).beta : 0.0f;
+                const float2 wf = *reinterpret_cast<const float2 *>(Rb + (kk + 1) * a.RS + 2 * a.Mpad);
+                const float2 wn = *reinterpret_cast<const float2 *>(Rb + kk * a.RS + 2 * a.Mpad);
+                const StepPts st{sf.dx, wf.x, wn.x, wf.y, wn.y};
+                // bin_z on each lane, and the reduced Doppler shift
+                const float2 z_f = __ffma2_rn(B, f2s(sf.beta), A), z_n = __ffma2_rn(B, f2s(beta_n), A);
+                const float2 m = __fmul2_rn(B, f2s(sf.dbw)), du = f2(-m.x, -m.y);
+                const bool t0 = fabsf(du.x) < thr, t1 = fabsf(du.y) < thr;
+                if (t0 == t1 && !(fabsf(fabsf(du.x) - thr) < band) && !(fabsf(fabsf(du.y) - thr) < band)) {
+                    float2 cf, cn;
+                    segment_pair(st, z_f, z_n, du, t0, a.width_mode, cf, cn);
+                    coef[q * cs + kk] = f2(cf.x, cn.x);
+                    if (two) coef[(q + 1) * cs + kk] = f2(cf.y, cn.y);
+                } else {
+                    one(kk, q, A.x, B.x, sf, z_f.x,
+                        [&] { return V2{point_gauss<float>(z_f.x, wf.y), point_gauss<float>(z_n.x, wn.y)}; });
+                    if (two)
+                        one(kk, q + 1, A.y, B.y, sf, z_f.y,
+                            [&] { return V2{point_gauss<float>(z_f.y, wf.y), point_gauss<float>(z_n.y, wn.y)}; });
                 }
-                return;
             }
+            return;
         }
+    }
+    // the subdivided reference (any precision)
 #pragma unroll 1
-        for (int it = it0; it < items; it += stride) {
-            const int k = k_lo + kk;
-            const StepG<T> sf = step_from<T>(Sb + (kk + 1) * SB);
-            const T beta_n = k > 1 ? step_from<T>(Sb + kk * SB).beta : T(0);
-            const T Aq = sA[q], Bq = sB[q];
-            const T z_f = bin_z<T>(Aq, Bq, sf.beta);
-            one(kk, q, Aq, Bq, sf, z_f, [&] {
-                return V2{point_gauss<T>(z_f, Rb[(kk + 1) * a.RS + 2 * a.Mpad + 1]),
-                          point_gauss<T>(bin_z<T>(Aq, Bq, beta_n), Rb[kk * a.RS + 2 * a.Mpad + 1])};
-            });
-            kk += dk;
-            q += dq;
-            if (q >= a.Q) {
-                q -= a.Q;
-                ++kk;
-            }
-        }
+    for (int it = tid; it < a.Q * nst; it += bd) {
+        const int kk = it / a.Q, q = it - kk * a.Q;
+        const StepG<T> sf = step_from<T>(Sb + (kk + 1) * SB);
+        const T Aq = sA[q], Bq = sB[q];
+        one(kk, q, Aq, Bq, sf, bin_z<T>(Aq, Bq, sf.beta), [&] { return V2{T(0), T(0)}; });
     }
 }
 
@@ -1140,11 +1107,11 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
 
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);                   // [2]
     int *abort_flag = reinterpret_cast<int *>(smem + 16);
-    unsigned char *steps_s = smem + lay.stage;                            // steps [2][NPT][SB]
-    unsigned char *rows_s = steps_s + 2 * NPT * SB;                       // rows [2][NPT][rowB]
+    unsigned char *steps_s = smem + lay.stage;                            // steps [kStepBufs][NPT][SB]
+    unsigned char *rows_s = steps_s + kStepBufs * NPT * SB;               // rows [2][NPT][rowB]
     V2 *coef = reinterpret_cast<V2 *>(smem + lay.coef);                   // [2][Q][CH + 1]
     T *ibg = reinterpret_cast<T *>(smem + lay.ibg);                       // [Mb][Q]
-    T *sA = reinterpret_cast<T *>(smem + lay.sab), *sB = sA + a.Q;        // [Q] each
+    T *sA = reinterpret_cast<T *>(smem + lay.sab), *sB = sA + bins_even(a.Q);   // [Q, rounded up to even] each
     T *acc = reinterpret_cast<T *>(smem + lay.acc);                       // [3][LPT][bd]
     T *half0 = reinterpret_cast<T *>(smem + lay.half0);                   // [3][LPT][bd] first half's P, Y, a
     longlong2 *ext = reinterpret_cast<longlong2 *>(smem + lay.ext);       // [2 P] half-ray extents
@@ -1158,8 +1125,8 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
 
     const double wo64 = a.w64[o];
     fill_extents(a, o, ext, tid, bd);
-    if (tid < a.Q) {
-        const T Aq = T(a.xq[tid]) * T(wo64);
+    if (tid < bins_even(a.Q)) {           // (an odd last bin's partner repeats it)
+        const T Aq = T(a.xq[min(tid, a.Q - 1)]) * T(wo64);
         sA[tid] = Aq;
         sB[tid] = T(1) + Aq;
     }
@@ -1174,10 +1141,30 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
     }
     __syncthreads();
 
-    Chunk cur;
-    const bool any = first_chunk_from(ext, a.P, 0, 0, CH, cur);
-    if (any && warp == 0) issue_chunk<T>(a, o, cur, steps_s + (ci & 1) * NPT * SB, rows_s + (ci & 1) * NPT * rowB,
-                                         &bar[ci & 1], rowB, lane);
+    // FP32 (AHEAD): step records travel one chunk ahead of the rows, so the
+    // point indices of the next chunk are in shared memory when its rows are
+    // asked for, and every warp asks for its share of them: a bulk copy is
+    // issued by one lane after the other, and 31 of them from one warp, after
+    // a global load of the indices, held that warp back by more than a trip of
+    // the pre-pass.  plan[] holds the coming chunks (k_hi = 0: none), written
+    // by warp 0 one chunk before all warps read it.  FP64 records have no
+    // point indices: warp 0 alone issues a chunk.
+    constexpr bool AHEAD = sizeof(T) == 4;
+    auto steps_of = [&](int c) { return steps_s + c * NPT * SB; };
+    Chunk *plan = reinterpret_cast<Chunk *>(smem + 32);                   // [kStepBufs]
+    int cs = 0;                                    // the chunk's step buffer and plan entry
+    if (warp == 0) {
+        Chunk cur, nx{};
+        if (first_chunk_from(ext, a.P, 0, 0, CH, cur)) {
+            const bool ahead = AHEAD && next_chunk(ext, a.P, cur, CH, nx);
+            issue_chunk<T>(a, o, cur, steps_of(0), ahead, nx, steps_of(1), rows_s + (ci & 1) * NPT * rowB,
+                           &bar[ci & 1], rowB, lane);
+            if (AHEAD && lane == 0) {
+                if (!ahead) nx.k_hi = 0;
+                plan[1] = nx;
+            }
+        }
+    }
 
     const T wqn = active ? T(a.wq[q]) : T(0);
     bool ok = true;
@@ -1208,11 +1195,11 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
             for (int k_hi = n; k_hi >= 1; k_hi -= CH) {
                 const int k_lo = max(1, k_hi - CH + 1);
                 ok = mbar_wait_bounded(&bar[ci & 1], (ci >> 1) & 1);
-                const unsigned char *Sb = steps_s + (ci & 1) * NPT * SB;
+                const unsigned char *Sb = steps_of(cs);
                 const T *Rb = reinterpret_cast<const T *>(rows_s + (ci & 1) * NPT * rowB);
                 V2 *cf_buf = coef + (ci & 1) * (CH + 1) * a.Q;
                 if constexpr (!FUSED) {
-                    if (ok) chunk_coefs<T, LPT == 4>(a, o, r, k_lo, k_hi, Sb, Rb, sA, sB, cf_buf, CH + 1, tid, bd);
+                    if (ok) chunk_coefs<T>(a, o, r, k_lo, k_hi, Sb, Rb, sA, sB, cf_buf, CH + 1, tid, bd);
                 }
                 // one barrier per chunk: this chunk's coefficients are complete, and
                 // everyone is done with the previous chunk (its staging buffer is
@@ -1223,12 +1210,35 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     goto done;
                 }
 
-                if (warp == 0) {
+                uint64_t *nbar = &bar[(ci + 1) & 1];
+                unsigned char *nrows = rows_s + ((ci + 1) & 1) * NPT * rowB;
+                if constexpr (AHEAD) {
+                    const int c1 = cs + 1 == kStepBufs ? 0 : cs + 1, c2 = c1 + 1 == kStepBufs ? 0 : c1 + 1;
+                    const int klo = plan[c1].k_lo, khi = plan[c1].k_hi;
+                    if (khi > 0) {
+                        const int npts = khi - klo + 2, nw = bd >> 5, j = warp + lane * nw;
+                        if (j < npts)
+                            copy_row(a, o, klo - 1 + j == 0 ? o : reinterpret_cast<const int4 *>(steps_of(c1))[j].x,
+                                     nrows + j * rowB, nbar, rowB);
+                        if (warp == 0) {
+                            const Chunk nx = plan[c1];
+                            Chunk n2{};
+                            const bool ahead = next_chunk(ext, a.P, nx, CH, n2);
+                            if (lane == 0) {
+                                // (copies that complete first leave the count below zero until this)
+                                mbar_expect_tx(nbar, (uint32_t)(npts * rowB) + (ahead ? step_bytes<T>(n2) : 0u));
+                                if (ahead) copy_steps<T>(a, n2, steps_of(c2), nbar);
+                                else n2.k_hi = 0;
+                                plan[c2] = n2;
+                            }
+                        }
+                    }
+                } else if (warp == 0) {
                     Chunk nx;
                     const Chunk c{p, h, s0, n, k_lo, k_hi};
                     if (next_chunk(ext, a.P, c, CH, nx))
-                        issue_chunk<T>(a, o, nx, steps_s + ((ci + 1) & 1) * NPT * SB,
-                                       rows_s + ((ci + 1) & 1) * NPT * rowB, &bar[(ci + 1) & 1], rowB, lane);
+                        issue_chunk<T>(a, o, nx, steps_of(cs + 1 == kStepBufs ? 0 : cs + 1), false, nx, nullptr, nrows,
+                                       nbar, rowB, lane);
                 }
                 if (FUSED && active) {
                     // the same rows with each step's coefficients computed here
@@ -1335,6 +1345,7 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     }
                 }
                 ++ci;
+                cs = cs + 1 == kStepBufs ? 0 : cs + 1;
             }
             if (h == 0) {
                 if (active) {
