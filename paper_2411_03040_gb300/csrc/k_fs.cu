@@ -123,6 +123,7 @@ struct FSArgs {
     int lpt;                   // lines per thread of the staged schedule (batched launches)
     int nblk;                  // line blocks per origin (ceil(Gtot / Gb))
     int fused;                 // staged schedule with each thread's coefficients in registers (Gtot == 1)
+    int step_bufs;             // buffers of step records (staged schedule; see staged_step_bufs)
     double *J, *Lst;           // [N][M]
     int *err;
     const int *range_bad;      // nonzero: a point's range figure exceeds 1 (set by the line data)
@@ -857,24 +858,24 @@ struct StagedLayout {
     int stage, coef, ibg, sab, acc, half0, ext, total;
 };
 
-// Bins rounded up to whole pairs.
-__host__ __device__ inline int bins_even(int Q) { return (Q + 1) & ~1; }
+// Bins rounded up to whole pairs (FP32, which takes them in pairs).
+template <typename T> __host__ __device__ inline int bins_held(int Q) { return sizeof(T) == 4 ? (Q + 1) & ~1 : Q; }
 
 // Buffers of step records: the chunk in work, the next, and the one after,
-// whose records are on their way.
+// whose records are on their way; two where the records do not travel ahead.
 constexpr int kStepBufs = 3;
 
 // Staging buffers and coefficient buffers [2] are contiguous; the final
 // FP64 reduction area aliases them once the last chunk is done.
 template <typename T, int LPT, int CH>
-__host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int bd, int P, bool fused)
+__host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int bd, int P, bool fused, int step_bufs)
 {
     constexpr int SB = sizeof(T) == 4 ? 16 : 32;
     constexpr int NPT = CH + 1;
     auto up = [](int x) { return (x + 15) & ~15; };
     StagedLayout L;
     const int rowB = RS * (int)sizeof(T);
-    const int stage_bytes = NPT * (kStepBufs * SB + 2 * rowB);
+    const int stage_bytes = NPT * (step_bufs * SB + 2 * rowB);
     const int coef_bytes = fused ? 0 : 2 * (CH + 1) * Q * 2 * (int)sizeof(T);
     const int red_bytes = 2 * Mb * Q * (int)sizeof(double);
     L.stage = 128;
@@ -882,7 +883,7 @@ __host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int
     const int pipe_end = L.coef + up(coef_bytes);
     L.ibg = pipe_end > L.stage + up(red_bytes) ? pipe_end : L.stage + up(red_bytes);
     L.sab = L.ibg + up(Mb * Q * (int)sizeof(T));
-    L.acc = L.sab + up(2 * bins_even(Q) * (int)sizeof(T));
+    L.acc = L.sab + up(2 * bins_held<T>(Q) * (int)sizeof(T));
     L.half0 = L.acc + up(3 * LPT * bd * (int)sizeof(T));
     L.ext = L.half0 + up(3 * LPT * bd * (int)sizeof(T));
     L.total = L.ext + 2 * P * 16;
@@ -1030,7 +1031,7 @@ __device__ __forceinline__ void chunk_coefs(const FSArgs &a, int64_t o, int r, i
         }
     } else {
         if (a.subdiv == 0) {
-            const int np = bins_even(a.Q) >> 1, nslots = bd / np;
+            const int np = bins_held<T>(a.Q) >> 1, nslots = bd / np;
             const int slot = tid / np, q = 2 * (tid - slot * np);
             if (slot >= nslots) return;
             const float2 A = *reinterpret_cast<const float2 *>(sA + q), B = *reinterpret_cast<const float2 *>(sB + q);
@@ -1103,15 +1104,15 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
     const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rowB = a.RS * (int)sizeof(T);
     const int Mb = a.Gb * LPT;
-    const StagedLayout lay = staged_layout<T, LPT, CH>(a.Q, Mb, a.RS, bd, a.P, FUSED);
+    const StagedLayout lay = staged_layout<T, LPT, CH>(a.Q, Mb, a.RS, bd, a.P, FUSED, a.step_bufs);
 
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);                   // [2]
     int *abort_flag = reinterpret_cast<int *>(smem + 16);
-    unsigned char *steps_s = smem + lay.stage;                            // steps [kStepBufs][NPT][SB]
-    unsigned char *rows_s = steps_s + kStepBufs * NPT * SB;               // rows [2][NPT][rowB]
+    unsigned char *steps_s = smem + lay.stage;                            // steps [step_bufs][NPT][SB]
+    unsigned char *rows_s = steps_s + a.step_bufs * NPT * SB;             // rows [2][NPT][rowB]
     V2 *coef = reinterpret_cast<V2 *>(smem + lay.coef);                   // [2][Q][CH + 1]
     T *ibg = reinterpret_cast<T *>(smem + lay.ibg);                       // [Mb][Q]
-    T *sA = reinterpret_cast<T *>(smem + lay.sab), *sB = sA + bins_even(a.Q);   // [Q, rounded up to even] each
+    T *sA = reinterpret_cast<T *>(smem + lay.sab), *sB = sA + bins_held<T>(a.Q);  // [bins_held] each
     T *acc = reinterpret_cast<T *>(smem + lay.acc);                       // [3][LPT][bd]
     T *half0 = reinterpret_cast<T *>(smem + lay.half0);                   // [3][LPT][bd] first half's P, Y, a
     longlong2 *ext = reinterpret_cast<longlong2 *>(smem + lay.ext);       // [2 P] half-ray extents
@@ -1125,7 +1126,7 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
 
     const double wo64 = a.w64[o];
     fill_extents(a, o, ext, tid, bd);
-    if (tid < bins_even(a.Q)) {           // (an odd last bin's partner repeats it)
+    if (tid < bins_held<T>(a.Q)) {           // (an odd last bin's partner repeats it)
         const T Aq = T(a.xq[min(tid, a.Q - 1)]) * T(wo64);
         sA[tid] = Aq;
         sB[tid] = T(1) + Aq;
@@ -1148,8 +1149,9 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
     // a global load of the indices, held that warp back by more than a trip of
     // the pre-pass.  plan[] holds the coming chunks (k_hi = 0: none), written
     // by warp 0 one chunk before all warps read it.  FP64 records have no
-    // point indices: warp 0 alone issues a chunk.
-    constexpr bool AHEAD = sizeof(T) == 4;
+    // point indices, and the third step buffer may not fit: warp 0 alone then
+    // issues a chunk.
+    const bool AHEAD = sizeof(T) == 4 && a.step_bufs == kStepBufs;
     auto steps_of = [&](int c) { return steps_s + c * NPT * SB; };
     Chunk *plan = reinterpret_cast<Chunk *>(smem + 32);                   // [kStepBufs]
     int cs = 0;                                    // the chunk's step buffer and plan entry
@@ -1212,7 +1214,7 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
 
                 uint64_t *nbar = &bar[(ci + 1) & 1];
                 unsigned char *nrows = rows_s + ((ci + 1) & 1) * NPT * rowB;
-                if constexpr (AHEAD) {
+                if (AHEAD) {
                     const int c1 = cs + 1 == kStepBufs ? 0 : cs + 1, c2 = c1 + 1 == kStepBufs ? 0 : c1 + 1;
                     const int klo = plan[c1].k_lo, khi = plan[c1].k_hi;
                     if (khi > 0) {
@@ -1237,7 +1239,7 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     Chunk nx;
                     const Chunk c{p, h, s0, n, k_lo, k_hi};
                     if (next_chunk(ext, a.P, c, CH, nx))
-                        issue_chunk<T>(a, o, nx, steps_of(cs + 1 == kStepBufs ? 0 : cs + 1), false, nx, nullptr, nrows,
+                        issue_chunk<T>(a, o, nx, steps_of(cs + 1 == a.step_bufs ? 0 : cs + 1), false, nx, nullptr, nrows,
                                        nbar, rowB, lane);
                 }
                 if (FUSED && active) {
@@ -1345,7 +1347,7 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     }
                 }
                 ++ci;
-                cs = cs + 1 == kStepBufs ? 0 : cs + 1;
+                cs = cs + 1 == a.step_bufs ? 0 : cs + 1;
             }
             if (h == 0) {
                 if (active) {
@@ -1577,7 +1579,19 @@ template <typename T, int LPT> FSArgs fill_fs_args(const mgt_model *m, bool accu
     a.n_rec = m->total_steps;
     a.lpt = LPT;
     a.nblk = ceil_div(a.Gtot, a.Gb);
+    a.step_bufs = 2;
     return a;
+}
+
+// Step buffers of a launch: FP32 records travel one chunk ahead where the third
+// buffer fits the shared memory with the rest (it does unless a model has some
+// hundred lines).
+template <typename T, int LPT, int CH> int staged_step_bufs(const FSArgs &a, int bd, bool fused)
+{
+    return sizeof(T) == 4 &&
+                   staged_layout<T, LPT, CH>(a.Q, a.Gb * LPT, a.RS, bd, a.P, fused, kStepBufs).total <= 227 * 1024
+               ? kStepBufs
+               : 2;
 }
 
 // The staged launch: the two-row kernel and, for the two-row form, the
@@ -1639,7 +1653,8 @@ mgt_status launch_typed(mgt_model *m, cudaStream_t s, int schedule, bool accumul
         const int threads = a.Q * a.Gb;
         const int bd = ((threads + 31) / 32) * 32;
         if (bd > 256) return set_error(MGT_ERR_ARG, "formal solve: more than 256 bins per origin");
-        const size_t smem = (size_t)staged_layout<T, LPT, kChunk>(a.Q, Mb, a.RS, bd, a.P, a.fused != 0).total;
+        a.step_bufs = staged_step_bufs<T, LPT, kChunk>(a, bd, a.fused != 0);
+        const size_t smem = (size_t)staged_layout<T, LPT, kChunk>(a.Q, Mb, a.RS, bd, a.P, a.fused != 0, a.step_bufs).total;
         dim3 grid((unsigned)m->N, (unsigned)ceil_div(a.Gtot, a.Gb));
         // the two-row elimination in FP32 (the subdivided reference keeps the
         // one-row form; the range argument needs half-rays below kFastSteps)
@@ -1707,6 +1722,9 @@ mgt_status fs_batch_args(const mgt_model *m, void *args, int *threads, int64_t *
     *items = a.N * a.nblk;
     *fused = a.fused;
     *lines = a.lpt;
+    // (by the long chunks, which need more)
+    a.step_bufs = lpt == 4 ? staged_step_bufs<float, 4, kChunk>(a, bd, a.fused != 0)
+                           : staged_step_bufs<float, 8, kChunk>(a, bd, a.fused != 0);
     std::memcpy(args, &a, sizeof a);
     return MGT_OK;
 }
@@ -1727,10 +1745,10 @@ size_t fs_batch_smem(const void *args, int bd)
     const int Mb = a.Gb * a.lpt;
     const bool f = a.fused != 0;
     if (narrow_chunks(bd, a.fused))
-        return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f).total
-                          : (size_t)staged_layout<float, 8, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f).total;
-    return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunk>(a.Q, Mb, a.RS, bd, a.P, f).total
-                      : (size_t)staged_layout<float, 8, kChunk>(a.Q, Mb, a.RS, bd, a.P, f).total;
+        return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total
+                          : (size_t)staged_layout<float, 8, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total;
+    return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunk>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total
+                      : (size_t)staged_layout<float, 8, kChunk>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total;
 }
 
 namespace {

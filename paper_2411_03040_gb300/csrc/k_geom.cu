@@ -211,22 +211,36 @@ mgt_status build_walk_tables(mgt_model *m, const double lo[3], const double hi[3
 // ---------------------------------------------------------------------------
 // LTE: n_i = n_spec g_i exp(-(E_i - E_0)/kT) / sum_j g_j exp(-(E_j - E_0)/kT).
 // ---------------------------------------------------------------------------
-__global__ void k_lte(int64_t N, int L, const double *__restrict__ T, const double *__restrict__ nspec,
-                      const double *__restrict__ level_tab, double *__restrict__ pops)
+// Eight lanes per point, lanes over levels; the partition function is summed
+// in level order by every lane from shared memory.  With one thread per point
+// a small model's launch was two dependent chains of L exponentials (31 us for
+// any point count up to 20,000, now 7 us).
+constexpr int kLteThreads = 128, kLteLanes = 8;
+
+__global__ void __launch_bounds__(kLteThreads) k_lte(int64_t N, int L, const double *__restrict__ T,
+                                                     const double *__restrict__ nspec,
+                                                     const double *__restrict__ level_tab, double *__restrict__ pops)
 {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= N) return;
+    __shared__ double ex[kLteThreads / kLteLanes][kMaxLevels];
+    const int grp = threadIdx.x / kLteLanes, t = threadIdx.x - grp * kLteLanes;
+    const int64_t p = blockIdx.x * (int64_t)(kLteThreads / kLteLanes) + grp;
     const double *E = level_tab, *g = level_tab + L;
-    double beta = 1.0 / (kKB * T[p]);
+    double beta = 0.0;
+    if (p < N) {
+        beta = 1.0 / (kKB * T[p]);
+        for (int i = t; i < L; i += kLteLanes) ex[grp][i] = exp(-(E[i] - E[0]) * beta);
+    }
+    __syncwarp();
+    if (p >= N) return;
     double Z = 0.0;
-    for (int i = 0; i < L; ++i) Z += g[i] * exp(-(E[i] - E[0]) * beta);
-    double f = nspec[p] / Z;
-    for (int i = 0; i < L; ++i) pops[p * L + i] = f * g[i] * exp(-(E[i] - E[0]) * beta);
+    for (int i = 0; i < L; ++i) Z = __fma_rn(g[i], ex[grp][i], Z);
+    const double f = nspec[p] / Z;
+    for (int i = t; i < L; i += kLteLanes) pops[p * L + i] = __dmul_rn(__dmul_rn(f, g[i]), ex[grp][i]);
 }
 
 mgt_status launch_lte(mgt_model *m, cudaStream_t s)
 {
-    k_lte<<<ceil_div(m->N, 128), 128, 0, s>>>(m->N, m->L, m->d_temp, m->d_nspec, m->d_level_tab, m->d_pops);
+    k_lte<<<ceil_div(m->N, (int64_t)(kLteThreads / kLteLanes)), kLteThreads, 0, s>>>(m->N, m->L, m->d_temp, m->d_nspec, m->d_level_tab, m->d_pops);
     MGT_LAUNCH_CHECK("k_lte");
     m->line_dirty = true;
     return MGT_OK;
@@ -246,7 +260,11 @@ mgt_status launch_lte(mgt_model *m, cudaStream_t s)
 // G = max(chi~max dxmax / 2^8, S'max / 2^80) of the formal solution's two-row
 // elimination (chi~max, S'max the largest over the point's lines, dxmax its
 // longest graph edge) and a zero.
-// One warp per point; lane j takes line slots j, j + 32, ...
+// A block takes kLDPoints points and deals out their (point, line slot) items
+// 256 at a time: bound by the FP64 pipe (16 cycles per warp instruction whatever
+// the active lanes), which with one warp per point ran 40 slots in two trips of
+// 32 lanes and three divisions per point in one lane.  100k points x 40 lines:
+// 0.42 -> 0.14 ms; x 4 lines 0.21 -> 0.04 ms.
 // ---------------------------------------------------------------------------
 struct LDArgs {
     int64_t N;
@@ -261,82 +279,107 @@ struct LDArgs {
     int *range_bad;           // set when a point's range figure exceeds 1 (zeroed before the launch)
 };
 
-__device__ __forceinline__ void line_data_point(const LDArgs &d, int64_t p, int lane)
+constexpr int kLDThreads = 256, kLDPoints = 32;
+
+// Points p0 .. p0 + kLDPoints - 1 of a model, by the whole block.
+__device__ __forceinline__ void line_data_block(const LDArgs &d, int64_t p0)
 {
-    if (p >= d.N) return;                            // whole warp: p is warp-uniform
+    __shared__ double s_cw[kLDPoints];
+    __shared__ int s_chi[kLDPoints], s_src[kLDPoints];   // largest chi~', S' (bits; non-negative, a NaN is largest)
+    const int n = (int)min((int64_t)kLDPoints, d.N - p0);
     const int Mpad = d.Mpad, RS = row_stride32(Mpad), RS64 = row_stride64(Mpad);
     const double *__restrict__ line_tab = d.line_tab;
     const int32_t *__restrict__ line_ul = d.line_ul;
-    float *__restrict__ r32 = d.out32 + p * RS;
-    double *__restrict__ r64 = d.out64 ? d.out64 + p * RS64 : nullptr;
-    float chi_max = 0.0f, S_max = 0.0f;
-    // h L_unit / (4 pi sqrt(pi) w): one FP64 division per point (lane 0), not per line
-    double cw = 0.0;
-    if (lane == 0) cw = kH * d.Lunit / (4.0 * kPi * kSqrtPi * d.w64[p]);
-    cw = __shfl_sync(0xffffffffu, cw, 0);
-    for (int k = lane; k < Mpad; k += 32) {
-        double a0 = 0.0, a1 = 0.0;
-        if (k < d.M) {
-            const int u = line_ul[k], l = line_ul[Mpad + k];
-            const double Bul = line_tab[2 * Mpad + k], Blu = line_tab[3 * Mpad + k];
-            const double nbgmax = line_tab[4 * Mpad + k];
-            const double nu_ = d.pops[p * d.L + u], nl_ = d.pops[p * d.L + l];
-            const double a = nl_ * Blu, b = nu_ * Bul;
-            double net = a - b;
-            const double floor_ = 1e-30 * (a + b);
-            if (net < floor_) {
-                net = floor_;
-                atomicAdd(d.n_floor, 1ULL);
-            }
-            if (net > 0.0) {
-                a0 = net * cw;
-                a1 = b / (net * nbgmax);
-            }
-        }
-        const float f0 = (float)a0, f1 = (float)a1;
-        r32[k] = f0;
-        r32[Mpad + k] = f1;
-        // !(x <= m) also carries a NaN into the bound, which then disables the
-        // fast elimination for every step through this point
-        chi_max = !(f0 <= chi_max) ? f0 : chi_max;
-        S_max = !(f1 <= S_max) ? f1 : S_max;
-        if (r64) {
-            r64[k] = a0;
-            r64[Mpad + k] = a1;
-        }
+    const int tid = threadIdx.x;
+    if (tid < n) {
+        // h L_unit / (4 pi sqrt(pi) w): one FP64 division per point, not per line
+        s_cw[tid] = kH * d.Lunit / (4.0 * kPi * kSqrtPi * d.w64[p0 + tid]);
+        s_chi[tid] = s_src[tid] = 0;
     }
+    __syncthreads();
+    // item e = (point e / Mpad, slot e mod Mpad); 8 neighbouring lanes share a
+    // point (Mpad and the block are multiples of 8)
+    const int dp = kLDThreads / Mpad, dk = kLDThreads - dp * Mpad;
+    int i = tid / Mpad, k = tid - i * Mpad;
+    for (int e0 = 0; e0 < n * Mpad; e0 += kLDThreads) {
+        float f0 = 0.0f, f1 = 0.0f;
+        if (i < n) {
+            const int64_t p = p0 + i;
+            double a0 = 0.0, a1 = 0.0;
+            if (k < d.M) {
+                const int u = line_ul[k], l = line_ul[Mpad + k];
+                const double Bul = line_tab[2 * Mpad + k], Blu = line_tab[3 * Mpad + k];
+                const double nbgmax = line_tab[4 * Mpad + k];
+                const double nu_ = d.pops[p * d.L + u], nl_ = d.pops[p * d.L + l];
+                const double a = nl_ * Blu, b = nu_ * Bul;
+                double net = a - b;
+                const double floor_ = 1e-30 * (a + b);
+                if (net < floor_) {
+                    net = floor_;
+                    atomicAdd(d.n_floor, 1ULL);
+                }
+                if (net > 0.0) {
+                    a0 = net * s_cw[i];
+                    a1 = b / (net * nbgmax);
+                }
+            }
+            f0 = (float)a0;
+            f1 = (float)a1;
+            float *r32 = d.out32 + p * RS;
+            r32[k] = f0;
+            r32[Mpad + k] = f1;
+            if (d.out64) {
+                double *r64 = d.out64 + p * RS64;
+                r64[k] = a0;
+                r64[Mpad + k] = a1;
+            }
+        }
+        int c = f0 == f0 ? __float_as_int(f0) : 0x7fffffff, t = f1 == f1 ? __float_as_int(f1) : 0x7fffffff;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float c = __shfl_xor_sync(0xffffffffu, chi_max, o), t = __shfl_xor_sync(0xffffffffu, S_max, o);
-        chi_max = !(c <= chi_max) ? c : chi_max;
-        S_max = !(t <= S_max) ? t : S_max;
+        for (int o = 4; o > 0; o >>= 1) {
+            c = max(c, __shfl_xor_sync(0xffffffffu, c, o));
+            t = max(t, __shfl_xor_sync(0xffffffffu, t, o));
+        }
+        if ((tid & 7) == 0 && i < n) {
+            atomicMax(&s_chi[i], c);
+            atomicMax(&s_src[i], t);
+        }
+        i += dp;
+        k += dk;
+        if (k >= Mpad) {
+            k -= Mpad;
+            ++i;
+        }
     }
-    if (lane == 0) {
-        const double w = d.w64[p];
+    __syncthreads();
+    if (tid < n) {
+        const int64_t p = p0 + tid;
+        const double w = d.w64[p], rw = 1.0 / w;
+        float *r32 = d.out32 + p * RS;
         r32[2 * Mpad] = (float)w;
-        r32[2 * Mpad + 1] = (float)(1.0 / w);
+        r32[2 * Mpad + 1] = (float)rw;
         // range figure of the formal solution's two-row elimination: at most 1
         // when every step through the point has half depths <= kTwoRowDepth and
         // sources <= kTwoRowSource; NaN and infinity give a figure above 1
         // (a width above 1% of c, where no real line is, would also let the
         // background of the far bins outgrow the range: it sets the flag too)
+        const float chi_max = __int_as_float(s_chi[tid]), S_max = __int_as_float(s_src[tid]);
         const float G = fmaxf(chi_max * d.dxmax[p] / kTwoRowDepth, S_max / kTwoRowSource);
         const bool inside = chi_max == chi_max && S_max == S_max && G <= 1.0f && w < 0.01;
         r32[2 * Mpad + 2] = inside ? G : 2.0f;
         r32[2 * Mpad + 3] = 0.0f;
         if (!inside) atomicOr(d.range_bad, 1);
-        if (r64) {
+        if (d.out64) {
+            double *r64 = d.out64 + p * RS64;
             r64[2 * Mpad] = w;
-            r64[2 * Mpad + 1] = 1.0 / w;
+            r64[2 * Mpad + 1] = rw;
         }
     }
 }
 
-constexpr int kLDThreads = 256, kLDPointsPerBlock = kLDThreads / 32;
-
 __global__ void __launch_bounds__(kLDThreads) k_line_data(LDArgs d)
 {
-    line_data_point(d, (int64_t)blockIdx.x * kLDPointsPerBlock + (threadIdx.x >> 5), threadIdx.x & 31);
+    line_data_block(d, (int64_t)blockIdx.x * kLDPoints);
 }
 
 // Many models in one launch: blk_end[i] is one past the last CTA of model i.
@@ -356,7 +399,7 @@ __global__ void __launch_bounds__(kLDThreads) k_line_data_batch(const LDArgs *__
         s_first = lo > 0 ? blk_end[lo - 1] : 0;
     }
     __syncthreads();
-    line_data_point(sd, ((int64_t)blockIdx.x - s_first) * kLDPointsPerBlock + (threadIdx.x >> 5), threadIdx.x & 31);
+    line_data_block(sd, ((int64_t)blockIdx.x - s_first) * kLDPoints);
 }
 
 static LDArgs fill_ld_args(const mgt_model *m)
@@ -373,7 +416,7 @@ mgt_status launch_line_data(mgt_model *m, cudaStream_t s)
         const double ld_bytes = (double)m->N * (8.0 * m->L + 8.0 + 4.0 * row_stride32(m->Mpad) +
                                                  (m->d_line64 ? 8.0 * row_stride64(m->Mpad) : 0.0));
         MGT_KTIMER_BYTES("k_line_data", s, ld_bytes);
-        k_line_data<<<ceil_div(m->N, (int64_t)kLDPointsPerBlock), kLDThreads, 0, s>>>(fill_ld_args(m));
+        k_line_data<<<ceil_div(m->N, (int64_t)kLDPoints), kLDThreads, 0, s>>>(fill_ld_args(m));
     }
     MGT_LAUNCH_CHECK("k_line_data");
     m->line_dirty = false;
@@ -386,7 +429,7 @@ mgt_status ld_batch_args(const mgt_model *m, void *args, int64_t *blocks)
 {
     const LDArgs a = fill_ld_args(m);
     std::memcpy(args, &a, sizeof a);
-    *blocks = ceil_div(m->N, (int64_t)kLDPointsPerBlock);
+    *blocks = ceil_div(m->N, (int64_t)kLDPoints);
     return MGT_OK;
 }
 
