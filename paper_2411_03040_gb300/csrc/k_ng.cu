@@ -29,6 +29,23 @@ __device__ __forceinline__ void atomic_max_pos(double *addr, double v)
     atomicMax(reinterpret_cast<unsigned long long *>(addr), (unsigned long long)__double_as_longlong(v));
 }
 
+// The block's maximum of v (non-negative, in every thread) into *addr: one
+// atomic per block.  With one per thread, 55,000 entries took 30 us in the
+// queue of one address.
+__device__ __forceinline__ void block_max_pos(double *addr, double v)
+{
+    __shared__ double red[kNgThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < kNgThreads / 32; ++k) v = fmax(v, red[k]);
+        atomic_max_pos(addr, v);
+    }
+    __syncthreads();
+}
+
 // Push: x_new = pops / n_spec into `out` (if not null); dots[k] = <r_new, r_k>
 // for the m-1 stored residuals and dots[m-1] = <r_new, r_new>, r_new = x_new -
 // h[m-1]; maxrel = max |pops - prev| / |prev| over prev != 0.
@@ -60,7 +77,7 @@ __global__ void __launch_bounds__(kNgThreads) k_ng_push(int64_t n, int L, const 
             out[e] = pv / nspec[e / L];
         }
     }
-    atomic_max_pos(maxrel, mr);
+    block_max_pos(maxrel, mr);
     __shared__ double red[kNgThreads];
     for (int k = 0; k < m; ++k) {
         double v = 0.0;
@@ -78,14 +95,23 @@ __global__ void __launch_bounds__(kNgThreads) k_ng_push(int64_t n, int L, const 
     }
 }
 
-// Sum block partials in block order: out[k] = sum_b partials[b][k].
-__global__ void k_ng_finish(int nblocks, int m, const double *__restrict__ partials, double *__restrict__ out)
+// Sum block partials in block order: out[k] = sum_b partials[b][k], one warp per
+// k.  The additions stay one chain (their order is part of the result); the
+// loads of 32 partials at a time run ahead of it.
+__global__ void __launch_bounds__(32 * kMaxNgHist) k_ng_finish(int nblocks, int m, const double *__restrict__ partials,
+                                                               double *__restrict__ out)
 {
-    const int k = threadIdx.x;
-    if (k >= m) return;
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * kMaxNgHist + k];
-    out[k] = s;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (k >= m) return;                           // whole warp
+    double s = 0.0, next = lane < nblocks ? partials[(size_t)lane * kMaxNgHist + k] : 0.0;
+    for (int b0 = 0; b0 < nblocks; b0 += 32) {
+        const double v = next;
+        const int b = b0 + 32 + lane;
+        next = b < nblocks ? partials[(size_t)b * kMaxNgHist + k] : 0.0;
+        const int n = min(32, nblocks - b0);
+        for (int j = 0; j < n; ++j) s += __shfl_sync(0xffffffffu, v, j);
+    }
+    if (lane == 0) out[k] = s;
 }
 
 struct Coef {
@@ -101,7 +127,9 @@ __global__ void __launch_bounds__(kNgThreads) k_ng_predict(int64_t n, Slots hs, 
     double mr = 0.0, neg = 0.0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         double x = 0.0;
-        for (int k = 0; k < nc; ++k) x += cf.c[k] * hs.h[k + 1][e];
+#pragma unroll
+        for (int k = 0; k < kMaxNgHist; ++k)      // (constant indices keep the parameters out of local memory)
+            if (k < nc) x += cf.c[k] * hs.h[k + 1][e];
         out[e] = x;
         if (x < 0.0) neg = 1.0;
         if (prev) {
@@ -109,8 +137,8 @@ __global__ void __launch_bounds__(kNgThreads) k_ng_predict(int64_t n, Slots hs, 
             if (pp != 0.0) mr = fmax(mr, fabs(x - pp) / fabs(pp));
         }
     }
-    atomic_max_pos(red + 0, mr);
-    atomic_max_pos(red + 1, neg);
+    block_max_pos(red + 0, mr);
+    block_max_pos(red + 1, neg);
 }
 
 __global__ void k_ng_apply(int64_t n, int L, const double *__restrict__ x, const double *__restrict__ nspec,
@@ -266,7 +294,7 @@ mgt_status ng_begin(mgt_model *m, const mgt_ng_opts *o, cudaStream_t s)
                                               hs, mh, ng.d_partials, ng.d_red + kMaxNgHist);
     }
     MGT_LAUNCH_CHECK("k_ng_push");
-    k_ng_finish<<<1, 32, 0, s>>>(grid, mh, ng.d_partials, ng.d_red);
+    k_ng_finish<<<1, 32 * kMaxNgHist, 0, s>>>(grid, mh, ng.d_partials, ng.d_red);
     MGT_LAUNCH_CHECK("k_ng_finish");
     MGT_CUDA(cudaMemcpyAsync(ng.h_red, ng.d_red, sizeof(double) * (kMaxNgHist + 1), cudaMemcpyDeviceToHost, s));
     ng.pend.phase = 1;
