@@ -1689,7 +1689,12 @@ int fs_lines_per_thread(const mgt_model *m, mgt_precision p)
 {
     if (p == MGT_FP64) return 4;
     if (m->opts.lines_per_thread == 4 || m->opts.lines_per_thread == 8) return m->opts.lines_per_thread;
-    return m->M <= 4 ? 4 : 8;
+    // 8 lines per thread share a bin's coefficient and opacity loads, unless
+    // padding the lines to 8 would waste more: up to 4 lines (half), and 9 to
+    // 12 (a quarter; 40k-point sphere, 31 bins: 10 lines 2.72 ms with 4 lines
+    // per thread, 3.47 with 8).  At 17 to 20 lines the two are even (4.16 and
+    // 4.18 ms for 20).  Results do not depend on it.
+    return m->M <= 4 || (m->M > 8 && m->M <= 12) ? 4 : 8;
 }
 
 mgt_status launch_formal_solve(mgt_model *m, mgt_precision p, cudaStream_t s, bool accumulate)
