@@ -93,7 +93,6 @@ template <> struct Prec<double> {
     static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
     static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
     static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
-    static __device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
     static __device__ __forceinline__ double bg(double f, double hk) { return f * f * f / expm1(hk * f); }
 };
 
@@ -123,16 +122,20 @@ struct FSArgs {
     int lpt;                   // lines per thread of the staged schedule (batched launches)
     int nblk;                  // line blocks per origin (ceil(Gtot / Gb))
     int fused;                 // staged schedule with each thread's coefficients in registers (Gtot == 1)
-    int step_bufs;             // buffers of step records (staged schedule; see staged_step_bufs)
     double *J, *Lst;           // [N][M]
     int *err;
     const int *range_bad;      // nonzero: a point's range figure exceeds 1 (set by the line data)
     int64_t n_rec;             // step records held (the ray offsets index below this)
 };
 
-// Geometry of one traced step in the solver's precision.
+// Geometry of one traced step in the solver's precision (FP64 also: the
+// inverse averaged width of the segment that ends at the step's point).
 template <typename T> struct StepG {
     T dx, beta, dbw;
+};
+
+template <> struct StepG<double> {
+    double dx, beta, dbw, iw;
 };
 
 template <typename T> __device__ __forceinline__ StepG<T> step_from(const void *p);
@@ -147,7 +150,7 @@ template <> __device__ __forceinline__ StepG<double> step_from<double>(const voi
 {
     const double2 *q = reinterpret_cast<const double2 *>(p);
     const double2 v0 = q[0], v1 = q[1];
-    return {v0.x, v0.y, v1.x};
+    return {v0.x, v0.y, v1.x, v1.y};
 }
 
 template <typename T> __device__ __forceinline__ StepG<T> step_global(const FSArgs &a, int64_t s);
@@ -162,7 +165,7 @@ template <> __device__ __forceinline__ StepG<double> step_global<double>(const F
 {
     const double2 *q = reinterpret_cast<const double2 *>(a.s64 + s);
     const double2 v0 = __ldg(q), v1 = __ldg(q + 1);
-    return {v0.x, v0.y, v1.x};
+    return {v0.x, v0.y, v1.x, v1.y};
 }
 
 // LPT consecutive scalars of a row (global or shared memory), 16-byte aligned.
@@ -229,18 +232,26 @@ __device__ __noinline__ bool trapezoid_fp64(const FSArgs &a, int r, int64_t c_fa
 // erfc values) or they straddle zero and E >= erf(|du|/2) (|du| >= threshold).
 // Both coefficients are returned halved: half the segment's optical depth is
 // cf chi~_far + cn chi~_near.
+// The averaged width's inverse comes from the FP64 step record (a square root
+// and a division, 21 instructions of the FP64 pipe per bin and step); in FP32
+// it is formed here.
 template <typename T>
-__device__ __forceinline__ void segment_coefs(bool trap, T dx, T du, T z_f, T g_f, T w_f, T g_n, T w_n, int width_mode,
-                                              T &cf, T &cn)
+__device__ __forceinline__ void segment_coefs(bool trap, const StepG<T> &st, T du, T z_f, T g_f, T w_f, T g_n, T w_n,
+                                              int width_mode, T &cf, T &cn)
 {
+    const T dx = st.dx;
     using P = Prec<T>;
     if (trap) {
         const T q = P::mul(T(0.25), dx);
         cf = P::mul(q, g_f);
         cn = P::mul(q, g_n);
     } else {
-        const T iwbar = width_mode == 0 ? P::rsqrt_(P::mul(T(0.5), P::fma(w_f, w_f, P::mul(w_n, w_n))))
-                                        : P::rcp(P::mul(T(0.5), P::add(w_f, w_n)));
+        T iwbar;
+        if constexpr (sizeof(T) == 8)
+            iwbar = st.iw;
+        else
+            iwbar = width_mode == 0 ? P::rsqrt_(P::mul(T(0.5), P::fma(w_f, w_f, P::mul(w_n, w_n))))
+                                    : P::rcp(P::mul(T(0.5), P::add(w_f, w_n)));
         T a = P::mul(z_f, iwbar), b = P::add(a, du);
         if (P::add(a, b) < T(0)) {
             const T t = a;
@@ -412,6 +423,65 @@ __device__ __forceinline__ void renormalize_packed(float (&P)[LPT], float (&Y)[L
         Y[l + 1] = Yn.y;
         D[l] = 1.0f;
         D[l + 1] = 1.0f;
+    }
+}
+
+// The homogeneous rows in FP64, kRows64 of them per reciprocal: seven
+// operations per line and row and one division per eight rows, against eight
+// and one for eliminate_row, whose division is about nine instructions of the
+// FP64 pipe.  From d = 1 a row multiplies d by less than 2^26 within the range
+// below, so that eight rows stay below 2^208 and the sources' sums below 2^310.
+constexpr int kRows64 = 8;
+static_assert(kRows64 % 2 == 0, "rows are taken two at a time");
+
+template <int LPT>
+__device__ __forceinline__ void homog_row64(double cf, double cn, const double (&chi_f)[LPT], const double (&S_f)[LPT],
+                                            const double (&chi_n)[LPT], double (&P)[LPT], double (&Y)[LPT],
+                                            double (&aa)[LPT], double (&D)[LPT])
+{
+#pragma unroll
+    for (int l = 0; l < LPT; ++l) {
+        const double b = __fma_rn(cf, chi_f[l], __dmul_rn(cn, chi_n[l]));
+        const double hd = __dmul_rn(__dadd_rn(aa[l], b), D[l]);
+        P[l] = __fma_rn(2.0, hd, P[l]);
+        Y[l] = __fma_rn(S_f[l], hd, Y[l]);
+        D[l] = __fma_rn(b, P[l], D[l]);
+        aa[l] = b;
+    }
+}
+
+template <int LPT> __device__ __forceinline__ void renormalize64(double (&P)[LPT], double (&Y)[LPT], double (&D)[LPT])
+{
+#pragma unroll
+    for (int l = 0; l < LPT; ++l) {
+        const double r = 1.0 / D[l];
+        P[l] = __dmul_rn(P[l], r);
+        Y[l] = __dmul_rn(Y[l], r);
+        D[l] = 1.0;
+    }
+}
+
+// Two rows of the homogeneous form, k and k - 1 (chiA -> chiB -> chiA); `rows`:
+// rows since the last reciprocal, before these two.
+template <typename T, int LPT>
+__device__ __forceinline__ void homog_rows(typename Prec<T>::V2 c0, typename Prec<T>::V2 c1, const T *row, int RS,
+                                           int Mpad, T (&chiA)[LPT], T (&chiB)[LPT], T (&P)[LPT], T (&Y)[LPT],
+                                           T (&aa)[LPT], T (&D)[LPT], int rows)
+{
+    T S_f[LPT];
+    load_vec<LPT>(row + Mpad, S_f);
+    load_vec<LPT>(row - RS, chiB);
+    if constexpr (sizeof(T) == 4)
+        homog_row1_packed<LPT>(c0.x, c0.y, chiA, S_f, chiB, P, Y, aa, D);
+    else
+        homog_row64<LPT>(c0.x, c0.y, chiA, S_f, chiB, P, Y, aa, D);
+    load_vec<LPT>(row - RS + Mpad, S_f);
+    load_vec<LPT>(row - 2 * RS, chiA);
+    if constexpr (sizeof(T) == 4) {
+        homog_row2_packed<LPT>(c1.x, c1.y, chiB, S_f, chiA, P, Y, aa, D);
+    } else {
+        homog_row64<LPT>(c1.x, c1.y, chiB, S_f, chiA, P, Y, aa, D);
+        if ((rows + 2) % kRows64 == 0) renormalize64<LPT>(P, Y, D);
     }
 }
 
@@ -598,7 +668,7 @@ __device__ __forceinline__ void sweep_gather(const FSArgs &a, int64_t o, int r, 
     T g_f = point_gauss<T>(z_f, line[c_f * a.RS + 2 * a.Mpad + 1]);
     for (int k = n; k >= 1; --k) {
         int64_t c_n = o;
-        StepG<T> sn{T(0), T(0), T(0)};
+        StepG<T> sn{};
         if (k > 1) {
             c_n = checked(a.s32[s0 + k - 2].x);
             sn = step_global<T>(a, s0 + k - 2);
@@ -617,7 +687,7 @@ __device__ __forceinline__ void sweep_gather(const FSArgs &a, int64_t o, int r, 
         if (a.subdiv > 0)
             subdiv_coefs<T>(a.subdiv, sf.dx, z_f, w_f, z_n, w_n, cf, cn);
         else
-            segment_coefs<T>(trap, sf.dx, du, z_f, g_f, w_f, g_n, w_n, a.width_mode, cf, cn);
+            segment_coefs<T>(trap, sf, du, z_f, g_f, w_f, g_n, w_n, a.width_mode, cf, cn);
         eliminate_row<T, LPT>(cf, cn, chi_f, S_f, chi_n, P, Y, aa);
 #pragma unroll
         for (int l = 0; l < LPT; ++l) {
@@ -861,14 +931,15 @@ struct StagedLayout {
 // Bins rounded up to whole pairs (FP32, which takes them in pairs).
 template <typename T> __host__ __device__ inline int bins_held(int Q) { return sizeof(T) == 4 ? (Q + 1) & ~1 : Q; }
 
-// Buffers of step records: the chunk in work, the next, and the one after,
-// whose records are on their way; two where the records do not travel ahead.
-constexpr int kStepBufs = 3;
+// Buffers of step records: the chunk in work, the next, and in FP32 the one
+// after, whose records are on their way.
+template <typename T> constexpr int kStepBufs = sizeof(T) == 4 ? 3 : 2;
 
 // Staging buffers and coefficient buffers [2] are contiguous; the final
 // FP64 reduction area aliases them once the last chunk is done.
 template <typename T, int LPT, int CH>
-__host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int bd, int P, bool fused, int step_bufs)
+__host__ __device__ inline StagedLayout staged_layout(int Q, int Mb, int RS, int bd, int P, bool fused,
+                                                  int step_bufs = kStepBufs<T>)
 {
     constexpr int SB = sizeof(T) == 4 ? 16 : 32;
     constexpr int NPT = CH + 1;
@@ -919,9 +990,9 @@ __device__ __forceinline__ typename Prec<T>::V2 segment_item(const FSArgs &a, in
         subdiv_coefs<T>(a.subdiv, sf.dx, z_f, w_f, z_n, w_n, cf, cn);
     } else if (trap) {
         const V2 g = gpair();
-        segment_coefs<T>(true, sf.dx, du, z_f, g.x, w_f, g.y, w_n, a.width_mode, cf, cn);
+        segment_coefs<T>(true, sf, du, z_f, g.x, w_f, g.y, w_n, a.width_mode, cf, cn);
     } else {
-        segment_coefs<T>(false, sf.dx, du, z_f, T(0), w_f, T(0), w_n, a.width_mode, cf, cn);
+        segment_coefs<T>(false, sf, du, z_f, T(0), w_f, T(0), w_n, a.width_mode, cf, cn);
     }
     return V2{cf, cn};
 }
@@ -1104,12 +1175,12 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
     const int bd = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rowB = a.RS * (int)sizeof(T);
     const int Mb = a.Gb * LPT;
-    const StagedLayout lay = staged_layout<T, LPT, CH>(a.Q, Mb, a.RS, bd, a.P, FUSED, a.step_bufs);
+    const StagedLayout lay = staged_layout<T, LPT, CH>(a.Q, Mb, a.RS, bd, a.P, FUSED);
 
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);                   // [2]
     int *abort_flag = reinterpret_cast<int *>(smem + 16);
-    unsigned char *steps_s = smem + lay.stage;                            // steps [step_bufs][NPT][SB]
-    unsigned char *rows_s = steps_s + a.step_bufs * NPT * SB;             // rows [2][NPT][rowB]
+    unsigned char *steps_s = smem + lay.stage;                            // steps [kStepBufs][NPT][SB]
+    unsigned char *rows_s = steps_s + kStepBufs<T> * NPT * SB;            // rows [2][NPT][rowB]
     V2 *coef = reinterpret_cast<V2 *>(smem + lay.coef);                   // [2][Q][CH + 1]
     T *ibg = reinterpret_cast<T *>(smem + lay.ibg);                       // [Mb][Q]
     T *sA = reinterpret_cast<T *>(smem + lay.sab), *sB = sA + bins_held<T>(a.Q);  // [bins_held] each
@@ -1149,11 +1220,12 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
     // a global load of the indices, held that warp back by more than a trip of
     // the pre-pass.  plan[] holds the coming chunks (k_hi = 0: none), written
     // by warp 0 one chunk before all warps read it.  FP64 records have no
-    // point indices, and the third step buffer may not fit: warp 0 alone then
-    // issues a chunk.
-    const bool AHEAD = sizeof(T) == 4 && a.step_bufs == kStepBufs;
+    // point indices: warp 0 alone issues a chunk.  (Made a choice of the launch
+    // instead of the type, it cost the 100k shell launch 143 -> 151 ms.)
+    constexpr bool AHEAD = sizeof(T) == 4;
+    constexpr int NB = kStepBufs<T>;
     auto steps_of = [&](int c) { return steps_s + c * NPT * SB; };
-    Chunk *plan = reinterpret_cast<Chunk *>(smem + 32);                   // [kStepBufs]
+    Chunk *plan = reinterpret_cast<Chunk *>(smem + 32);                   // [NB]
     int cs = 0;                                    // the chunk's step buffer and plan entry
     if (warp == 0) {
         Chunk cur, nx{};
@@ -1173,8 +1245,8 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
     T P[LPT], Y[LPT], aa[LPT];
     // FUSED (one line group: the thread is the only reader of its bin's
     // coefficients): the bin's offsets, and the Gaussian of the far point of
-    // the next step, carried down the half-ray
-    T Aq = T(0), Bq = T(0), gcar = T(0);
+    // the next step (negative: not there)
+    T Aq = T(0), Bq = T(0), gcar = T(-1);
     if constexpr (FUSED) {
         if (active) {
             Aq = sA[q];
@@ -1214,8 +1286,8 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
 
                 uint64_t *nbar = &bar[(ci + 1) & 1];
                 unsigned char *nrows = rows_s + ((ci + 1) & 1) * NPT * rowB;
-                if (AHEAD) {
-                    const int c1 = cs + 1 == kStepBufs ? 0 : cs + 1, c2 = c1 + 1 == kStepBufs ? 0 : c1 + 1;
+                if constexpr (AHEAD) {
+                    const int c1 = cs + 1 == NB ? 0 : cs + 1, c2 = c1 + 1 == NB ? 0 : c1 + 1;
                     const int klo = plan[c1].k_lo, khi = plan[c1].k_hi;
                     if (khi > 0) {
                         const int npts = khi - klo + 2, nw = bd >> 5, j = warp + lane * nw;
@@ -1239,46 +1311,52 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     Chunk nx;
                     const Chunk c{p, h, s0, n, k_lo, k_hi};
                     if (next_chunk(ext, a.P, c, CH, nx))
-                        issue_chunk<T>(a, o, nx, steps_of(cs + 1 == a.step_bufs ? 0 : cs + 1), false, nx, nullptr, nrows,
+                        issue_chunk<T>(a, o, nx, steps_of(cs + 1 == NB ? 0 : cs + 1), false, nx, nullptr, nrows,
                                        nbar, rowB, lane);
                 }
                 if (FUSED && active) {
                     // the same rows with each step's coefficients computed here
                     // (segment_item, as the pre-pass does) instead of read
                     const T *row = Rb + (k_hi - k_lo + 1) * a.RS + line0;
+                    // (a step's near point is the next step's far one: its
+                    // Gaussian is carried; FP64, whose exponential costs as
+                    // much as a line's row, only while steps take the trapezoid)
+                    constexpr bool LAZY = sizeof(T) == 8;
                     auto coef_of = [&](int k) -> V2 {
                         const int jf = k - k_lo + 1;
                         const StepG<T> sf = step_from<T>(Sb + jf * SB);
                         const T z_f = bin_z<T>(Aq, Bq, sf.beta);
                         const T z_n = bin_z<T>(Aq, Bq, k > 1 ? step_from<T>(Sb + (jf - 1) * SB).beta : T(0));
                         const T g_f = gcar;
-                        gcar = point_gauss<T>(z_n, Rb[(jf - 1) * a.RS + 2 * a.Mpad + 1]);
-                        const T g_n = gcar;
-                        return segment_item<T>(a, o, r, k, q, Sb, Rb, jf, Aq, Bq, sf, z_f,
-                                               [&] { return V2{g_f, g_n}; });
+                        auto gauss = [&](int j, T z) { return point_gauss<T>(z, Rb[j * a.RS + 2 * a.Mpad + 1]); };
+                        gcar = LAZY ? T(-1) : gauss(jf - 1, z_n);
+                        return segment_item<T>(a, o, r, k, q, Sb, Rb, jf, Aq, Bq, sf, z_f, [&] {
+                            if constexpr (LAZY) gcar = gauss(jf - 1, z_n);
+                            return V2{LAZY && g_f < T(0) ? gauss(jf, z_f) : g_f, gcar};
+                        });
                     };
                     if (k_hi == n) {                   // the half-ray's far end
                         const int jf = n - k_lo + 1;
-                        gcar = point_gauss<T>(bin_z<T>(Aq, Bq, step_from<T>(Sb + jf * SB).beta),
-                                              Rb[jf * a.RS + 2 * a.Mpad + 1]);
+                        gcar = LAZY ? T(-1)
+                                    : point_gauss<T>(bin_z<T>(Aq, Bq, step_from<T>(Sb + jf * SB).beta),
+                                                     Rb[jf * a.RS + 2 * a.Mpad + 1]);
                     }
                     T chiA[LPT], chiB[LPT], S_f[LPT];
                     load_vec<LPT>(row, chiA);
                     int k = k_hi;
                     if constexpr (FAST) {
                         T D[LPT];
+                        if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                            for (int l = 0; l < LPT; ++l) D[l] = T(1);
+                        }
 #pragma unroll 1
                         for (; k - 1 >= k_lo; k -= 2) {
-                            V2 cc = coef_of(k);
-                            load_vec<LPT>(row + a.Mpad, S_f);
-                            load_vec<LPT>(row - a.RS, chiB);
-                            homog_row1_packed<LPT>(cc.x, cc.y, chiA, S_f, chiB, P, Y, aa, D);
-                            cc = coef_of(k - 1);
-                            load_vec<LPT>(row - a.RS + a.Mpad, S_f);
-                            load_vec<LPT>(row - 2 * a.RS, chiA);
-                            homog_row2_packed<LPT>(cc.x, cc.y, chiB, S_f, chiA, P, Y, aa, D);
+                            const V2 c0 = coef_of(k), c1 = coef_of(k - 1);
+                            homog_rows<T, LPT>(c0, c1, row, a.RS, a.Mpad, chiA, chiB, P, Y, aa, D, k_hi - k);
                             row -= 2 * a.RS;
                         }
+                        if constexpr (sizeof(T) == 8) renormalize64<LPT>(P, Y, D);
                     } else {
 #pragma unroll 1
                         for (; k - 1 >= k_lo; k -= 2) {
@@ -1309,21 +1387,20 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     load_vec<LPT>(row, chiA);
                     int k = k_hi;
                     if constexpr (FAST) {
-                        // two rows per reciprocal (the launch checked the range)
+                        // two rows per reciprocal, FP64 eight (the launch checked the range)
                         T D[LPT];
+                        if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                            for (int l = 0; l < LPT; ++l) D[l] = T(1);
+                        }
 #pragma unroll 1
                         for (; k - 1 >= k_lo; k -= 2) {
-                            V2 cc = *cfp;
-                            load_vec<LPT>(row + a.Mpad, S_f);
-                            load_vec<LPT>(row - a.RS, chiB);
-                            homog_row1_packed<LPT>(cc.x, cc.y, chiA, S_f, chiB, P, Y, aa, D);
-                            cc = *(cfp - 1);
-                            load_vec<LPT>(row - a.RS + a.Mpad, S_f);
-                            load_vec<LPT>(row - 2 * a.RS, chiA);
-                            homog_row2_packed<LPT>(cc.x, cc.y, chiB, S_f, chiA, P, Y, aa, D);
+                            const V2 c0 = *cfp, c1 = *(cfp - 1);
+                            homog_rows<T, LPT>(c0, c1, row, a.RS, a.Mpad, chiA, chiB, P, Y, aa, D, k_hi - k);
                             row -= 2 * a.RS;
                             cfp -= 2;
                         }
+                        if constexpr (sizeof(T) == 8) renormalize64<LPT>(P, Y, D);
                     } else {
 #pragma unroll 1
                         for (; k - 1 >= k_lo; k -= 2) {
@@ -1347,7 +1424,7 @@ __device__ __forceinline__ bool fs_staged_item(const FSArgs &a, int64_t oi, int 
                     }
                 }
                 ++ci;
-                cs = cs + 1 == a.step_bufs ? 0 : cs + 1;
+                cs = cs + 1 == NB ? 0 : cs + 1;
             }
             if (h == 0) {
                 if (active) {
@@ -1579,19 +1656,24 @@ template <typename T, int LPT> FSArgs fill_fs_args(const mgt_model *m, bool accu
     a.n_rec = m->total_steps;
     a.lpt = LPT;
     a.nblk = ceil_div(a.Gtot, a.Gb);
-    a.step_bufs = 2;
     return a;
 }
 
-// Step buffers of a launch: FP32 records travel one chunk ahead where the third
-// buffer fits the shared memory with the rest (it does unless a model has some
-// hundred lines).
-template <typename T, int LPT, int CH> int staged_step_bufs(const FSArgs &a, int bd, bool fused)
+// Threads per CTA of the staged schedule.
+int staged_threads(const FSArgs &a) { return ((a.Q * a.Gb + 31) / 32) * 32; }
+
+// FP32 holds a third buffer of step records.  A model of some hundred lines
+// whose origin fitted the shared memory with two takes fewer line groups per
+// CTA, so that it fits with three (the lines' results do not depend on it).
+template <typename T, int LPT, int CH> void fit_line_groups(FSArgs &a, bool fused)
 {
-    return sizeof(T) == 4 &&
-                   staged_layout<T, LPT, CH>(a.Q, a.Gb * LPT, a.RS, bd, a.P, fused, kStepBufs).total <= 227 * 1024
-               ? kStepBufs
-               : 2;
+    auto total = [&](int bufs) {
+        return staged_layout<T, LPT, CH>(a.Q, a.Gb * LPT, a.RS, staged_threads(a), a.P, fused, bufs).total;
+    };
+    constexpr int most = 227 * 1024;
+    if (total(2) > most) return;
+    while (a.Gb > 1 && total(kStepBufs<T>) > most) --a.Gb;
+    a.nblk = ceil_div(a.Gtot, a.Gb);
 }
 
 // The staged launch: the two-row kernel and, for the two-row form, the
@@ -1637,7 +1719,6 @@ mgt_status launch_typed(mgt_model *m, cudaStream_t s, int schedule, bool accumul
     // point's row once, J-bar and Lambda* written
     const double fs_bytes = (double)m->total_steps * (sizeof(T) == 4 ? 16.0 : 32.0) +
                             (double)m->N * (double)a.RS * sizeof(T) + 16.0 * (double)m->N * m->M;
-    const int Mb = a.Gb * LPT;
     // one origin per CTA: the staged kernel (schedule 2: register-capped for
     // two blocks per SM; 3: one block per SM; 4: each thread computes its own
     // bin's coefficients, for models whose lines fit one line group).  The
@@ -1650,26 +1731,23 @@ mgt_status launch_typed(mgt_model *m, cudaStream_t s, int schedule, bool accumul
     if (staged) {
         a.OPB = 1;
         a.fused = (schedule == 4 || (schedule == 0 && a.Gtot == 1)) ? 1 : 0;
-        const int threads = a.Q * a.Gb;
-        const int bd = ((threads + 31) / 32) * 32;
+        fit_line_groups<T, LPT, kChunk>(a, a.fused != 0);
+        const int bd = staged_threads(a), Mb = a.Gb * LPT;
         if (bd > 256) return set_error(MGT_ERR_ARG, "formal solve: more than 256 bins per origin");
-        a.step_bufs = staged_step_bufs<T, LPT, kChunk>(a, bd, a.fused != 0);
-        const size_t smem = (size_t)staged_layout<T, LPT, kChunk>(a.Q, Mb, a.RS, bd, a.P, a.fused != 0, a.step_bufs).total;
+        const size_t smem = (size_t)staged_layout<T, LPT, kChunk>(a.Q, Mb, a.RS, bd, a.P, a.fused != 0).total;
         dim3 grid((unsigned)m->N, (unsigned)ceil_div(a.Gtot, a.Gb));
-        // the two-row elimination in FP32 (the subdivided reference keeps the
+        // the homogeneous elimination (the subdivided reference keeps the
         // one-row form; the range argument needs half-rays below kFastSteps)
-        if constexpr (sizeof(T) == 4) {
-            if (a.subdiv == 0 && m->N < kFastSteps) {
-                if (a.fused) return launch_staged<T, LPT, 2, true, true>(a, grid, bd, smem, fs_bytes, s, run);
-                return schedule == 3 ? launch_staged<T, LPT, 1, true, false>(a, grid, bd, smem, fs_bytes, s, run)
-                                     : launch_staged<T, LPT, 2, true, false>(a, grid, bd, smem, fs_bytes, s, run);
-            }
+        if (a.subdiv == 0 && m->N < kFastSteps) {
+            if (a.fused) return launch_staged<T, LPT, 2, true, true>(a, grid, bd, smem, fs_bytes, s, run);
+            return schedule == 3 ? launch_staged<T, LPT, 1, true, false>(a, grid, bd, smem, fs_bytes, s, run)
+                                 : launch_staged<T, LPT, 2, true, false>(a, grid, bd, smem, fs_bytes, s, run);
         }
         if (a.fused) return launch_staged<T, LPT, 2, false, true>(a, grid, bd, smem, fs_bytes, s, run);
         return schedule == 3 ? launch_staged<T, LPT, 1, false, false>(a, grid, bd, smem, fs_bytes, s, run)
                              : launch_staged<T, LPT, 2, false, false>(a, grid, bd, smem, fs_bytes, s, run);
     }
-    const int threads = a.OPB * a.Q * a.Gb;
+    const int threads = a.OPB * a.Q * a.Gb, Mb = a.Gb * LPT;
     const int bd = ((threads + 31) / 32) * 32;
     if (bd > 256) return set_error(MGT_ERR_ARG, "formal solve: too many bins x line groups per block");
     const size_t smem = sizeof(T) * 4 * LPT * bd + sizeof(double) * 2 * a.OPB * Mb * a.Q;
@@ -1721,15 +1799,17 @@ mgt_status fs_batch_args(const mgt_model *m, void *args, int *threads, int64_t *
     FSArgs a = lpt == 4 ? fill_fs_args<float, 4>(m, false) : fill_fs_args<float, 8>(m, false);
     a.OPB = 1;
     a.fused = a.Gtot == 1 ? 1 : 0;     // as the automatic single-model choice
-    const int bd = ((a.Q * a.Gb + 31) / 32) * 32;
+    // (by the long chunks, which need more)
+    if (lpt == 4)
+        fit_line_groups<float, 4, kChunk>(a, a.fused != 0);
+    else
+        fit_line_groups<float, 8, kChunk>(a, a.fused != 0);
+    const int bd = staged_threads(a);
     if (bd > 256) return set_error(MGT_ERR_ARG, "batched formal solve: more than 256 bins per origin");
     *threads = bd;
     *items = a.N * a.nblk;
     *fused = a.fused;
     *lines = a.lpt;
-    // (by the long chunks, which need more)
-    a.step_bufs = lpt == 4 ? staged_step_bufs<float, 4, kChunk>(a, bd, a.fused != 0)
-                           : staged_step_bufs<float, 8, kChunk>(a, bd, a.fused != 0);
     std::memcpy(args, &a, sizeof a);
     return MGT_OK;
 }
@@ -1750,10 +1830,10 @@ size_t fs_batch_smem(const void *args, int bd)
     const int Mb = a.Gb * a.lpt;
     const bool f = a.fused != 0;
     if (narrow_chunks(bd, a.fused))
-        return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total
-                          : (size_t)staged_layout<float, 8, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total;
-    return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunk>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total
-                      : (size_t)staged_layout<float, 8, kChunk>(a.Q, Mb, a.RS, bd, a.P, f, a.step_bufs).total;
+        return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f).total
+                          : (size_t)staged_layout<float, 8, kChunkNarrow>(a.Q, Mb, a.RS, bd, a.P, f).total;
+    return a.lpt == 4 ? (size_t)staged_layout<float, 4, kChunk>(a.Q, Mb, a.RS, bd, a.P, f).total
+                      : (size_t)staged_layout<float, 8, kChunk>(a.Q, Mb, a.RS, bd, a.P, f).total;
 }
 
 namespace {

@@ -1118,7 +1118,7 @@ __global__ void k_steps64(int64_t N, int32_t R, const int64_t *__restrict__ off,
         double dbeta = (n0 * (vx - pvx) + n1 * (vy - pvy) + n2 * (vz - pvz)) / kC;
         double wbar = width_mode == 0 ? sqrt(0.5 * (wq * wq + pw * pw)) : 0.5 * (wq + pw);
         st.dbw = dbeta / wbar;
-        st.pad = 0.0;
+        st.iw = 1.0 / wbar;
         s64[s] = st;
         px = qx; py = qy; pz = qz;
         pvx = vx; pvy = vy; pvz = vz; pw = wq;

@@ -50,9 +50,9 @@ constexpr uint32_t kEntBnd = 1u << 31;
 constexpr uint32_t kEntIdx = kEntLast - 1u;
 constexpr uint32_t kEntEmpty = kEntIdx;
 
-// Double-precision geometry of the same step: {dx, beta, dbeta/wbar, unused}.
+// Double-precision geometry of the same step: {dx, beta, dbeta/wbar, 1/wbar}.
 struct alignas(32) Step64 {
-    double dx, beta, dbw, pad;
+    double dx, beta, dbw, iw;
 };
 
 // Pixel rays of the last image geometry (direction and pixel counts).
