@@ -68,13 +68,30 @@ struct Chan {
     double rf64;
 };
 
-__device__ Chan channel(const ImgArgs &a, int f)
+// The channel's constants, by a warp (lanes over the lines; the nearest line,
+// the lower index on ties).
+__device__ __forceinline__ Chan channel(const ImgArgs &a, int f, int lane)
 {
     Chan c;
     const double nu = a.fmin + f * a.fstep;
-    int l = 0;
-    for (int k = 1; k < a.M; ++k)
-        if (fabs(nu - a.line_tab[k]) < fabs(nu - a.line_tab[l])) l = k;
+    int l = lane < a.M ? lane : 0;
+    double best = fabs(nu - a.line_tab[l]);
+    for (int k = lane + 32; k < a.M; k += 32) {
+        const double d = fabs(nu - a.line_tab[k]);
+        if (d < best) {
+            best = d;
+            l = k;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double d = __shfl_xor_sync(0xffffffffu, best, o);
+        const int k = __shfl_xor_sync(0xffffffffu, l, o);
+        if (d < best || (d == best && k < l)) {
+            best = d;
+            l = k;
+        }
+    }
     c.l = l;
     const double r = nu / a.line_tab[l];
     c.rf64 = r;
@@ -187,10 +204,11 @@ __device__ __forceinline__ void weights(float t, float &E, float &w0, float &w1,
 
 // Stage ray points c0 .. c0+n-1 of pixel ray `base` (n <= kImgStage): the
 // velocity projection, width, 1/width and length of the segment ending at the
-// point, that segment's inverse mean width, and, with `theta`, the width's
-// temperature factor.  Every thread of the block calls it.
-__device__ __forceinline__ void stage_points(const ImgArgs &a, int64_t base, int64_t c0, int n, bool theta,
-                                             float4 *geo, float *siw, float *sth, int32_t *pid)
+// point, that segment's inverse mean width, with `theta` the width's
+// temperature factor, and with line >= 0 that line's scaled opacity and source
+// function.  Every thread of the block calls it.
+__device__ __forceinline__ void stage_points(const ImgArgs &a, int64_t base, int64_t c0, int n, bool theta, int line,
+                                             float4 *geo, float *siw, float *sth, float2 *scs, int32_t *pid)
 {
     __syncthreads();                 // the previous stage is consumed
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -211,20 +229,38 @@ __device__ __forceinline__ void stage_points(const ImgArgs &a, int64_t base, int
         siw[i] = iw;
         pid[i] = c;
         if (theta) sth[i] = a.theta_k * (float)a.temp[c];
+        if (line >= 0) scs[i] = make_float2(row[line], row[a.Mpad + line]);
     }
     __syncthreads();
 }
 
-// Staged point i with line l's scaled opacity and source function.
-__device__ __forceinline__ Pt staged_pt(const ImgArgs &a, const float4 *geo, const float *sth, const int32_t *pid,
-                                        int i, int l, bool theta)
+// The one line that channels f0 .. f1 - 1 all see, or -1: the channels nearest
+// to a line are an interval, so the first and the last tell.  Its opacities and
+// sources are then staged with the points; read by each thread from the point
+// rows, they put an L2 round trip into every segment.
+__device__ __forceinline__ int common_line(const ImgArgs &a, int f0, int f1)
+{
+    const int l = a.chan[f0].l;
+    return a.chan[min(f1, a.nfreq) - 1].l == l ? l : -1;
+}
+
+// Staged point i with line l's scaled opacity and source function (scs: staged
+// ones, or NULL).
+__device__ __forceinline__ Pt staged_pt(const ImgArgs &a, const float4 *geo, const float *sth, const float2 *scs,
+                                        const int32_t *pid, int i, int l, bool theta)
 {
     const float4 g = geo[i];
     Pt p;
     p.c = pid[i];
-    const float *row = a.line + p.c * a.RS;
-    p.chi = row[l];
-    p.S = row[a.Mpad + l];
+    if (scs) {
+        const float2 v = scs[i];
+        p.chi = v.x;
+        p.S = v.y;
+    } else {
+        const float *row = a.line + p.c * a.RS;
+        p.chi = row[l];
+        p.S = row[a.Mpad + l];
+    }
     p.w = g.y;
     p.winv = g.z;
     p.beta = g.x;
@@ -232,11 +268,14 @@ __device__ __forceinline__ Pt staged_pt(const ImgArgs &a, const float4 *geo, con
     return p;
 }
 
-// The channel constants depend only on the channel: computed once per call.
+// The channel constants depend only on the channel: computed once per call,
+// one warp per channel.
 __global__ void k_image_chan(ImgArgs a, Chan *__restrict__ out)
 {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f < a.nfreq) out[f] = channel(a, f);
+    const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (f >= a.nfreq) return;                     // whole warp
+    const Chan c = channel(a, f, lane);
+    if (lane == 0) out[f] = c;
 }
 
 // One block per pixel, threads over channels.  The ray's point geometry (the
@@ -248,6 +287,7 @@ __global__ void __launch_bounds__(256) k_image_fwd(ImgArgs a)
 {
     __shared__ float4 geo[kImgStage];
     __shared__ float siw[kImgStage];
+    __shared__ float2 scs[kImgStage];
     __shared__ int32_t pid[kImgStage];
     const int64_t q = blockIdx.x;
     const int64_t base = a.off[q];
@@ -257,14 +297,15 @@ __global__ void __launch_bounds__(256) k_image_fwd(ImgArgs a)
         const int f = f0 + threadIdx.x;
         const bool active = f < a.nfreq;
         const Chan ch = a.chan[active ? f : 0];
+        const int ul = common_line(a, f0, f0 + blockDim.x);
         float I = ch.I0;
         Pt A{};
         for (int64_t c0 = 0; c0 < np; c0 += kImgStage) {
             const int n = (int)min((int64_t)kImgStage, np - c0);
-            stage_points(a, base, c0, n, false, geo, siw, nullptr, pid);
+            stage_points(a, base, c0, n, false, ul, geo, siw, nullptr, scs, pid);
             if (!active) continue;
             for (int i = 0; i < n; ++i) {
-                const Pt B = staged_pt(a, geo, nullptr, pid, i, ch.l, false);
+                const Pt B = staged_pt(a, geo, nullptr, ul >= 0 ? scs : nullptr, pid, i, ch.l, false);
                 if (c0 + i > 0) {
                     const float t = seg_dtau<false>(a, ch, A, B, geo[i].w, siw[i], dd);
                     float E, w0, w1, gp;
@@ -275,6 +316,136 @@ __global__ void __launch_bounds__(256) k_image_fwd(ImgArgs a)
             }
         }
         if (active) a.out[(int64_t)f * a.npix + q] = I * ch.U;
+    }
+}
+
+// Optical depth of a segment for two channels on packed FP32 (one lane per
+// channel), the rule of seg_dtau: z the comoving offsets at the far and near
+// point, chi the opacities, both lanes on one branch.
+__device__ __forceinline__ float2 pair_dtau(bool trap, float2 za, float2 zb, float2 chi_a, float2 chi_b, float dx,
+                                            float iw, float wa, float wb, float rwa, float rwb)
+{
+    const auto s2 = [](float x) { return make_float2(x, x); };
+    if (trap) {
+        const float2 ua = __fmul2_rn(za, s2(rwa)), ub = __fmul2_rn(zb, s2(rwb));
+        const float2 ya = __fmul2_rn(__fmul2_rn(ua, ua), s2(-kLog2E)), yb = __fmul2_rn(__fmul2_rn(ub, ub), s2(-kLog2E));
+        const float2 ga = make_float2(ex2_mufu(ya.x), ex2_mufu(ya.y)), gb = make_float2(ex2_mufu(yb.x), ex2_mufu(yb.y));
+        return __fmul2_rn(s2(0.5f * dx), __ffma2_rn(chi_a, ga, __fmul2_rn(chi_b, gb)));
+    }
+    const float2 a = __fmul2_rn(za, s2(iw)), b = __fmul2_rn(zb, s2(iw));
+    const float2 sum = __fadd2_rn(a, b);
+    float2 lo = a, hi = b;
+    if (sum.x < 0.0f) {                              // reflect: same difference, no cancellation
+        lo.x = -b.x;
+        hi.x = -a.x;
+    }
+    if (sum.y < 0.0f) {
+        lo.y = -b.y;
+        hi.y = -a.y;
+    }
+    const float2 el = erfc_fit2(lo.x, lo.y), eh = erfc_fit2(hi.x, hi.y);
+    const float2 E = __fadd2_rn(el, make_float2(-eh.x, -eh.y));
+    const float2 D = __fadd2_rn(zb, make_float2(-za.x, -za.y));
+    const float2 iD = make_float2(rcp_mufu(D.x), rcp_mufu(D.y));
+    const float2 K = __fmul2_rn(s2(dx * (0.25f * kSqrtPiF)), __ffma2_rn(chi_a, s2(wa), __fmul2_rn(chi_b, s2(wb))));
+    return __fmul2_rn(__fmul2_rn(K, E), iD);
+}
+
+// I <- e^-t I + w0 S_a + w1 S_b for two channels (the weights of `weights`).
+__device__ __forceinline__ float2 pair_update(float2 t, float2 I, float2 Sa, float2 Sb)
+{
+    const auto s2 = [](float x) { return make_float2(x, x); };
+    const float2 y = __fmul2_rn(t, s2(-kLog2E));
+    const float2 E = make_float2(ex2_mufu(y.x), ex2_mufu(y.y)), nE = make_float2(-E.x, -E.y);
+    const float2 nt = make_float2(-t.x, -t.y);
+    // series for t < 0.05, else from (1 - E)/t
+    float2 w1 = __fmul2_rn(
+        t, __ffma2_rn(nt, __ffma2_rn(nt, __ffma2_rn(nt, s2(1.0f / 120.0f), s2(1.0f / 24.0f)), s2(1.0f / 6.0f)), s2(0.5f)));
+    float2 w0 = __ffma2_rn(nt, s2(1.0f / 144.0f), s2(1.0f / 30.0f));
+    w0 = __ffma2_rn(nt, w0, s2(1.0f / 8.0f));
+    w0 = __ffma2_rn(nt, w0, s2(1.0f / 3.0f));
+    w0 = __fmul2_rn(t, __ffma2_rn(nt, w0, s2(0.5f)));
+    const float2 g = __fmul2_rn(__fadd2_rn(s2(1.0f), nE), make_float2(rcp_mufu(t.x), rcp_mufu(t.y)));
+    const float2 v0 = __fadd2_rn(g, nE), v1 = __fadd2_rn(s2(1.0f), make_float2(-g.x, -g.y));
+    if (!(t.x < 0.05f)) {
+        w0.x = v0.x;
+        w1.x = v1.x;
+    }
+    if (!(t.y < 0.05f)) {
+        w0.y = v0.y;
+        w1.y = v1.y;
+    }
+    return __ffma2_rn(E, I, __ffma2_rn(w0, Sa, __fmul2_rn(w1, Sb)));
+}
+
+// k_image_fwd with two neighbouring channels per thread on packed FP32: the
+// kernel is bound by issue (114 instructions per segment and channel, 82 % of
+// the slots), and a packed instruction serves both channels.  For more than 32
+// channels; with fewer the pairs would leave lanes of the one warp idle.  256 x
+// 256 pixels x 100 channels on 100k points: 595 -> 504 us.
+__global__ void __launch_bounds__(256) k_image_fwd2(ImgArgs a)
+{
+    __shared__ float4 geo[kImgStage];
+    __shared__ float siw[kImgStage];
+    __shared__ float2 scs[kImgStage];
+    __shared__ int32_t pid[kImgStage];
+    const int64_t q = blockIdx.x;
+    const int64_t base = a.off[q];
+    const int64_t np = a.off[q + 1] - base;  // points on the ray (segments + 1)
+    const float thr = (float)a.thr, band = kImgBand * thr;
+    float dd[6];
+    for (int f0 = 0; f0 < a.nfreq; f0 += 2 * blockDim.x) {   // the same trip count for the whole block
+        const int f = f0 + 2 * threadIdx.x;
+        const bool active = f < a.nfreq, two = f + 1 < a.nfreq;
+        const Chan c0 = a.chan[active ? f : 0], c1 = a.chan[two ? f + 1 : active ? f : 0];
+        const float2 nrf = make_float2(-c0.rf, -c1.rf), rf1 = make_float2(c0.rf1, c1.rf1);
+        const int ul = common_line(a, f0, f0 + 2 * blockDim.x);
+        float2 I = make_float2(c0.I0, c1.I0);
+        float2 za{}, chi_a{}, S_a{};
+        float4 ga{};
+        int64_t ca = 0;
+        for (int64_t i0 = 0; i0 < np; i0 += kImgStage) {
+            const int n = (int)min((int64_t)kImgStage, np - i0);
+            stage_points(a, base, i0, n, false, ul, geo, siw, nullptr, scs, pid);
+            if (!active) continue;
+            for (int i = 0; i < n; ++i) {
+                const float4 g = geo[i];             // beta, w, 1/w, length of the segment ending here
+                const int64_t c = pid[i];
+                float2 chi, S;
+                if (ul >= 0) {
+                    const float2 v = scs[i];
+                    chi = make_float2(v.x, v.x);
+                    S = make_float2(v.y, v.y);
+                } else {
+                    const float *row = a.line + c * a.RS;
+                    chi = make_float2(row[c0.l], row[c1.l]);
+                    S = make_float2(row[a.Mpad + c0.l], row[a.Mpad + c1.l]);
+                }
+                const float2 z = __ffma2_rn(nrf, make_float2(g.x, g.x), rf1);
+                if (i0 + i > 0) {
+                    const float iw = siw[i];
+                    const float2 du = __fmul2_rn(__fadd2_rn(z, make_float2(-za.x, -za.y)), make_float2(iw, iw));
+                    const bool t0 = fabsf(du.x) < thr, t1 = fabsf(du.y) < thr;
+                    float2 t;
+                    if (t0 == t1 && !(fabsf(fabsf(du.x) - thr) < band) && !(fabsf(fabsf(du.y) - thr) < band)) {
+                        t = pair_dtau(t0, za, z, chi_a, chi, g.w, iw, ga.y, g.y, ga.z, g.z);
+                    } else {                         // near the switch: one channel after the other
+                        const Pt A0{ca, chi_a.x, S_a.x, ga.y, ga.z, ga.x, 0.0f}, B0{c, chi.x, S.x, g.y, g.z, g.x, 0.0f};
+                        const Pt A1{ca, chi_a.y, S_a.y, ga.y, ga.z, ga.x, 0.0f}, B1{c, chi.y, S.y, g.y, g.z, g.x, 0.0f};
+                        t.x = seg_dtau<false>(a, c0, A0, B0, g.w, iw, dd);
+                        t.y = seg_dtau<false>(a, c1, A1, B1, g.w, iw, dd);
+                    }
+                    I = pair_update(t, I, S_a, S);
+                }
+                za = z;
+                chi_a = chi;
+                S_a = S;
+                ga = g;
+                ca = c;
+            }
+        }
+        if (active) a.out[(int64_t)f * a.npix + q] = I.x * c0.U;
+        if (two) a.out[(int64_t)(f + 1) * a.npix + q] = I.y * c1.U;
     }
 }
 
@@ -309,6 +480,7 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
     __shared__ float4 geo[kImgStage];
     __shared__ float siw[kImgStage];
     __shared__ float sth[kImgStage];
+    __shared__ float2 scs[kImgStage];
     __shared__ int32_t pid[kImgStage];
     const int64_t q = blockIdx.x;
     const int64_t base = a.off[q];
@@ -324,6 +496,9 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
         const int f = f0 + threadIdx.x;
         const bool active = f < a.nfreq;
         const Chan ch = a.chan[active ? f : 0];
+        const int ul = common_line(a, f0, f0 + blockDim.x);
+        const float2 *cs = ul >= 0 ? scs : nullptr;
+        // (threads past the last channel run channel 0 with zero weight: its line or any other)
         // forward, keeping checkpoints
         float I = ch.I0;
         {
@@ -332,9 +507,9 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
             int ick = 0;
             for (int64_t c0 = 0; c0 <= D; c0 += kImgStage) {
                 const int n = (int)min((int64_t)kImgStage, D + 1 - c0);
-                stage_points(a, base, c0, n, false, geo, siw, sth, pid);
+                stage_points(a, base, c0, n, false, ul, geo, siw, sth, scs, pid);
                 for (int i = 0; i < n; ++i) {
-                    const Pt B = staged_pt(a, geo, sth, pid, i, ch.l, false);
+                    const Pt B = staged_pt(a, geo, sth, cs, pid, i, ch.l, false);
                     const int64_t d = c0 + i - 1;              // the segment ending at this point
                     if (d >= 0) {
                         if (d == next_ck) {
@@ -354,13 +529,13 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
         float pT = 0.0f, pn = 0.0f, pb = 0.0f;      // pending gradient of point P_{d+1}
         for (int64_t blk = nblk - 1; blk >= 0; --blk) {
             const int64_t d0 = blk * s, d1 = min(D, d0 + s);
-            stage_points(a, base, d0, (int)(d1 - d0 + 1), true, geo, siw, sth, pid);
+            stage_points(a, base, d0, (int)(d1 - d0 + 1), true, ul, geo, siw, sth, scs, pid);
             float Ir = ck[blk];
-            Pt A = staged_pt(a, geo, sth, pid, 0, ch.l, false);
+            Pt A = staged_pt(a, geo, sth, cs, pid, 0, ch.l, false);
             for (int64_t d = d0; d < d1; ++d) {
                 const int i = (int)(d - d0) + 1;
                 loc[i - 1] = Ir;
-                const Pt B = staged_pt(a, geo, sth, pid, i, ch.l, false);
+                const Pt B = staged_pt(a, geo, sth, cs, pid, i, ch.l, false);
                 const float t = seg_dtau<false>(a, ch, A, B, geo[i].w, siw[i], dd);
                 float E, w0, w1, gp;
                 weights(t, E, w0, w1, gp);
@@ -369,8 +544,8 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
             }
             for (int64_t d = d1 - 1; d >= d0; --d) {
                 const int i = (int)(d - d0);
-                const Pt Pa = staged_pt(a, geo, sth, pid, i, ch.l, true);
-                const Pt Pb = staged_pt(a, geo, sth, pid, i + 1, ch.l, true);
+                const Pt Pa = staged_pt(a, geo, sth, cs, pid, i, ch.l, true);
+                const Pt Pb = staged_pt(a, geo, sth, cs, pid, i + 1, ch.l, true);
                 const float t = seg_dtau<true>(a, ch, Pa, Pb, geo[i + 1].w, siw[i + 1], dd);
                 float E, w0, w1, gp;
                 weights(t, E, w0, w1, gp);
@@ -479,12 +654,23 @@ ImgArgs image_args(mgt_model *m, const double *dir, int32_t nfreq, double fmin, 
     return a;
 }
 
+// A temporary of one call, from the library's pool: the default pool gives its
+// memory back at the next synchronisation and maps it again for the next call
+// (240 us).
+template <typename T> mgt_status image_temp(T **p, int64_t n, cudaStream_t s)
+{
+    cudaMemPool_t pool = nullptr;
+    MGT_TRY_STATUS(scratch_pool(&pool));
+    MGT_CUDA(cudaMallocFromPoolAsync((void **)p, sizeof(T) * n, pool, s));
+    return MGT_OK;
+}
+
 // The per-channel constants of one call, stream-ordered; the caller frees a.chan.
 mgt_status image_channels(ImgArgs &a, cudaStream_t s)
 {
     Chan *c = nullptr;
-    MGT_CUDA(cudaMallocAsync(&c, sizeof(Chan) * a.nfreq, s));
-    k_image_chan<<<ceil_div(a.nfreq, 128), 128, 0, s>>>(a, c);
+    MGT_TRY_STATUS(image_temp(&c, a.nfreq, s));
+    k_image_chan<<<ceil_div(a.nfreq * (int64_t)32, 128), 128, 0, s>>>(a, c);
     MGT_LAUNCH_CHECK("k_image_chan");
     a.chan = c;
     return MGT_OK;
@@ -532,11 +718,15 @@ mgt_status mgt_image(mgt_model *m, const double dir[3], int32_t npx, int32_t npy
     ImgArgs a = image_args(m, dir, nfreq, fmin, fmax);
     const int64_t n = a.npix * nfreq;
     float *dev = out;
-    if (!on_device) MGT_CUDA(cudaMallocAsync(&dev, sizeof(float) * n, s));
+    if (!on_device) MGT_TRY_STATUS(image_temp(&dev, n, s));
     a.out = dev;
     MGT_TRY_STATUS(image_channels(a, s));
-    const int bd = nfreq >= 256 ? 256 : (nfreq + 31) / 32 * 32;
-    k_image_fwd<<<(unsigned)a.npix, bd, 0, s>>>(a);
+    if (nfreq > 32) {
+        const int pairs = (nfreq + 1) / 2, bd = pairs >= 256 ? 256 : (pairs + 31) / 32 * 32;
+        k_image_fwd2<<<(unsigned)a.npix, bd, 0, s>>>(a);
+    } else {
+        k_image_fwd<<<(unsigned)a.npix, 32, 0, s>>>(a);
+    }
     MGT_LAUNCH_CHECK("k_image_fwd");
     MGT_CUDA(cudaFreeAsync((void *)a.chan, s));
     if (!on_device) {
@@ -562,11 +752,11 @@ mgt_status mgt_image_adjoint(mgt_model *m, const double dir[3], int32_t npx, int
     const int64_t n = a.npix * nfreq, N = m->N;
     double *acc = nullptr, *gv = nullptr;
     float *gdev = nullptr;
-    MGT_CUDA(cudaMallocAsync(&acc, sizeof(double) * 3 * N, s));
-    MGT_CUDA(cudaMallocAsync(&gv, sizeof(double) * 3 * N, s));
+    MGT_TRY_STATUS(image_temp(&acc, 3 * N, s));
+    MGT_TRY_STATUS(image_temp(&gv, 3 * N, s));
     MGT_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * N, s));
     if (!on_device) {
-        MGT_CUDA(cudaMallocAsync(&gdev, sizeof(float) * n, s));
+        MGT_TRY_STATUS(image_temp(&gdev, n, s));
         MGT_CUDA(cudaMemcpyAsync(gdev, grad_out, sizeof(float) * n, cudaMemcpyHostToDevice, s));
     }
     a.gout = on_device ? grad_out : gdev;
@@ -611,7 +801,7 @@ mgt_status mgt_set_point_fields(mgt_model *m, const double *temp, const double *
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (n_spec) {
         double *ns = nullptr;
-        MGT_CUDA(cudaMallocAsync(&ns, sizeof(double) * N, s));
+        MGT_TRY_STATUS(image_temp(&ns, N, s));
         MGT_CUDA(cudaMemcpyAsync(ns, n_spec, sizeof(double) * N, kind, s));
         k_rescale_pops<<<ceil_div(N * m->L, kRescaleItems), kRescaleThreads, 0, s>>>(N, m->L, m->d_nspec, ns, m->d_pops, m->d_pops_prev);
         MGT_LAUNCH_CHECK("k_rescale_pops");

@@ -257,3 +257,18 @@ def test_pixel_rays_longer_than_their_slots(mgt):
     r = O.image_rays(m, d, 4, 3)
     assert np.max(np.diff(roff)) > 1000
     assert np.array_equal(anchor, r.anchor) and np.array_equal(roff, r.off) and np.array_equal(pts, r.pts)
+
+
+@pytest.mark.parametrize("nfreq", [32, 33, 63, 65, 514])
+def test_channel_counts_around_the_pairs(mgt, nfreq):
+    # one channel per thread up to 32 channels, two neighbours per thread above
+    # (an odd last one, more than one trip of 256 pairs), over a band of three
+    # lines, so that some pairs see different lines; tolerance of the images
+    m = synth.shell_model(3000, 4, 1, 5, grf_sigma=2e3, seed=8, name="grf")
+    nu = m.lines.freq_Hz
+    lo, hi = 0.9999 * nu[0], 1.0001 * nu[2]
+    h = mgt.mgt_model_create(m)
+    for a, b in ((lo, hi), _band(m, line=1)):
+        img = mgt.mgt_image(h, DIR, 5, 4, nfreq, a, b)
+        ref, _ = O.image(m, _pops(m), DIR, 5, 4, nfreq, a, b)
+        assert np.max(np.abs(img - ref) / np.abs(ref)) < 1e-4
