@@ -440,6 +440,8 @@ static mgt_status build_model(mgt_model *m, const mgt_model_desc *d, cudaStream_
         tab[4 * Mp + k] = nbgmax;
         tab[5 * Mp + k] = hk;
         tab[6 * Mp + k] = 2.0 * kH * nu * nu * nu / (kC * kC) * nbgmax;
+        const float bg32[2] = {hk > 0.0 ? (float)hk : -1.0f, (float)nbgmax};
+        std::memcpy(&tab[7 * Mp + k], bg32, sizeof(bg32));
         ul[k] = m->up[k];
         ul[Mp + k] = m->lo[k];
     }

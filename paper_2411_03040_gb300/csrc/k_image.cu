@@ -47,7 +47,7 @@ struct ImgArgs {
     const float *line;        // [N][RS] rows: chi~' of every line, S' of every line, w, 1/w
     const float *pos_hl, *vel_hl;
     const double *vel, *w64, *temp;
-    const double *line_tab;   // [8][Mpad]: nu, A, Bul, Blu, nbgmax, h nu/k T_bg, U_line, unused
+    const double *line_tab;   // [8][Mpad]: nu, A, Bul, Blu, nbgmax, h nu/k T_bg, U_line, FP32 copies
     const int64_t *off;
     const int32_t *pts;
     double fmin, fstep;       // nu_f = fmin + f fstep

@@ -137,7 +137,8 @@ struct mgt_model {
     int2 *d_pairs = nullptr;
     // device: per line / level tables
     double *d_xq = nullptr, *d_wq = nullptr;
-    double *d_line_tab = nullptr;              // [8][Mpad]: nu, A, Bul, Blu, nbgmax, hnu_kTbg, U, unused
+    double *d_line_tab = nullptr;              // [8][Mpad]: nu, A, Bul, Blu, nbgmax, hnu_kTbg, U, the two before as
+                                               // float {hnu_kTbg (-1 where not positive), nbgmax}
     int32_t *d_line_ul = nullptr;              // [2][Mpad]: up, lo (-1 for padding)
     double *d_level_tab = nullptr;             // [2][L]: energy, g
     double *d_coll_tab = nullptr;              // [K]: K_ul
