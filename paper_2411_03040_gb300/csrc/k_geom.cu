@@ -75,11 +75,12 @@ __global__ void k_nbr_pos(int64_t nnz, const int32_t *__restrict__ nb, const dou
 __device__ __forceinline__ void put_entry(float4 *ent, int64_t e, const float *phl, int64_t mpt, uint32_t word,
                                           int32_t noff)
 {
-    float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float nan = __int_as_float(0x7fffffff);  // empty: no comparison of the walk's filter holds
+    float v[6] = {nan, nan, nan, nan, nan, nan};
     if (mpt >= 0)
         for (int c = 0; c < 6; ++c) v[c] = phl[6 * mpt + c];
-    ent[2 * e] = make_float4(v[0], v[1], v[2], v[3]);
-    ent[2 * e + 1] = make_float4(v[4], v[5], __uint_as_float(word), __int_as_float(noff));
+    ent[2 * e] = make_float4(v[0], v[1], v[2], __uint_as_float(word));
+    ent[2 * e + 1] = make_float4(v[3], v[4], v[5], __int_as_float(noff));
 }
 
 // One thread per point (rows of ~15 entries).  A row is padded with empty
@@ -612,12 +613,21 @@ template <int G> __device__ __forceinline__ float group_min(float v)
 // the candidates: one dependent L2 round trip per load.
 //
 // The lanes evaluate the candidates with FP32 arithmetic and error bounds that
-// cover both the FP32 and the FP64 rounding (generous multiples of the
-// rounding analysis):
-//   offsets    |d32 - d64| <= ed = 2e-6 (|d32|_max + slack)
-//   projection |Z32 - Z64| <= eZ = 2e-6 |d32|_1 + 2 ed
-//   perpendicular components  ep = ed + eZ + 2e-7 (|p32|_max + |Z32|)
-//   squared distance |d2_32 - d2_64| <= 4 |p32| ep + 4 ep^2 + 1e-6 d2_32.
+// cover both the FP32 and the FP64 rounding.  With u = 2^-24 = 6e-8, S the sum
+// of the offset's three magnitudes, and s = pos_slack = 2^-46 for what hi + lo
+// leave out and the low parts' rounding:
+//   offsets    d = (h - h_o) + (l - l_o): |d32 - d64| <= 2u |d| + 2s per component
+//   projection |Z32 - Z64| <= 2u S + 2s sqrt(3)  (offsets) + u S (direction in FP32)
+//              + 3u S (three operations) + u S (adding the bound)
+//              <= eZ = 5e-7 S + 4s
+//   p = d - Z n: the error's length <= 2u S + 2s sqrt(3) + eZ + 2u S
+//              <= ep = 8e-7 S + 8s
+//   squared distance |d2_32 - d2_64| <= 2 |p32| ep + ep^2 + 3u d2, and u d2 for
+//              each of Lo, U = 2 d2 - Lo and their rounding
+//              <= e2 = ep (2.5 |p32| + ep) + 4e-7 d2
+// (2.5 for 2 covers the approximate square root).  Coarser bounds from the
+// largest components, ten times these, took a quarter more instructions per
+// candidate and sent ten times as many steps to FP64.
 // The current point's projection Z_c is carried as the winner's FP32 value
 // with its bound eZ_c.  A neighbour is a candidate when Z32 - eZ clears
 // Z_c + eZ_c, not one when Z32 + eZ stays at or below Z_c - eZ_c; anything in
@@ -739,7 +749,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
     float Zc = 0.0f, eZc = 0.0f;                // Z of o is exactly 0 (image walks: the anchor's Z)
     if (IMG) {
         Zc = (float)(img_Z0 * a.pos_scale);     // the filter works in scaled units (exact factor)
-        eZc = 1e-7f * fabsf(Zc) + 1e-30f;
+        eZc = 2e-7f * fabsf(Zc) + 1e-30f;
     }
     // where point index k goes (lane sl keeps the index of step k = sl mod G
     // until the group's G indices are written together)
@@ -766,6 +776,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
     // clock, a row scan by the number of chunks; running out records the site
     // and returns.  All live walks of the warp have taken `it` steps.
     const uint64_t t_start = walk_clock_ns();
+    const float slack4 = 4.0f * a.pos_slack, slack8 = 8.0f * a.pos_slack;
     int it = 0;
     for (; __any_sync(full, !done); ++it) {
         if ((it & 15) == 15 && __any_sync(full, walk_clock_ns() - t_start > 2000000000ull)) {
@@ -776,44 +787,37 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
         // each lane keeps the best of its own entries over the row's chunks
         // (smallest d2, the earlier chunk on ties) and the least lower bound
         // of its other candidates; the group decides once per step
-        float bd2 = 3.0e38f, bU = 0.0f, bLo = 3.0e38f, bZ = 0.0f, beZ = 0.0f, lo2 = 3.0e38f;
+        float bd2 = 3.0e38f, bLo = 3.0e38f, bZ = 0.0f, beZ = 0.0f, lo2 = 3.0e38f;
         uint32_t bword = 0u;
         int brow = 0;
         bool und = false;
         const float Zhi = Zc + eZc, Zlo = Zc - eZc;
         auto candidate = [&](const float4 &e0, const float4 &e1) {
-            const uint32_t word = __float_as_uint(e1.z);
-            if ((word & kEntIdx) == kEntEmpty) return;
-            const float dx = (e0.x - f.ohx) + (e0.w - f.olx);
-            const float dy = (e0.y - f.ohy) + (e1.x - f.oly);
-            const float dz = (e0.z - f.ohz) + (e1.y - f.olz);
-            const float adx = fabsf(dx), ady = fabsf(dy), adz = fabsf(dz);
-            const float ed = 2e-6f * (fmaxf(adx, fmaxf(ady, adz)) + a.pos_slack);
+            const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(e0.x, e0.y), make_float2(-f.ohx, -f.ohy)),
+                                          __fadd2_rn(make_float2(e1.x, e1.y), make_float2(-f.olx, -f.oly)));
+            const float dx = dxy.x, dy = dxy.y, dz = (e0.z - f.ohz) + (e1.z - f.olz);
+            const float S = fabsf(dx) + fabsf(dy) + fabsf(dz);
             const float Z = fmaf(dz, f.f2, fmaf(dy, f.f1, dx * f.f0));
-            const float eZ = 2e-6f * (adx + ady + adz) + 2.0f * ed;
+            const float eZ = fmaf(5e-7f, S, slack4);
             if (Z - eZ > Zhi) {
                 const float px = fmaf(-Z, f.f0, dx), py = fmaf(-Z, f.f1, dy), pz = fmaf(-Z, f.f2, dz);
                 const float d2 = fmaf(pz, pz, fmaf(py, py, px * px));
-                const float ep_ = ed + eZ + 2e-7f * (fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))) + fabsf(Z));
-                // |p32| from the approximate square root, raised by 2^-10
-                // (far above its error) so that the bound stays an upper one
+                const float ep = fmaf(8e-7f, S, slack8);
                 float rp;
                 asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(d2));
-                const float e2 = 4.0f * (rp * 1.0009765625f) * ep_ + 4.0f * ep_ * ep_ + 1e-6f * d2;
+                const float e2 = fmaf(ep, fmaf(2.5f, rp, ep), 4e-7f * d2);
                 const float Lo = d2 - e2;
-                if (d2 < bd2) {
-                    lo2 = fminf(lo2, bLo);
+                const bool best = d2 < bd2;
+                lo2 = fminf(lo2, best ? bLo : Lo);
+                if (best) {
                     bd2 = d2;
-                    bU = d2 + e2;
                     bLo = Lo;
                     bZ = Z;
                     beZ = eZ;
-                    bword = word;
+                    bword = __float_as_uint(e0.w);
                     brow = __float_as_int(e1.w);
-                } else {
-                    lo2 = fminf(lo2, Lo);
                 }
-            } else if (!(Z + eZ <= Zlo)) {
+            } else if (Z + eZ > Zlo) {
                 und = true;
             }
         };
@@ -825,7 +829,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
                 }
                 const Vec8 e = load32(a.ent + 2 * ((int64_t)kb * kWalkRow + sl));
                 // (the same in every lane of the group)
-                kb = (__float_as_uint(e.b.z) & kEntLast) ? -1 : kb + 1;
+                kb = (__float_as_uint(e.a.w) & kEntLast) ? -1 : kb + 1;
                 candidate(e.a, e.b);
             }
         } else {
@@ -840,7 +844,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
                 Vec8 e{};
                 if (in) e = load32(a.ent + 2 * ((int64_t)chunk * kWalkRow + sl % kWalkRow));
                 // chunks up to the group's first one with the last-chunk flag belong to the row
-                const unsigned last = __ballot_sync(full, in && (__float_as_uint(e.b.z) & kEntLast)) & gmask;
+                const unsigned last = __ballot_sync(full, in && (__float_as_uint(e.a.w) & kEntLast)) & gmask;
                 if (in && (last & ((1u << (lane & ~(kWalkRow - 1))) - 1u)) == 0u) candidate(e.a, e.b);
                 open = open && last == 0u;
             }
@@ -854,7 +858,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
         const bool have = dmin < 3.0e38f;
         const unsigned wins = __ballot_sync(full, have && bd2 == dmin) & gmask;
         const int src = wins ? __ffs(wins) - 1 : lane;
-        bU = __shfl_sync(full, bU, src);
+        const float bU = 2.0f * dmin - __shfl_sync(full, bLo, src);
         bZ = __shfl_sync(full, bZ, src);
         beZ = __shfl_sync(full, beZ, src);
         bword = __shfl_sync(full, bword, src);
@@ -911,7 +915,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkBlocks) k_walk(WalkArgs a, 
                     nx = -1;
                 }
                 Zc = (float)(Zn * a.pos_scale);      // the filter works in scaled units (exact factor)
-                eZc = 1e-7f * fabsf(Zc) + 1e-30f;
+                eZc = 2e-7f * fabsf(Zc) + 1e-30f;
                 if (nx >= 0) {
                     nx_bnd = a.bnd[nx] != 0;
                     c_row = a.ent_row[nx];

@@ -38,12 +38,12 @@ constexpr int kMaxNgHist = 16;
 using Step32 = int4;
 
 // Packed neighbour entry of the ray walk, 32 bytes (two float4):
-//   {hx, hy, hz, lx}, {ly, lz, word, row}
+//   {hx, hy, hz, word}, {lx, ly, lz, row}
 // h + l = the neighbour's position times pos_scale (float hi + lo); word holds
 // the neighbour's index (bits 0-29), a flag carried by every entry of its
 // row's last chunk (bit 30) and the neighbour's boundary flag (bit 31); row is
 // the first chunk of the neighbour's own row.  Rows are whole chunks of
-// kWalkRow entries, padded with entries of index kEntEmpty.
+// kWalkRow entries, padded with entries of index kEntEmpty and NaN positions.
 constexpr int kWalkRow = 4;
 constexpr uint32_t kEntLast = 1u << 30;
 constexpr uint32_t kEntBnd = 1u << 31;

@@ -47,6 +47,29 @@ def test_rows_around_chunk_edges(mgt, n, degrees):
     assert st["n_stalls"] == r.stalls and st["total_steps"] == r.off[-1]
 
 
+@pytest.mark.parametrize("jitter", [0.0, 1e-15, 1e-13, 1e-10, 1e-8, 1e-7, 1e-6, 1e-4])
+@pytest.mark.parametrize("side,shift", [(12, 0.0), (16, 0.0), (16, 40.0)])
+def test_near_ties_at_every_scale(mgt, side, shift, jitter):
+    # a lattice disturbed by less or more than the filter's error bounds: along
+    # the axes and the diagonals of the 12 directions candidates tie up to the
+    # jitter, in projection and in distance; with the shift the coordinates are
+    # large against the spacing; 12 a side runs 16 lanes per walk, 16 a side 4
+    rng = np.random.default_rng(7)
+    g = np.arange(side)
+    pos = np.stack(np.meshgrid(g, g, g, indexing="ij"), axis=-1).reshape(-1, 3).astype(float)
+    nbrs = []
+    for i, p in enumerate(pos):
+        d = np.abs(pos - p).max(axis=1)
+        nbrs.append(np.flatnonzero((d <= 1) & (np.arange(len(pos)) != i)))
+    edge = np.flatnonzero((pos.min(axis=1) == 0) | (pos.max(axis=1) == side - 1))
+    m = _model(pos + shift + jitter * rng.normal(size=pos.shape), nbrs, edge, rng)
+    h = mgt.mgt_model_create(m)
+    mgt.mgt_trace_rays(h)
+    off, idx = mgt.mgt_get_rays(h)
+    r = O.trace(m)
+    assert np.array_equal(off, r.off) and np.array_equal(idx, r.idx)
+
+
 @pytest.mark.parametrize("n", [300, 700])
 def test_walks_longer_than_the_first_guess(mgt, n):
     # a bent chain: half-rays up to n - 1 points, beyond the first trace's slot
