@@ -297,14 +297,16 @@ def issue_roof(sm_max_mhz):
 
 def walk_bytes(model, total_steps, walk_launches):
     """Compulsory DRAM bytes of the ray walks of one step: the packed neighbour
-    table once per walk launch (32 B per entry, one sentinel per row, 16 pads),
-    the 16-byte step records written and the half-ray lengths; and the bytes the
-    walks gather through L2 (the current point's packed row at every step)."""
+    table once per walk launch (32 B per entry, each row padded to whole chunks
+    of 4 entries), the 4-byte point index of every step and the half-ray lengths;
+    and the bytes the walks gather through L2 (the current point's packed row at
+    every step)."""
     N = model.n_points
-    entries = int(model.nbrs.shape[0]) + N + 16
+    degree = np.diff(np.asarray(model.nbr_offsets))
+    entries = int((np.maximum(degree + 3, 4) // 4 * 4).sum())
     R = int(model.dirs.shape[0])
-    compulsory = walk_launches * (32.0 * entries + 8.0 * R * N) + 16.0 * total_steps
-    gathered = total_steps * 32.0 * (entries / N) + 16.0 * total_steps
+    compulsory = walk_launches * (32.0 * entries + 8.0 * R * N) + 4.0 * total_steps
+    gathered = total_steps * 32.0 * (entries / N)
     return compulsory, gathered
 
 
@@ -453,7 +455,7 @@ def run_mine(args, model, cfg, emit=True, n_error_origins=None, min_warmup=3):
                                           "the timed steps (trace = walk + compaction)"}
     out["kernels"] = kernel_table(kt, args.steps, hbm, extra_bytes={"k_walk<fused>": wc})
     out["kernels_note"] = (f"hbm_frac against the measured {hbm:.0f} GB/s; algorithmic bytes = the least a launch "
-                           "must read and write (k_walk: the packed neighbour table once per launch, records and "
+                           "must read and write (k_walk: the packed neighbour table once per launch, indices and "
                            f"lengths written; its L2 gather of rows is {wg / 1e9:.1f} GB per step)")
     out["ray_steps_per_s"] = {"value": model.n_quad * (tst["total_steps"] + model.n_points * pairs) / (fs_ms * 1e-3),
                               "unit": "ray steps/s (formal solve)"}

@@ -664,8 +664,8 @@ struct ImgWalkArgs {
     double n[3];              // unit direction toward the observer
 };
 
-// What bounds it: instruction issue (about 75 warp instructions per step at
-// 100k shell points) and the L2 round trips of the rows.  Four lanes per walk
+// What bounds it: instruction issue (73 warp instructions per step, 75 % of the
+// slots, 20k shell points) and the L2 round trips of the rows.  Four lanes per walk
 // read a row (15.5 entries on average) in its own 128-byte lines with few lanes
 // past its end; the decision's shuffles and the loop serve eight walks at once;
 // and walks of neighbouring origins step together, so their rows coincide in
@@ -673,7 +673,8 @@ struct ImgWalkArgs {
 // with 16 lanes per walk, records made inside, 64 registers; 16.0 ms with 4
 // lanes and the records left to k_walk_compact; 14.9 ms at 48 registers (ten
 // blocks of 128 threads per SM; 16.0 at eight, 18.8 at six, 17.5 at fourteen);
-// 14.4 ms with 256-bit loads.  8 lanes per walk: 18.7 ms, 2 lanes: 16.2 ms.
+// 14.4 ms with 256-bit loads; 13.2 ms with the bounds above.  Before those, 8
+// lanes per walk took 18.7 ms, 2 lanes 16.2 ms.
 // Not kept: loading the next chunk ahead (16.8 ms, a quarter of the loads
 // wasted), and giving a finished group the warp's next walk (16.7 ms: the
 // walks of a warp no longer pass the same rows together).
