@@ -1595,7 +1595,10 @@ template <typename T, int CH, bool FUSED, int LPT> __global__ void __launch_boun
         const int model = s_model;
         if (model < 0) return;
         cur = model;
-        if (!two_row_ok(sa)) continue;            // the model's items are k_fs_batch_exact's
+        if (!two_row_ok(sa)) {                    // the model's items are k_fs_batch_exact's
+            __syncthreads();                      // every warp has read s_model and sa: thread 0 may write them
+            continue;
+        }
         const int64_t local = s_item - s_first;
         const int64_t oi = local / sa.nblk;
         const int blk = (int)(local - oi * sa.nblk);

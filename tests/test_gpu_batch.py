@@ -189,6 +189,35 @@ def test_extreme_bin_counts_in_one_batch(mgt):
     assert np.max(np.abs(singles[0][1].T - L) / np.abs(L)) < TOL32
 
 
+# (levels, bins) of CTAs of 2, 3, 5 and 8 warps
+@pytest.mark.parametrize("levels,bins", [(11, 31), (21, 31), (41, 31), (41, 64)])
+def test_models_outside_the_two_row_range_among_others(mgt, levels, bins):
+    # the persistent kernel skips the items of models outside the two-row range
+    # (inner points 1e12 times denser, as in the parity tests) on its way to the
+    # next model's: one class of such models and normal ones, taken in turn and
+    # with a skipped model last, gives the single-model values bit for bit.
+    # Decreasing sizes: the items run in the order of the list.
+    models = []
+    for i in range(7):
+        m = synth.sphere_model(700 - 60 * i, levels, 1, bins, seed=600 + i, name=f"r{i}")
+        if i % 2 == 0:
+            r = np.linalg.norm(m.pos, axis=1)
+            m.n_spec = np.where(r < 0.5 * r.max(), m.n_spec * 1e12, m.n_spec)
+        models.append(m)
+    hs = [_handle(mgt, m, 8) for m in models]
+    singles = [mgt.mgt_formal_solve(h, mgt.MGT_FP32_MIXED) for h in hs]
+    b = mgt.mgt_batch_create(hs)
+    assert mgt.mgt_batch_get_layout(b)["fs_launches"] == 1
+    for _ in range(3):
+        mgt.mgt_batch_formal_solve(b)
+        for h, (J, L) in zip(hs, singles):
+            Jb, Lb = mgt.mgt_get_jbar(h)
+            np.testing.assert_array_equal(Jb, J)
+            np.testing.assert_array_equal(Lb, L)
+    for h in hs:
+        mgt.mgt_sync(h)
+
+
 def test_batch_follows_model_changes(mgt, batch_models):
     hs = [_handle(mgt, m, s[4]) for m, s in zip(batch_models[:3], SPECS[:3])]
     b = mgt.mgt_batch_create(hs)
