@@ -69,7 +69,7 @@ struct Chan {
 };
 
 // The channel's constants, by a warp (lanes over the lines; the nearest line,
-// the lower index on ties).
+// the lower index on ties).  Complete in lane 0.
 __device__ __forceinline__ Chan channel(const ImgArgs &a, int f, int lane)
 {
     Chan c;
@@ -85,6 +85,7 @@ __device__ __forceinline__ Chan channel(const ImgArgs &a, int f, int lane)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
+        if (o >= a.M) continue;                   // (lanes past the lines hold line 0)
         const double d = __shfl_xor_sync(0xffffffffu, best, o);
         const int k = __shfl_xor_sync(0xffffffffu, l, o);
         if (d < best || (d == best && k < l)) {
@@ -244,23 +245,16 @@ __device__ __forceinline__ int common_line(const ImgArgs &a, int f0, int f1)
     return a.chan[min(f1, a.nfreq) - 1].l == l ? l : -1;
 }
 
-// Staged point i with line l's scaled opacity and source function (scs: staged
-// ones, or NULL).
-__device__ __forceinline__ Pt staged_pt(const ImgArgs &a, const float4 *geo, const float *sth, const float2 *scs,
-                                        const int32_t *pid, int i, int l, bool theta)
+// Staged point i with line l's scaled opacity and source function.
+__device__ __forceinline__ Pt staged_pt(const ImgArgs &a, const float4 *geo, const float *sth, const int32_t *pid,
+                                        int i, int l, bool theta)
 {
     const float4 g = geo[i];
     Pt p;
     p.c = pid[i];
-    if (scs) {
-        const float2 v = scs[i];
-        p.chi = v.x;
-        p.S = v.y;
-    } else {
-        const float *row = a.line + p.c * a.RS;
-        p.chi = row[l];
-        p.S = row[a.Mpad + l];
-    }
+    const float *row = a.line + p.c * a.RS;
+    p.chi = row[l];
+    p.S = row[a.Mpad + l];
     p.w = g.y;
     p.winv = g.z;
     p.beta = g.x;
@@ -269,13 +263,13 @@ __device__ __forceinline__ Pt staged_pt(const ImgArgs &a, const float4 *geo, con
 }
 
 // The channel constants depend only on the channel: computed once per call,
-// one warp per channel.
-__global__ void k_image_chan(ImgArgs a, Chan *__restrict__ out)
+// one warp, a block of its own, per channel (the FP64 pipe takes 16 cycles per
+// warp instruction: the SMs share them).
+__global__ void __launch_bounds__(32) k_image_chan(ImgArgs a, Chan *__restrict__ out)
 {
-    const int f = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (f >= a.nfreq) return;                     // whole warp
-    const Chan c = channel(a, f, lane);
-    if (lane == 0) out[f] = c;
+    const int f = blockIdx.x;
+    const Chan c = channel(a, f, threadIdx.x);
+    if (threadIdx.x == 0) out[f] = c;
 }
 
 // One block per pixel, threads over channels.  The ray's point geometry (the
@@ -287,7 +281,6 @@ __global__ void __launch_bounds__(256) k_image_fwd(ImgArgs a)
 {
     __shared__ float4 geo[kImgStage];
     __shared__ float siw[kImgStage];
-    __shared__ float2 scs[kImgStage];
     __shared__ int32_t pid[kImgStage];
     const int64_t q = blockIdx.x;
     const int64_t base = a.off[q];
@@ -297,15 +290,14 @@ __global__ void __launch_bounds__(256) k_image_fwd(ImgArgs a)
         const int f = f0 + threadIdx.x;
         const bool active = f < a.nfreq;
         const Chan ch = a.chan[active ? f : 0];
-        const int ul = common_line(a, f0, f0 + blockDim.x);
         float I = ch.I0;
         Pt A{};
         for (int64_t c0 = 0; c0 < np; c0 += kImgStage) {
             const int n = (int)min((int64_t)kImgStage, np - c0);
-            stage_points(a, base, c0, n, false, ul, geo, siw, nullptr, scs, pid);
+            stage_points(a, base, c0, n, false, -1, geo, siw, nullptr, nullptr, pid);
             if (!active) continue;
             for (int i = 0; i < n; ++i) {
-                const Pt B = staged_pt(a, geo, nullptr, ul >= 0 ? scs : nullptr, pid, i, ch.l, false);
+                const Pt B = staged_pt(a, geo, nullptr, pid, i, ch.l, false);
                 if (c0 + i > 0) {
                     const float t = seg_dtau<false>(a, ch, A, B, geo[i].w, siw[i], dd);
                     float E, w0, w1, gp;
@@ -378,11 +370,11 @@ __device__ __forceinline__ float2 pair_update(float2 t, float2 I, float2 Sa, flo
     return __ffma2_rn(E, I, __ffma2_rn(w0, Sa, __fmul2_rn(w1, Sb)));
 }
 
-// k_image_fwd with two neighbouring channels per thread on packed FP32: the
+// k_image_fwd with two neighbouring channels per thread on packed FP32: that
 // kernel is bound by issue (114 instructions per segment and channel, 82 % of
-// the slots), and a packed instruction serves both channels.  For more than 32
-// channels; with fewer the pairs would leave lanes of the one warp idle.  256 x
-// 256 pixels x 100 channels on 100k points: 595 -> 504 us.
+// the slots at 100 channels), and a packed instruction serves both channels.
+// 256 x 256 pixels x 100 channels on 100k points: 595 us with one channel per
+// thread, 504 with two.
 __global__ void __launch_bounds__(256) k_image_fwd2(ImgArgs a)
 {
     __shared__ float4 geo[kImgStage];
@@ -449,6 +441,13 @@ __global__ void __launch_bounds__(256) k_image_fwd2(ImgArgs a)
     }
 }
 
+// Two channels per thread (w2 warps per ray) instead of one (w1 warps): a warp
+// of pairs takes about 1.7 times a warp of single channels, so the pairs need
+// fewer warps by more than that.  190 x 190 pixels, one and two per thread:
+// 34 channels (2 warps, 1) 178 and 149 us; 70 and 95 (3, 2) 337 and 350, 212 and
+// 228; 130 (5, 3) 344 and 346.
+inline bool paired_channels(int w1, int w2) { return 10 * w1 > 17 * w2; }
+
 __device__ __forceinline__ float warp_sum_f(float v)
 {
 #pragma unroll
@@ -507,7 +506,7 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
                 const int n = (int)min((int64_t)kImgStage, D + 1 - c0);
                 stage_points(a, base, c0, n, false, -1, geo, siw, sth, nullptr, pid);
                 for (int i = 0; i < n; ++i) {
-                    const Pt B = staged_pt(a, geo, sth, nullptr, pid, i, ch.l, false);
+                    const Pt B = staged_pt(a, geo, sth, pid, i, ch.l, false);
                     const int64_t d = c0 + i - 1;              // the segment ending at this point
                     if (d >= 0) {
                         if (d == next_ck) {
@@ -529,11 +528,11 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
             const int64_t d0 = blk * s, d1 = min(D, d0 + s);
             stage_points(a, base, d0, (int)(d1 - d0 + 1), true, -1, geo, siw, sth, nullptr, pid);
             float Ir = ck[blk];
-            Pt A = staged_pt(a, geo, sth, nullptr, pid, 0, ch.l, false);
+            Pt A = staged_pt(a, geo, sth, pid, 0, ch.l, false);
             for (int64_t d = d0; d < d1; ++d) {
                 const int i = (int)(d - d0) + 1;
                 loc[i - 1] = Ir;
-                const Pt B = staged_pt(a, geo, sth, nullptr, pid, i, ch.l, false);
+                const Pt B = staged_pt(a, geo, sth, pid, i, ch.l, false);
                 const float t = seg_dtau<false>(a, ch, A, B, geo[i].w, siw[i], dd);
                 float E, w0, w1, gp;
                 weights(t, E, w0, w1, gp);
@@ -542,8 +541,8 @@ __global__ void __launch_bounds__(128) k_image_adj(ImgArgs a)
             }
             for (int64_t d = d1 - 1; d >= d0; --d) {
                 const int i = (int)(d - d0);
-                const Pt Pa = staged_pt(a, geo, sth, nullptr, pid, i, ch.l, true);
-                const Pt Pb = staged_pt(a, geo, sth, nullptr, pid, i + 1, ch.l, true);
+                const Pt Pa = staged_pt(a, geo, sth, pid, i, ch.l, true);
+                const Pt Pb = staged_pt(a, geo, sth, pid, i + 1, ch.l, true);
                 const float t = seg_dtau<true>(a, ch, Pa, Pb, geo[i + 1].w, siw[i + 1], dd);
                 float E, w0, w1, gp;
                 weights(t, E, w0, w1, gp);
@@ -668,7 +667,7 @@ mgt_status image_channels(ImgArgs &a, cudaStream_t s)
 {
     Chan *c = nullptr;
     MGT_TRY_STATUS(image_temp(&c, a.nfreq, s));
-    k_image_chan<<<ceil_div(a.nfreq * (int64_t)32, 128), 128, 0, s>>>(a, c);
+    k_image_chan<<<a.nfreq, 32, 0, s>>>(a, c);
     MGT_LAUNCH_CHECK("k_image_chan");
     a.chan = c;
     return MGT_OK;
@@ -719,12 +718,11 @@ mgt_status mgt_image(mgt_model *m, const double dir[3], int32_t npx, int32_t npy
     if (!on_device) MGT_TRY_STATUS(image_temp(&dev, n, s));
     a.out = dev;
     MGT_TRY_STATUS(image_channels(a, s));
-    if (nfreq > 32) {
-        const int pairs = (nfreq + 1) / 2, bd = pairs >= 256 ? 256 : (pairs + 31) / 32 * 32;
-        k_image_fwd2<<<(unsigned)a.npix, bd, 0, s>>>(a);
-    } else {
-        k_image_fwd<<<(unsigned)a.npix, 32, 0, s>>>(a);
-    }
+    const int w1 = ceil_div(nfreq, 32), w2 = ceil_div(nfreq, 64);
+    if (paired_channels(w1, w2))
+        k_image_fwd2<<<(unsigned)a.npix, 32 * std::min(w2, 8), 0, s>>>(a);
+    else
+        k_image_fwd<<<(unsigned)a.npix, 32 * std::min(w1, 8), 0, s>>>(a);
     MGT_LAUNCH_CHECK("k_image_fwd");
     MGT_CUDA(cudaFreeAsync((void *)a.chan, s));
     if (!on_device) {

@@ -272,3 +272,17 @@ def test_channel_counts_around_the_pairs(mgt, nfreq):
         img = mgt.mgt_image(h, DIR, 5, 4, nfreq, a, b)
         ref, _ = O.image(m, _pops(m), DIR, 5, 4, nfreq, a, b)
         assert np.max(np.abs(img - ref) / np.abs(ref)) < 1e-4
+
+
+@pytest.mark.parametrize("nfreq", [64, 96, 97, 128, 129, 160, 161, 257])
+def test_channel_counts_where_pairs_begin_and_end(mgt, nfreq):
+    # two channels per thread where that saves enough warps (33 to 64 channels,
+    # 97 to 128, from 161), one per thread elsewhere; one line and a band of
+    # three; tolerance of the images
+    m = synth.shell_model(1500, 4, 1, 5, grf_sigma=2e3, seed=8, name="grf")
+    nu = m.lines.freq_Hz
+    h = mgt.mgt_model_create(m)
+    for a, b in ((0.9999 * nu[0], 1.0001 * nu[2]), _band(m, line=1)):
+        img = mgt.mgt_image(h, DIR, 3, 4, nfreq, a, b)
+        ref, _ = O.image(m, _pops(m), DIR, 3, 4, nfreq, a, b)
+        assert np.max(np.abs(img - ref) / np.abs(ref)) < 1e-4
