@@ -434,7 +434,9 @@ def mgt_remesh(pos, rho, r_max, max_level, n_side, stream=None):
     n = pos.shape[0]
     k = _i64(0)
     # one call: at most one box per point, and the surface nodes of the lattice
-    cap = n + max(0, 6 * int(n_side) ** 2 - 12 * int(n_side) + 8)
+    # (the library refuses an n_side outside 2..1024, whatever the capacity)
+    side = min(max(int(n_side), 2), 1024)
+    cap = n + 6 * side ** 2 - 12 * side + 8
     out = np.empty((cap, 3), np.float64)
     flags = np.empty(cap, np.uint8)
     _check(load().mgt_remesh(n, _ptr(pos), _ptr(rho), float(r_max), int(max_level), int(n_side), _ptr(out),

@@ -198,6 +198,17 @@ def test_remesh_rejects_bad_input_before_any_device_work(lib, kw, fragment):
     assert fragment in str(e.value)
 
 
+@pytest.mark.parametrize("n_side", [1, 0, -5, 1025, 100_000, -100_000, 2**31 - 1])
+def test_remesh_rejects_any_n_side_outside_its_range(lib, n_side):
+    # the output arrays are sized from n_side: an argument the library refuses
+    # must not ask for memory first
+    from paper_2411_03040_gb300 import mgt
+    with pytest.raises(mgt.MgtError) as e:
+        mgt.mgt_remesh(np.zeros((5, 3)), np.ones(5), 0.4, 5, n_side)
+    assert e.value.status == mgt.MGT_ERR_ARG
+    assert "n_side" in str(e.value)
+
+
 def test_noalloc_ng_rejects_sizes_and_null_pointers_before_any_device_work(lib):
     import ctypes as C
     buf = (C.c_double * 4)()
