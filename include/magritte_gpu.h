@@ -188,11 +188,13 @@ mgt_status mgt_set_solve_opts(mgt_model *m, const mgt_solve_opts *opts);
  * Most steps are settled by FP32 arithmetic with rigorous error bounds that
  * prove the FP64 predicates agree; the others are evaluated in FP64.
  * Stores the ray geometry on the device.  `stats` (host, may be NULL) is
- * filled after a stream synchronisation.  The walk's working memory (one
- * index slot per walk, a few GB for 10^5 points and 48 rays) comes
- * from a memory pool of this library, one per device, that keeps it reserved
- * for the next trace of any model; the reserve is returned to the driver when
- * the last model on that device is destroyed.  The model's ray buffer (16 B
+ * filled after a stream synchronisation.  The walk's working memory comes from
+ * a memory pool of this library, one per device, that keeps it reserved for the
+ * next trace of any model; the reserve is returned to the driver when the last
+ * model on that device is destroyed.  It is one slot of 4-byte point indices
+ * per walk: for a model's first trace 4 (4 N^(1/3) + 16) indices each (16 GB for
+ * 10^5 points and 48 rays, at most a third of the free memory), then what its
+ * longest half-ray needs.  The model's ray buffer (16 B
  * per step) comes from the same pool and is returned to it by
  * mgt_model_destroy.
  */
@@ -302,7 +304,10 @@ mgt_status mgt_ali_solve(mgt_model *m, const mgt_ali_opts *opts, mgt_ali_stats *
  *    optical depth over each segment, from B_nu_f(T_bg) at the far end.
  * Uses the current populations.  out: [nfreq][npy][npx] f32 intensities in
  * W m^-2 Hz^-1 sr^-1, host or device per on_device.  Pixel rays are traced on
- * the first call for a (dir, npx, npy) and kept.  The image is computed in
+ * the first call for a (dir, npx, npy) and kept.  Working memory: up to 1 GB of
+ * walk slots while rays are traced, and the image itself when `out` is host
+ * memory; buffers of up to 256 MB stay reserved in the library's pool (see
+ * mgt_trace_rays), larger ones go back to the driver.  The image is computed in
  * FP32.  MGT_ERR_ARG for a non-unit or non-finite dir, npx * npy > 2^26,
  * nfreq outside 1..65536 or not 0 < fmin <= fmax.
  */

@@ -125,6 +125,15 @@ mgt_status scratch_pool(cudaMemPool_t *pool)
     return MGT_OK;
 }
 
+mgt_status buffer_pool(size_t bytes, cudaMemPool_t *pool)
+{
+    if (bytes <= kPooledBytes) return scratch_pool(pool);
+    int dev = 0;
+    MGT_CUDA(cudaGetDevice(&dev));
+    MGT_CUDA(cudaDeviceGetMemPool(pool, dev));
+    return MGT_OK;
+}
+
 static void model_born(int dev)
 {
     std::lock_guard<std::mutex> lk(g_pool_mu);

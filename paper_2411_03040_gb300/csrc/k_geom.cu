@@ -1636,6 +1636,14 @@ static void image_release(ImageGeom &g, cudaStream_t s)
     g = ImageGeom{};
 }
 
+// Rays kept from a view four times as large, in buffers that do not go back to
+// the library's pool: a new view gets its own.
+static bool image_oversized(const ImageGeom &g, int64_t npix)
+{
+    const int64_t bytes = std::max<int64_t>(24 * g.npix_cap, 4 * g.pts_cap);
+    return g.npix_cap > 4 * npix && bytes > (int64_t)kPooledBytes;
+}
+
 void image_free(mgt_model *m)          // the device is idle
 {
     if (!m->img.d_ref) return;
@@ -1656,8 +1664,6 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
     g.shared = false;
     g.stream = s;
     const int64_t npix = (int64_t)npx * npy, N = m->N;
-    cudaMemPool_t pool = nullptr;
-    MGT_TRY_STATUS(scratch_pool(&pool));
     std::vector<void *> tmp;               // this call's temporaries
     struct Guard {
         std::vector<void *> &v;
@@ -1667,17 +1673,17 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
             for (void *p : v) cudaFreeAsync(p, s);
         }
     } guard{tmp, s};
-    auto temp = [&](auto **p, size_t count) -> cudaError_t {
-        const cudaError_t e = cudaMallocFromPoolAsync((void **)p, sizeof(**p) * count, pool, s);
-        if (e == cudaSuccess) tmp.push_back((void *)*p);
-        return e;
+    auto temp = [&](auto **p, int64_t count) -> mgt_status {
+        const mgt_status st = buffer_alloc(p, count, s);
+        if (st == MGT_OK) tmp.push_back((void *)*p);
+        return st;
     };
-    if (npix > g.npix_cap) {
+    if (npix > g.npix_cap || image_oversized(g, npix)) {
         image_release(g, s);
         g.stream = s;
-        MGT_CUDA(cudaMallocFromPoolAsync((void **)&g.d_ref, sizeof(double) * 3 * npix, pool, s));
-        MGT_CUDA(cudaMallocFromPoolAsync((void **)&g.d_anchor, sizeof(int32_t) * npix, pool, s));
-        MGT_CUDA(cudaMallocFromPoolAsync((void **)&g.d_off, sizeof(int64_t) * (npix + 1), pool, s));
+        MGT_TRY_STATUS(buffer_alloc(&g.d_ref, 3 * npix, s));
+        MGT_TRY_STATUS(buffer_alloc(&g.d_anchor, npix, s));
+        MGT_TRY_STATUS(buffer_alloc(&g.d_off, npix + 1, s));
         g.npix_cap = npix;
     }
     // the image plane's basis: e1 = unit(a x n), a the coordinate axis least
@@ -1700,9 +1706,10 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
     // search grid: two points per cell on average
     const int grid = (int)std::min(2048.0, std::max(1.0, std::ceil(std::sqrt(0.5 * (double)N))));
     const int64_t cells = (int64_t)grid * grid;
-    // scratch slot per half-ray, as in trace_range, at most 1 GB in all
+    // scratch slot per half-ray, as in trace_range, at most 1 GB in all: above
+    // 8.4 million pixels none, and every ray is walked again into its place
     const int64_t usual = ((int64_t)(8.0 * std::cbrt((double)N)) + 16 + 15) / 16 * 16;
-    const int32_t K = (int32_t)std::max<int64_t>(16, std::min(usual, ((int64_t)1 << 30) / (8 * npix) / 16 * 16));
+    const int32_t K = (int32_t)std::min(usual, ((int64_t)1 << 30) / (8 * npix) / 16 * 16);
     ImgPlane *d_pl = nullptr;
     double2 *d_s12 = nullptr;
     int32_t *d_count = nullptr, *d_start = nullptr, *d_scratch = nullptr;
@@ -1713,16 +1720,16 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
     size_t cub1 = 0, cub2 = 0;
     MGT_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, cub1, d_count, d_start, (int)(cells + 1), s));
     MGT_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, cub2, d_sizes, g.d_off, npix + 1, s));
-    MGT_CUDA(temp(&d_pl, 1));
-    MGT_CUDA(temp(&d_s12, N));
-    MGT_CUDA(temp(&d_count, cells + 1));
-    MGT_CUDA(temp(&d_start, cells + 1));
-    MGT_CUDA(temp(&d_sorted, 2 * N));
-    MGT_CUDA(temp(&d_scratch, 2 * npix * K));
-    MGT_CUDA(temp(&d_lens, 2 * npix));
-    MGT_CUDA(temp(&d_sizes, npix + 1));
-    MGT_CUDA(temp(&d_longest, 2));
-    MGT_CUDA(temp(&d_cub, std::max<size_t>(std::max(cub1, cub2), 1)));
+    MGT_TRY_STATUS(temp(&d_pl, 1));
+    MGT_TRY_STATUS(temp(&d_s12, N));
+    MGT_TRY_STATUS(temp(&d_count, cells + 1));
+    MGT_TRY_STATUS(temp(&d_start, cells + 1));
+    MGT_TRY_STATUS(temp(&d_sorted, 2 * N));
+    MGT_TRY_STATUS(temp(&d_scratch, 2 * npix * K));
+    MGT_TRY_STATUS(temp(&d_lens, 2 * npix));
+    MGT_TRY_STATUS(temp(&d_sizes, npix + 1));
+    MGT_TRY_STATUS(temp(&d_longest, 2));
+    MGT_TRY_STATUS(temp(&d_cub, std::max<size_t>(std::max(cub1, cub2), 1)));
     MGT_CUDA(cudaMemcpyAsync(d_pl, &pl, sizeof pl, cudaMemcpyHostToDevice, s));
     MGT_CUDA(cudaMemsetAsync(d_count, 0, sizeof(int32_t) * (cells + 1), s));
     MGT_CUDA(cudaMemsetAsync(d_longest, 0, sizeof(int) * 2, s));
@@ -1760,7 +1767,7 @@ mgt_status trace_image(mgt_model *m, const double n[3], int32_t npx, int32_t npy
         if (g.d_pts) MGT_CUDA(cudaFreeAsync(g.d_pts, s));
         g.d_pts = nullptr;
         g.pts_cap = 0;
-        MGT_CUDA(cudaMallocFromPoolAsync((void **)&g.d_pts, sizeof(int32_t) * total, pool, s));
+        MGT_TRY_STATUS(buffer_alloc(&g.d_pts, total, s));
         g.pts_cap = total;
     }
     k_img_place<<<ceil_div(npix * 32, kImgThreads), kImgThreads, 0, s>>>(npix, d_lens, g.d_off, g.d_anchor, K, d_scratch,

@@ -651,22 +651,11 @@ ImgArgs image_args(mgt_model *m, const double *dir, int32_t nfreq, double fmin, 
     return a;
 }
 
-// A temporary of one call, from the library's pool: the default pool gives its
-// memory back at the next synchronisation and maps it again for the next call
-// (240 us).
-template <typename T> mgt_status image_temp(T **p, int64_t n, cudaStream_t s)
-{
-    cudaMemPool_t pool = nullptr;
-    MGT_TRY_STATUS(scratch_pool(&pool));
-    MGT_CUDA(cudaMallocFromPoolAsync((void **)p, sizeof(T) * n, pool, s));
-    return MGT_OK;
-}
-
 // The per-channel constants of one call, stream-ordered; the caller frees a.chan.
 mgt_status image_channels(ImgArgs &a, cudaStream_t s)
 {
     Chan *c = nullptr;
-    MGT_TRY_STATUS(image_temp(&c, a.nfreq, s));
+    MGT_TRY_STATUS(buffer_alloc(&c, a.nfreq, s));
     k_image_chan<<<a.nfreq, 32, 0, s>>>(a, c);
     MGT_LAUNCH_CHECK("k_image_chan");
     a.chan = c;
@@ -715,7 +704,7 @@ mgt_status mgt_image(mgt_model *m, const double dir[3], int32_t npx, int32_t npy
     ImgArgs a = image_args(m, dir, nfreq, fmin, fmax);
     const int64_t n = a.npix * nfreq;
     float *dev = out;
-    if (!on_device) MGT_TRY_STATUS(image_temp(&dev, n, s));
+    if (!on_device) MGT_TRY_STATUS(buffer_alloc(&dev, n, s));
     a.out = dev;
     MGT_TRY_STATUS(image_channels(a, s));
     const int w1 = ceil_div(nfreq, 32), w2 = ceil_div(nfreq, 64);
@@ -748,11 +737,11 @@ mgt_status mgt_image_adjoint(mgt_model *m, const double dir[3], int32_t npx, int
     const int64_t n = a.npix * nfreq, N = m->N;
     double *acc = nullptr, *gv = nullptr;
     float *gdev = nullptr;
-    MGT_TRY_STATUS(image_temp(&acc, 3 * N, s));
-    MGT_TRY_STATUS(image_temp(&gv, 3 * N, s));
+    MGT_TRY_STATUS(buffer_alloc(&acc, 3 * N, s));
+    MGT_TRY_STATUS(buffer_alloc(&gv, 3 * N, s));
     MGT_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * N, s));
     if (!on_device) {
-        MGT_TRY_STATUS(image_temp(&gdev, n, s));
+        MGT_TRY_STATUS(buffer_alloc(&gdev, n, s));
         MGT_CUDA(cudaMemcpyAsync(gdev, grad_out, sizeof(float) * n, cudaMemcpyHostToDevice, s));
     }
     a.gout = on_device ? grad_out : gdev;
@@ -797,7 +786,7 @@ mgt_status mgt_set_point_fields(mgt_model *m, const double *temp, const double *
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (n_spec) {
         double *ns = nullptr;
-        MGT_TRY_STATUS(image_temp(&ns, N, s));
+        MGT_TRY_STATUS(buffer_alloc(&ns, N, s));
         MGT_CUDA(cudaMemcpyAsync(ns, n_spec, sizeof(double) * N, kind, s));
         k_rescale_pops<<<ceil_div(N * m->L, kRescaleItems), kRescaleThreads, 0, s>>>(N, m->L, m->d_nspec, ns, m->d_pops, m->d_pops_prev);
         MGT_LAUNCH_CHECK("k_rescale_pops");

@@ -66,7 +66,7 @@ struct ImageGeom {
     int32_t *d_anchor = nullptr;        // [npix]
     int64_t *d_off = nullptr;           // [npix+1]
     int32_t *d_pts = nullptr;           // [total] far end first
-    int64_t npix_cap = 0, pts_cap = 0;  // what the buffers hold (from the library's pool)
+    int64_t npix_cap = 0, pts_cap = 0;  // what the buffers hold
     cudaStream_t stream = nullptr;      // the stream they were filled on
     bool shared = false;                // read on another stream too
 };
@@ -206,6 +206,26 @@ private:
 void note_launch();
 mgt_status set_error(mgt_status s, const std::string &msg);
 mgt_status cuda_status(cudaError_t e, const char *what);
+
+// Where a buffer of the image calls comes from: up to kPooledBytes from the
+// library's pool, since the device's own pool unmaps what a call gives back at
+// the next synchronisation and maps it again for the next call (240 us at 256 x
+// 256 pixels x 100 channels); larger ones, where that weighs little, from the
+// device's pool, so that no call leaves more than some hundred MB reserved.
+constexpr size_t kPooledBytes = (size_t)256 << 20;
+mgt_status buffer_pool(size_t bytes, cudaMemPool_t *pool);
+
+template <typename T> mgt_status buffer_alloc(T **p, int64_t n, cudaStream_t s)
+{
+    const size_t bytes = sizeof(T) * (size_t)(n > 0 ? n : 1);
+    cudaMemPool_t pool = nullptr;
+    const mgt_status st = buffer_pool(bytes, &pool);
+    if (st != MGT_OK) return st;
+    const cudaError_t e = cudaMallocFromPoolAsync((void **)p, bytes, pool, s);
+    if (e == cudaSuccess) return MGT_OK;
+    cudaGetLastError();                  // (a later launch check would report it again)
+    return cuda_status(e, "cudaMallocFromPoolAsync");
+}
 mgt_status check_device_error(mgt_model *m, cudaStream_t s);
 
 // geometry / line-data kernels (k_geom.cu)
