@@ -1424,11 +1424,14 @@ __global__ void k_img_sort(int64_t N, const double2 *__restrict__ s12, const Img
 // Anchor of each pixel: the point whose squared distance to the pixel line
 // |(x - p) - ((x - p).n) n|^2 is smallest, ties to the smaller index.  One
 // warp per pixel looks at the points in a window of grid cells around the
-// pixel: FP32 distances from hi + lo positions with the error bounds of the
-// walk, an FP64 scan of the window (the defining expressions) when the bounds
-// do not separate the winner from every other point.  The window grows until
-// every point within the winner's upper bound (plus the rounding of the
-// projections) lies inside it, so no point outside can win or tie.
+// pixel: FP32 distances from hi + lo positions with the error bounds ep and e2
+// of the walk (its offsets' 2s holds here too: the reference point's scaled
+// coordinates are at most 3.1, so hi + lo leaves 4.1 2^-48 out of an offset and
+// its low parts round by as much, 3.6 s in all over the three components), an
+// FP64 scan of the window (the defining expressions) when the bounds do not
+// separate the winner from every other point.  The window grows until every
+// point within the winner's upper bound (plus the rounding of the projections)
+// lies inside it, so no point outside can win or tie.
 //
 // Every pixel against every point took 5.3 ms for 16,384 pixels and 100k
 // points (issue bound, 1.6e9 distances); the grid holds two points per cell on
@@ -1500,14 +1503,12 @@ __global__ void __launch_bounds__(kImgThreads) k_img_anchor(WalkArgs a, const Im
             const int i = __float_as_int(h.b.z);
             const float dx = (h.a.x - ohx) + (h.a.w - olx), dy = (h.a.y - ohy) + (h.b.x - oly),
                         dz = (h.a.z - ohz) + (h.b.y - olz);
-            const float adx = fabsf(dx), ady = fabsf(dy), adz = fabsf(dz);
-            const float ed = 2e-6f * (fmaxf(adx, fmaxf(ady, adz)) + a.pos_slack);
+            const float S = fabsf(dx) + fabsf(dy) + fabsf(dz);
             const float Z = fmaf(dz, f2, fmaf(dy, f1, dx * f0));
-            const float eZ = 2e-6f * (adx + ady + adz) + 2.0f * ed;
             const float px = fmaf(-Z, f0, dx), py = fmaf(-Z, f1, dy), pz = fmaf(-Z, f2, dz);
             const float d2 = fmaf(pz, pz, fmaf(py, py, px * px));
-            const float ep = ed + eZ + 2e-7f * (fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))) + fabsf(Z));
-            const float e2 = 4.0f * sqrtf(d2) * ep + 4.0f * ep * ep + 1e-6f * d2;
+            const float ep = fmaf(8e-7f, S, 8.0f * a.pos_slack);
+            const float e2 = fmaf(ep, fmaf(2.5f, sqrtf(d2), ep), 4e-7f * d2);
             if (d2 < bd2) {
                 minLo = fminf(minLo, bL);
                 bd2 = d2;

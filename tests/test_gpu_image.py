@@ -286,3 +286,34 @@ def test_channel_counts_where_pairs_begin_and_end(mgt, nfreq):
         img = mgt.mgt_image(h, DIR, 3, 4, nfreq, a, b)
         ref, _ = O.image(m, _pops(m), DIR, 3, 4, nfreq, a, b)
         assert np.max(np.abs(img - ref) / np.abs(ref)) < 1e-4
+
+
+def _bare_cloud(pos, rng):
+    """Points with random neighbours and plain fields, for the pixel rays alone."""
+    n = pos.shape[0]
+    nb = [rng.choice(n, size=8, replace=False) for _ in range(n)]
+    return synth.Model("cloud", pos, np.zeros((n, 3)), np.full(n, 50.0), np.full(n, 1e4), np.full(n, 1e10),
+                       np.full(n, 1e5), 8 * np.arange(n + 1, dtype=np.int64),
+                       np.concatenate([np.sort(v) for v in nb]).astype(np.int32), np.arange(0, n, 10, dtype=np.int32),
+                       synth.healpix_directions(1), 3, synth.linear_rotor(3, rng))
+
+
+def test_anchors_among_points_closer_than_float_pairs_resolve(mgt):
+    # around every pixel's reference point eight points at 1e-11 of the model's
+    # extent from the pixel line, whose distances differ by less than float
+    # hi + lo positions resolve: FP64 decides, equality
+    rng = np.random.default_rng(17)
+    npx, npy = 12, 10
+    pos = rng.uniform(-1, 1, size=(200, 3)) * 1e11
+    r = O.image_rays(_bare_cloud(pos, rng), DIR, npx, npy)
+    ang = rng.uniform(0, 2 * np.pi, (npx * npy, 8))
+    rad = 1.0 + rng.uniform(0.0, 4e-4, ang.shape)                     # m: 4e-15 of 1e11 m
+    off = rad[..., None] * (np.cos(ang)[..., None] * r.e1 + np.sin(ang)[..., None] * r.e2)
+    near = (r.ref[:, None, :] + off).reshape(-1, 3)
+    inside = np.all(np.abs(near) < 0.9e11, axis=1)                   # the frame stays the cloud's
+    assert inside.sum() > 200
+    m = _bare_cloud(np.concatenate([pos, near[inside]]), rng)
+    ref = O.image_rays(m, DIR, npx, npy)
+    assert np.array_equal(ref.ref, r.ref) and (ref.anchor >= 200).sum() > 40
+    anchor, _, _ = mgt.mgt_image_rays(mgt.mgt_model_create(m), DIR, npx, npy)
+    assert np.array_equal(anchor, ref.anchor)
