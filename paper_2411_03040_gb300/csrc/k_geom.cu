@@ -1430,8 +1430,11 @@ __global__ void k_img_sort(int64_t N, const double2 *__restrict__ s12, const Img
 // its low parts round by as much, 3.6 s in all over the three components), an
 // FP64 scan of the window (the defining expressions) when the bounds do not
 // separate the winner from every other point.  The window grows until every
-// point within the winner's upper bound (plus the rounding of the projections)
-// lies inside it, so no point outside can win or tie.
+// point within the winner's upper bound (plus a margin for the projections)
+// lies inside it, so no point outside can win or tie.  The margin: a direction
+// may be 5e-13 from unit length, e2 = n x e1 with it, and then a pixel lies up to
+// 2 x 5e-13 x 2.6 beside its place among the projections (in units of the
+// scaled positions).
 //
 // Every pixel against every point took 5.3 ms for 16,384 pixels and 100k
 // points (issue bound, 1.6e9 distances); the grid holds two points per cell on
@@ -1459,7 +1462,7 @@ __global__ void __launch_bounds__(kImgThreads) k_img_anchor(WalkArgs a, const Im
                  t2 = pl.first2 + ((double)jy + 0.5) * pl.step2;
     const int cx = img_cell(t1, pl.first1, pl, grid), cy = img_cell(t2, pl.first2, pl, grid);
     const double inv_scale = 1.0 / a.pos_scale;
-    const double margin = 1e-12 * inv_scale;       // far above the rounding of projections and cell edges
+    const double margin = 1e-11 * inv_scale;       // (far above the rounding of projections and cell edges)
     float bd2, bU, bL, minLo;
     int bi, best = -1;
     // every point of the window, 32 at a time: rows of cells are contiguous

@@ -317,3 +317,20 @@ def test_anchors_among_points_closer_than_float_pairs_resolve(mgt):
     assert np.array_equal(ref.ref, r.ref) and (ref.anchor >= 200).sum() > 40
     anchor, _, _ = mgt.mgt_image_rays(mgt.mgt_model_create(m), DIR, npx, npy)
     assert np.array_equal(anchor, ref.anchor)
+
+
+def test_anchors_of_a_small_cloud_far_away_with_a_rounded_direction(mgt):
+    # a direction as far from unit length as the call accepts shifts the pixels
+    # against the projections by 1e-12 of their distance from the plane's
+    # origin: here by about a cell of the search grid (points in the plane of
+    # the reference points, 1.2 from its origin).  FP64 decides, equality
+    rng = np.random.default_rng(23)
+    d = np.array([-0.576, 0.578, 0.578]) / np.linalg.norm([-0.576, 0.578, 0.578])
+    e2 = np.array([1.0, 0.0, 0.0]) - d[0] * d
+    e2 /= np.linalg.norm(e2)
+    uv = rng.uniform(-3e-11, 3e-11, size=(5000, 2))
+    m = _bare_cloud((1.2 * e2 + uv[:, :1] * np.cross(d, e2) + uv[:, 1:] * e2) * 2.0 ** 37, rng)
+    h = mgt.mgt_model_create(m)
+    for scale in (1.0 - 4.9e-13, 1.0 + 4.9e-13):
+        anchor, _, _ = mgt.mgt_image_rays(h, d * scale, 80, 80)
+        assert np.array_equal(anchor, O.image_rays(m, d * scale, 80, 80).anchor)
