@@ -51,6 +51,7 @@ struct SEArgs {
 
 constexpr int kMaxWarpsPerBlock = 4;
 constexpr size_t kSEMaxSmem = 227 * 1024;
+constexpr size_t kSEBatchStatic = (sizeof(SEArgs) + sizeof(int64_t) + 31) / 16 * 16;   // k_se_batch's static arrays
 
 // A point's working memory in doubles: the rates, the reciprocals 1/bz (later
 // the unnormalised populations), and the lines' rates (later the pivots'
@@ -309,12 +310,13 @@ SEArgs fill_se_args(const mgt_model *m)
     return a;
 }
 
-// Warps per CTA, CTAs and a CTA's shared memory; false if no warp's points fit.
-bool se_layout(const mgt_model *m, int *wpb, int64_t *blocks, size_t *smem)
+// Warps per CTA, CTAs and a CTA's dynamic shared memory (at most `most`); false
+// if no warp's points fit.
+bool se_layout(const mgt_model *m, size_t most, int *wpb, int64_t *blocks, size_t *smem)
 {
     const int points = 32 / se_lanes(m->L);
     const size_t per_warp = sizeof(double) * points * (size_t)se_point_doubles(m->L, m->M);
-    *wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, kSEMaxSmem / per_warp);
+    *wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, most / per_warp);
     if (*wpb < 1) return false;
     *blocks = ceil_div(m->N, (int64_t)*wpb * points);
     *smem = per_warp * *wpb;
@@ -328,7 +330,7 @@ mgt_status launch_stat_eq(mgt_model *m, cudaStream_t s)
     SEArgs a = fill_se_args(m);
     int64_t blocks = 0;
     size_t smem = 0;
-    if (!se_layout(m, &a.wpb, &blocks, &smem))
+    if (!se_layout(m, kSEMaxSmem, &a.wpb, &blocks, &smem))
         return set_error(MGT_ERR_ARG, "statistical equilibrium: too many levels/lines for shared memory");
     MGT_TRY_STATUS(raise_smem_limit((const void *)k_se, smem));
     {
@@ -347,7 +349,8 @@ mgt_status se_batch_args(const mgt_model *m, void *args, int64_t *blocks, size_t
     // the batch's documented limit
     if (4 * sizeof(double) * ((size_t)m->L * m->L + 3 * m->L + 2 * m->Mpad) > kSEMaxSmem)
         return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
-    if (!se_layout(m, &a.wpb, blocks, smem))
+    // (k_se_batch also holds a model's arguments in shared memory)
+    if (!se_layout(m, kSEMaxSmem - kSEBatchStatic, &a.wpb, blocks, smem))
         return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
     std::memcpy(args, &a, sizeof a);
     return MGT_OK;

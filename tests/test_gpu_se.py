@@ -50,3 +50,27 @@ def test_level_and_point_edges(mgt, levels, n, batched):
     # the previous populations are kept for the change that Ng reports
     _, change = mgt.mgt_ng_accelerate(h)
     assert change == pytest.approx(np.max(np.abs(got - p0) / p0), rel=1e-9)
+
+
+def test_batch_at_the_shared_memory_limit(mgt):
+    # 64 levels x 340 lines: three warps of the batched kernel hold 232,320 of the
+    # 232,448 bytes of shared memory that a CTA may use, and the kernel's copy of
+    # a model's arguments takes 144 more
+    levels, n_lines = 64, 340
+    m = synth.sphere_model(40, levels, 1, 3, seed=9)
+    ln = m.lines
+    pairs = np.array([(u, l) for u in range(levels) for l in range(u)], np.int32)[-n_lines:]
+    ln.up, ln.lo = np.ascontiguousarray(pairs[:, 0]), np.ascontiguousarray(pairs[:, 1])
+    ln.freq_Hz = 1e11 * 1.02 ** np.arange(n_lines)
+    ln.A = np.full(n_lines, 1e-6)
+    m.n_coll = m.n_coll * 1e-4
+    h = mgt.mgt_model_create(m)
+    mgt.mgt_trace_rays(h)
+    b = mgt.mgt_batch_create([h])
+    mgt.mgt_batch_formal_solve(b)
+    mgt.mgt_batch_stat_equilibrium(b)
+    J, L = mgt.mgt_get_jbar(h)
+    p0 = O.lte_populations(m.temp, m.n_spec, ln.energy_J, ln.g)
+    ref = O.stat_equilibrium(p0, J.T, L.T, m.temp, m.n_coll, m.n_spec, ln)
+    got = mgt.mgt_get_populations(h)
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-8
