@@ -1685,12 +1685,15 @@ int staged_threads(const FSArgs &a) { return ((a.Q * a.Gb + 31) / 32) * 32; }
 // FP32 holds a third buffer of step records.  A model of some hundred lines
 // whose origin fitted the shared memory with two takes fewer line groups per
 // CTA, so that it fits with three (the lines' results do not depend on it).
-template <typename T, int LPT, int CH> void fit_line_groups(FSArgs &a, bool fused)
+// `most`: what a CTA may take as dynamic shared memory.
+constexpr int kFSMaxSmem = 227 * 1024;
+constexpr int kFSBatchStatic = ((int)sizeof(FSArgs) + 24 + 15) / 16 * 16;    // k_fs_batch's static arrays
+
+template <typename T, int LPT, int CH> void fit_line_groups(FSArgs &a, bool fused, int most)
 {
     auto total = [&](int bufs) {
         return staged_layout<T, LPT, CH>(a.Q, a.Gb * LPT, a.RS, staged_threads(a), a.P, fused, bufs).total;
     };
-    constexpr int most = 227 * 1024;
     if (total(2) > most) return;
     while (a.Gb > 1 && total(kStepBufs<T>) > most) --a.Gb;
     a.nblk = ceil_div(a.Gtot, a.Gb);
@@ -1751,7 +1754,7 @@ mgt_status launch_typed(mgt_model *m, cudaStream_t s, int schedule, bool accumul
     if (staged) {
         a.OPB = 1;
         a.fused = (schedule == 4 || (schedule == 0 && a.Gtot == 1)) ? 1 : 0;
-        fit_line_groups<T, LPT, kChunk>(a, a.fused != 0);
+        fit_line_groups<T, LPT, kChunk>(a, a.fused != 0, kFSMaxSmem);
         const int bd = staged_threads(a), Mb = a.Gb * LPT;
         if (bd > 256) return set_error(MGT_ERR_ARG, "formal solve: more than 256 bins per origin");
         const size_t smem = (size_t)staged_layout<T, LPT, kChunk>(a.Q, Mb, a.RS, bd, a.P, a.fused != 0).total;
@@ -1821,9 +1824,9 @@ mgt_status fs_batch_args(const mgt_model *m, void *args, int *threads, int64_t *
     a.fused = a.Gtot == 1 ? 1 : 0;     // as the automatic single-model choice
     // (by the long chunks, which need more)
     if (lpt == 4)
-        fit_line_groups<float, 4, kChunk>(a, a.fused != 0);
+        fit_line_groups<float, 4, kChunk>(a, a.fused != 0, kFSMaxSmem - kFSBatchStatic);
     else
-        fit_line_groups<float, 8, kChunk>(a, a.fused != 0);
+        fit_line_groups<float, 8, kChunk>(a, a.fused != 0, kFSMaxSmem - kFSBatchStatic);
     const int bd = staged_threads(a);
     if (bd > 256) return set_error(MGT_ERR_ARG, "batched formal solve: more than 256 bins per origin");
     *threads = bd;

@@ -305,3 +305,24 @@ def test_autotune_picks_a_timed_candidate(mgt, batch_models):
     np.testing.assert_array_equal(Ja, Jb)
     r64 = mgt.mgt_autotune(h, mgt.MGT_FP64, staged_only=True, reps=1)
     assert [(s, l) for s, l, _ in r64["tried"]] == [(0, 4)]
+
+
+@pytest.mark.parametrize("n_lines", [328, 330, 336])
+def test_batch_lines_at_the_shared_memory_limit(mgt, n_lines):
+    # 329 to 336 lines x 10 bins x 48 rays: 232,224 of the 232,448 bytes of a CTA's
+    # shared memory with all line groups, and the persistent kernel's copy of
+    # the arguments takes 256 more: fewer line groups per CTA, the same values
+    levels = 27
+    m = synth.sphere_model(30, levels, 2, 10, seed=9)
+    ln = m.lines
+    pairs = np.array([(u, l) for u in range(levels) for l in range(u)], np.int32)[:n_lines]
+    ln.up, ln.lo = np.ascontiguousarray(pairs[:, 0]), np.ascontiguousarray(pairs[:, 1])
+    ln.freq_Hz = 1e11 * 1.02 ** np.arange(n_lines)
+    ln.A = np.full(n_lines, 1e-6)
+    h = _handle(mgt, m, 8)
+    J, L = mgt.mgt_formal_solve(h, mgt.MGT_FP32_MIXED)
+    b = mgt.mgt_batch_create([h])
+    mgt.mgt_batch_formal_solve(b)
+    Jb, Lb = mgt.mgt_get_jbar(h)
+    np.testing.assert_array_equal(Jb, J)
+    np.testing.assert_array_equal(Lb, L)
