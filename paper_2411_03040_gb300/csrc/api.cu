@@ -156,6 +156,7 @@ mgt_status set_error(mgt_status s, const std::string &msg)
 
 mgt_status cuda_status(cudaError_t e, const char *what)
 {
+    cudaGetLastError();                  // reported here: the next launch check must not find it again
     std::string msg = std::string(what) + ": " + cudaGetErrorString(e);
     return set_error(e == cudaErrorMemoryAllocation ? MGT_ERR_OOM : MGT_ERR_CUDA, msg);
 }

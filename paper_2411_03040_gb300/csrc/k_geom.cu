@@ -1245,7 +1245,10 @@ mgt_status trace_range(mgt_model *m, cudaStream_t s, int32_t p0, int32_t np)
     m->steps64_width_mode = -1;                // the FP64 geometry describes the previous rays
     if (!m->d_steps32 && total > 0) {
         cudaError_t e = cudaMallocFromPoolAsync(&m->d_steps32, sizeof(Step32) * total, pool, s);
-        if (e != cudaSuccess) return set_error(MGT_ERR_OOM, "cannot allocate the ray buffer");
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(MGT_ERR_OOM, "cannot allocate the ray buffer");
+        }
         m->steps32_cap = total;
     }
     m->total_steps = total;
@@ -1292,7 +1295,10 @@ mgt_status build_steps64(mgt_model *m, cudaStream_t s)
     if (!m->d_steps64) {
         m->steps64_cap = m->total_steps;
         cudaError_t e = cudaMalloc(&m->d_steps64, sizeof(Step64) * m->total_steps);
-        if (e != cudaSuccess) return set_error(MGT_ERR_OOM, "cannot allocate the FP64 ray geometry");
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(MGT_ERR_OOM, "cannot allocate the FP64 ray geometry");
+        }
     }
     const bool all = m->rays_p0 == 0 && m->rays_np == m->P;
     const int32_t Rw = all ? m->R : 2 * m->rays_np;

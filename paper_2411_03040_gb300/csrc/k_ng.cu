@@ -207,7 +207,10 @@ static mgt_status ng_alloc(mgt_model *m, const mgt_ng_opts &o)
         if (ng.d_slots) MGT_CUDA(cudaFree(ng.d_slots));
         ng.d_slots = nullptr;
         cudaError_t e = cudaMalloc(&ng.d_slots, sizeof(double) * n * need);
-        if (e != cudaSuccess) return set_error(MGT_ERR_OOM, "cannot allocate the Ng history");
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(MGT_ERR_OOM, "cannot allocate the Ng history");
+        }
         ng.n_slots = need;
         ng.hist.clear();
         ng.have_prev_pred = false;

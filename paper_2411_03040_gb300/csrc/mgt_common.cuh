@@ -222,9 +222,7 @@ template <typename T> mgt_status buffer_alloc(T **p, int64_t n, cudaStream_t s)
     const mgt_status st = buffer_pool(bytes, &pool);
     if (st != MGT_OK) return st;
     const cudaError_t e = cudaMallocFromPoolAsync((void **)p, bytes, pool, s);
-    if (e == cudaSuccess) return MGT_OK;
-    cudaGetLastError();                  // (a later launch check would report it again)
-    return cuda_status(e, "cudaMallocFromPoolAsync");
+    return e == cudaSuccess ? MGT_OK : cuda_status(e, "cudaMallocFromPoolAsync");
 }
 mgt_status check_device_error(mgt_model *m, cudaStream_t s);
 

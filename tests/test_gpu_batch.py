@@ -326,3 +326,23 @@ def test_batch_lines_at_the_shared_memory_limit(mgt, n_lines):
     Jb, Lb = mgt.mgt_get_jbar(h)
     np.testing.assert_array_equal(Jb, J)
     np.testing.assert_array_equal(Lb, L)
+
+
+def test_a_refused_call_leaves_the_next_one_alone(mgt):
+    # 336 lines x 11 bins x 48 rays fit a CTA alone but not beside the persistent
+    # kernel's copy of the arguments: the driver refuses the shared memory, and
+    # the error is reported by that call only
+    levels, n_lines = 27, 336
+    m = synth.sphere_model(30, levels, 2, 11, seed=9)
+    ln = m.lines
+    pairs = np.array([(u, l) for u in range(levels) for l in range(u)], np.int32)[:n_lines]
+    ln.up, ln.lo = np.ascontiguousarray(pairs[:, 0]), np.ascontiguousarray(pairs[:, 1])
+    ln.freq_Hz = 1e11 * 1.02 ** np.arange(n_lines)
+    ln.A = np.full(n_lines, 1e-6)
+    h = _handle(mgt, m, 8)
+    with pytest.raises(mgt.MgtError):
+        mgt.mgt_batch_create([h])
+    other = mgt.mgt_model_create(synth.sphere_model(40, 3, 1, 3, seed=2))
+    assert mgt.mgt_trace_rays(other)["total_steps"] > 0
+    J, _ = mgt.mgt_formal_solve(h, mgt.MGT_FP32_MIXED)
+    assert np.all(np.isfinite(J))
