@@ -133,6 +133,8 @@ mgt_status refresh(mgt_batch *b, cudaStream_t s)
         return cost[x] > cost[y];
     });
 
+    int64_t points = 0;
+    for (const mgt_model *m : b->models) points += m->N;
     std::vector<unsigned char> fa(fsz * n), sa(ssz * n), la(lsz * n);
     std::vector<int64_t> fe(n), se(n), le(n);
     std::vector<mgt_batch::FsClass> classes;
@@ -166,7 +168,7 @@ mgt_status refresh(mgt_batch *b, cudaStream_t s)
         }
         int64_t sblocks = 0, lblocks = 0;
         size_t ssm = 0;
-        MGT_TRY_STATUS(se_batch_args(m, sa.data() + k * ssz, &sblocks, &ssm));
+        MGT_TRY_STATUS(se_batch_args(m, points, sa.data() + k * ssz, &sblocks, &ssm));
         MGT_TRY_STATUS(ld_batch_args(m, la.data() + k * lsz, &lblocks));
         se_smem = std::max(se_smem, ssm);
         se[k] = (si += sblocks);

@@ -47,6 +47,7 @@ struct SEArgs {
     double *pops_out;         // [N][L] (may be pops_old: each point's row is read before it is written)
     double *pops_prev;        // [N][L] copy of pops_old
     int wpb;                  // warps of a CTA that take points (what its shared memory holds)
+    int lanes;                // lanes per point
 };
 
 constexpr int kMaxWarpsPerBlock = 4;
@@ -58,12 +59,42 @@ constexpr size_t kSEBatchStatic = (sizeof(SEArgs) + sizeof(int64_t) + 31) / 16 *
 // reciprocals).
 __host__ __device__ inline int se_point_doubles(int L, int M) { return L * L + L + (L > 2 * M ? L : 2 * M); }
 
-// Lanes per point: enough points per warp to fill the FP64 instructions, enough
-// warps to hide their latency.  41 levels: 16 lanes 8.1 ms per 100k points, 8
-// lanes (16 points of 14.4 KB fill an SM's shared memory, so one warp per
-// scheduler) 10.4; 21 levels: 8 lanes 1.6, 4 lanes 2.1, 16 lanes 2.3; 11 levels:
-// 4 lanes 0.48, 8 lanes 0.72.
-__host__ __device__ inline int se_lanes(int L) { return L > 32 ? 16 : L > 16 ? 8 : 4; }
+constexpr int kLevelsPerLane = 4;                 // G lanes hold up to 4 G levels
+static_assert(kMaxLevels <= 16 * kLevelsPerLane, "levels per lane");
+
+// Lanes per point.  Many points: the fewest lanes, so that an FP64 instruction
+// serves as many points as possible, with two warps per scheduler in an SM's
+// shared memory.  100k points: 11 levels 4 lanes 0.44 ms, 8 lanes 0.60; 21
+// levels 8 lanes 1.49, 16 lanes 2.08; 28 levels 2.90, 3.34; 32 levels (8 lanes:
+// one warp per scheduler) 5.89, 16 lanes 4.25; 41 levels 16 lanes 7.51, 32 lanes
+// 9.34; 48 levels 15.9, 13.2.  Few points: more lanes while they still get a
+// scheduler to themselves, or half of one above 16 levels (a point's chain is
+// what lasts then): 1,200 points of 11 levels 16 lanes 18.5 us, 4 lanes 36.4; 21
+// levels 32 lanes 41, 8 lanes 63; 3,000 points of 21 levels 16 lanes 82, 8 lanes
+// 80.  Results do not depend on it.
+inline int se_lanes(int L, int M, int64_t points, int sms)
+{
+    constexpr size_t sm_smem = 228 * 1024, cta_smem = 1024;    // an SM's, and what a CTA takes of it by itself
+    auto few_resident = [&](int g) {
+        return 2 * (kMaxWarpsPerBlock * sizeof(double) * (32 / g) * (size_t)se_point_doubles(L, M) + cta_smem) > sm_smem;
+    };
+    int g = 4;
+    while (g < 32 && (L > kLevelsPerLane * g || few_resident(g))) g *= 2;
+    while (g < 32 && points * 2 * g <= (int64_t)sms * 32 * (L > 16 ? 8 : 4)) g *= 2;
+    return g;
+}
+
+// The device's SMs (0 where there is none: host checks).
+int se_sms()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return sms;
+}
 
 // Sum of v[0 .. n-1] (n <= 64) over the point's lanes, in the order of a warp
 // that holds v[l] + v[l + 32] in lane l and adds lanes 16, 8, 4, 2 and 1 apart,
@@ -88,9 +119,6 @@ template <int G> __device__ __forceinline__ double point_sum(const double *v, in
         if (n > o) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o, G);
     return __shfl_sync(0xffffffffu, s[0], 0, G);
 }
-
-constexpr int kLevelsPerLane = 4;                 // G lanes hold up to 4 G levels
-static_assert(kMaxLevels <= 16 * kLevelsPerLane, "levels per lane");
 
 // v > 0 for a sum of non-negative numbers (false for NaN), by its bits: a
 // comparison on the FP64 pipe costs as much as a multiply-add.
@@ -174,7 +202,7 @@ template <int G> __device__ __forceinline__ void se_point(const SEArgs &a, int64
         // rows i, columns j < n: entry e = i n + j, the stride advances (i, j)
         // by (di, dj); with few warps per scheduler two entries at a time,
         // loads before stores, so that their latencies overlap
-        constexpr int kUpdate = G == 16 ? 2 : 1;
+        constexpr int kUpdate = G >= 16 ? 2 : 1;
         const int di = G / n, dj = G - di * n;
         int i = t / n, j = t - i * n;
         for (int e = t; e < n * n; e += kUpdate * G) {
@@ -247,10 +275,12 @@ __device__ __forceinline__ void se_block(const SEArgs &a, int64_t block, double 
 {
     const int w = threadIdx.x >> 5;
     if (w >= a.wpb) return;               // whole warp
-    const int G = se_lanes(a.L);
+    const int G = a.lanes;
     const int64_t warp = block * a.wpb + w;
     sm += (int64_t)w * (32 / G) * se_point_doubles(a.L, a.M);
-    if (G == 16)
+    if (G == 32)
+        se_warp<32>(a, warp, sm);
+    else if (G == 16)
         se_warp<16>(a, warp, sm);
     else if (G == 8)
         se_warp<8>(a, warp, sm);
@@ -286,7 +316,8 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerBlock) k_se_batch(const SEArg
     se_block(sa, (int64_t)blockIdx.x - s_first, sm);
 }
 
-SEArgs fill_se_args(const mgt_model *m)
+// Arguments of model m in a launch over `points` points.
+SEArgs fill_se_args(const mgt_model *m, int64_t points)
 {
     SEArgs a{};
     a.N = m->N;
@@ -307,14 +338,15 @@ SEArgs fill_se_args(const mgt_model *m)
     a.coll_ul = m->d_coll_ul;
     a.pops_out = m->d_pops;
     a.pops_prev = m->d_pops_prev;
+    a.lanes = se_lanes(m->L, m->M, points, se_sms());
     return a;
 }
 
 // Warps per CTA, CTAs and a CTA's dynamic shared memory (at most `most`); false
 // if no warp's points fit.
-bool se_layout(const mgt_model *m, size_t most, int *wpb, int64_t *blocks, size_t *smem)
+bool se_layout(const mgt_model *m, int lanes, size_t most, int *wpb, int64_t *blocks, size_t *smem)
 {
-    const int points = 32 / se_lanes(m->L);
+    const int points = 32 / lanes;
     const size_t per_warp = sizeof(double) * points * (size_t)se_point_doubles(m->L, m->M);
     *wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, most / per_warp);
     if (*wpb < 1) return false;
@@ -327,10 +359,10 @@ bool se_layout(const mgt_model *m, size_t most, int *wpb, int64_t *blocks, size_
 
 mgt_status launch_stat_eq(mgt_model *m, cudaStream_t s)
 {
-    SEArgs a = fill_se_args(m);
+    SEArgs a = fill_se_args(m, m->N);
     int64_t blocks = 0;
     size_t smem = 0;
-    if (!se_layout(m, kSEMaxSmem, &a.wpb, &blocks, &smem))
+    if (!se_layout(m, a.lanes, kSEMaxSmem, &a.wpb, &blocks, &smem))
         return set_error(MGT_ERR_ARG, "statistical equilibrium: too many levels/lines for shared memory");
     MGT_TRY_STATUS(raise_smem_limit((const void *)k_se, smem));
     {
@@ -343,14 +375,14 @@ mgt_status launch_stat_eq(mgt_model *m, cudaStream_t s)
 
 size_t se_args_bytes() { return sizeof(SEArgs); }
 
-mgt_status se_batch_args(const mgt_model *m, void *args, int64_t *blocks, size_t *smem)
+mgt_status se_batch_args(const mgt_model *m, int64_t points, void *args, int64_t *blocks, size_t *smem)
 {
-    SEArgs a = fill_se_args(m);
+    SEArgs a = fill_se_args(m, points);
     // the batch's documented limit
     if (4 * sizeof(double) * ((size_t)m->L * m->L + 3 * m->L + 2 * m->Mpad) > kSEMaxSmem)
         return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
     // (k_se_batch also holds a model's arguments in shared memory)
-    if (!se_layout(m, kSEMaxSmem - kSEBatchStatic, &a.wpb, blocks, smem))
+    if (!se_layout(m, a.lanes, kSEMaxSmem - kSEBatchStatic, &a.wpb, blocks, smem))
         return set_error(MGT_ERR_ARG, "batched statistical equilibrium: too many levels");
     std::memcpy(args, &a, sizeof a);
     return MGT_OK;

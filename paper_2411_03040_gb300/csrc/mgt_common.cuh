@@ -272,7 +272,7 @@ int64_t fs_batch_wave(const void *args, int threads, size_t smem);
 // run = false prepares it (kernel attributes) without launching
 mgt_status fs_batch_solo(mgt_model *m, cudaStream_t s, bool run);
 size_t se_args_bytes();
-mgt_status se_batch_args(const mgt_model *m, void *args, int64_t *blocks, size_t *smem);
+mgt_status se_batch_args(const mgt_model *m, int64_t points, void *args, int64_t *blocks, size_t *smem);
 mgt_status se_batch_prepare(size_t smem);
 mgt_status se_batch_launch(const void *d_args, const int64_t *d_blk_end, int n_models, int64_t n_blocks, size_t smem,
                            cudaStream_t s);

@@ -52,6 +52,25 @@ def test_level_and_point_edges(mgt, levels, n, batched):
     assert change == pytest.approx(np.max(np.abs(got - p0) / p0), rel=1e-9)
 
 
+# (levels, points): every number of lanes per point, whose choice depends on both
+# (152 SMs: 32 lanes up to 608 points, 16 up to 1,216, 8 up to 2,432 and 4 above
+# for up to 16 levels; 32 up to 1,216, 16 up to 2,432 and then 8 or 16 above);
+# odd counts, the last warp partly empty
+@pytest.mark.parametrize("levels,n", [(16, 607), (11, 1215), (16, 2431), (2, 2435), (16, 2435), (17, 1215), (28, 2431),
+                                      (28, 2435), (32, 2435), (48, 1219)])
+def test_lanes_per_point(mgt, levels, n):
+    m = synth.sphere_model(n, levels, 1, 3, seed=50 + levels)
+    m.n_coll = m.n_coll * 1e-4
+    h = mgt.mgt_model_create(m)
+    mgt.mgt_trace_rays(h)
+    mgt.mgt_formal_solve(h, want=False)
+    got = mgt.mgt_stat_equilibrium(h)
+    J, L = mgt.mgt_get_jbar(h)
+    p0 = O.lte_populations(m.temp, m.n_spec, m.lines.energy_J, m.lines.g)
+    ref = O.stat_equilibrium(p0, J.T, L.T, m.temp, m.n_coll, m.n_spec, m.lines)
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-8
+
+
 def test_batch_at_the_shared_memory_limit(mgt):
     # 64 levels x 340 lines: three warps of the batched kernel hold 232,320 of the
     # 232,448 bytes of shared memory that a CTA may use, and the kernel's copy of
