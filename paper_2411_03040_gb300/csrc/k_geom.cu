@@ -212,36 +212,56 @@ mgt_status build_walk_tables(mgt_model *m, const double lo[3], const double hi[3
 // ---------------------------------------------------------------------------
 // LTE: n_i = n_spec g_i exp(-(E_i - E_0)/kT) / sum_j g_j exp(-(E_j - E_0)/kT).
 // ---------------------------------------------------------------------------
-// Eight lanes per point, lanes over levels; the partition function is summed
-// in level order by every lane from shared memory.  With one thread per point
-// a small model's launch was two dependent chains of L exponentials (31 us for
-// any point count up to 20,000, now 7 us).
-constexpr int kLteThreads = 128, kLteLanes = 8;
+// G lanes per point, lanes over levels, the exponentials in shared memory; the
+// partition function is summed in level order by every lane (the same bits for
+// any G).  Few points: eight lanes, as one lane's chain of L exponentials is
+// what lasts (2,000 points, host time per call included: 41 levels 34 us with
+// two lanes, 23 with eight; 11 levels 24 with one, 18.6).  Above eight warps of
+// eight lanes per SM the FP64 pipe's instructions count, and fewer lanes serve
+// more points with each: 100k points of 3, 11 and 16 levels 34, 69 and 89 us with
+// one lane, 48, 82 and 91 with two, 72, 135 and 112 with eight; 41 levels 195 with
+// two, 288 with eight.  Each lane computing its levels' exponentials twice,
+// one lane per point, took 45, 112, 152 and 364 us there and 75 us for 2,000
+// points of 41 levels.
+constexpr int kLteThreads = 128;
 
+template <int G>
 __global__ void __launch_bounds__(kLteThreads) k_lte(int64_t N, int L, const double *__restrict__ T,
                                                      const double *__restrict__ nspec,
                                                      const double *__restrict__ level_tab, double *__restrict__ pops)
 {
-    __shared__ double ex[kLteThreads / kLteLanes][kMaxLevels];
-    const int grp = threadIdx.x / kLteLanes, t = threadIdx.x - grp * kLteLanes;
-    const int64_t p = blockIdx.x * (int64_t)(kLteThreads / kLteLanes) + grp;
+    extern __shared__ double lte_ex[];               // [kLteThreads / G][L, made odd]
+    const int grp = threadIdx.x / G, t = threadIdx.x - grp * G;
+    const int64_t p = blockIdx.x * (int64_t)(kLteThreads / G) + grp;
     const double *E = level_tab, *g = level_tab + L;
-    double beta = 0.0;
+    double *ex = lte_ex + grp * (L | 1);
     if (p < N) {
-        beta = 1.0 / (kKB * T[p]);
-        for (int i = t; i < L; i += kLteLanes) ex[grp][i] = exp(-(E[i] - E[0]) * beta);
+        const double beta = 1.0 / (kKB * T[p]);
+        for (int i = t; i < L; i += G) ex[i] = exp(-(E[i] - E[0]) * beta);
     }
     __syncwarp();
     if (p >= N) return;
     double Z = 0.0;
-    for (int i = 0; i < L; ++i) Z = __fma_rn(g[i], ex[grp][i], Z);
+    for (int i = 0; i < L; ++i) Z = __fma_rn(g[i], ex[i], Z);
     const double f = nspec[p] / Z;
-    for (int i = t; i < L; i += kLteLanes) pops[p * L + i] = __dmul_rn(__dmul_rn(f, g[i]), ex[grp][i]);
+    for (int i = t; i < L; i += G) pops[p * L + i] = __dmul_rn(__dmul_rn(f, g[i]), ex[i]);
 }
 
 mgt_status launch_lte(mgt_model *m, cudaStream_t s)
 {
-    k_lte<<<ceil_div(m->N, (int64_t)(kLteThreads / kLteLanes)), kLteThreads, 0, s>>>(m->N, m->L, m->d_temp, m->d_nspec, m->d_level_tab, m->d_pops);
+    int sms = 0;
+    MGT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
+    const auto run = [&](auto kernel, int lanes) {
+        const int points = kLteThreads / lanes;
+        kernel<<<ceil_div(m->N, (int64_t)points), kLteThreads, sizeof(double) * points * (m->L | 1), s>>>(
+            m->N, m->L, m->d_temp, m->d_nspec, m->d_level_tab, m->d_pops);
+    };
+    if (m->N * 8 <= (int64_t)sms * 8 * 32)
+        run(k_lte<8>, 8);
+    else if (m->L <= 16)
+        run(k_lte<1>, 1);
+    else
+        run(k_lte<2>, 2);
     MGT_LAUNCH_CHECK("k_lte");
     m->line_dirty = true;
     return MGT_OK;

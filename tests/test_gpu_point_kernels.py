@@ -56,3 +56,26 @@ def test_block_edges(mgt, n, levels, dense):
     scaled = mgt.mgt_get_populations(h)
     ref = got * (new / m.n_spec)[:, None]
     assert np.max(np.abs(scaled - ref) / ref) < 1e-13
+
+
+# lanes per point of the LTE kernel: eight up to 64 points per SM (4,864 on 152
+# SMs), above that one for up to 16 levels and two for more; the last block
+# full, with one point, partly filled.  The arithmetic does not depend on it:
+# every population is that of the same points in a model of half the size, bit
+# for bit, down to levels that underflow
+@pytest.mark.parametrize("n,levels", [(4864, 16), (4865, 2), (4993, 16), (5000, 17), (4929, 64)])
+def test_lte_lanes_per_point(mgt, n, levels):
+    rng = np.random.default_rng(n)
+    nbrs = np.stack([np.arange(1, n + 1) % n, np.arange(-1, n - 1) % n], axis=1)
+    m = synth.Model("ring", rng.uniform(-1, 1, (n, 3)) * 1e11, np.zeros((n, 3)), rng.uniform(5.0, 500.0, n),
+                    np.full(n, 1e4), np.full(n, 1e10), rng.uniform(1e3, 1e6, n), 2 * np.arange(n + 1, dtype=np.int64),
+                    np.sort(nbrs, axis=1).astype(np.int32).ravel(), np.array([0], np.int32),
+                    synth.healpix_directions(1), 3, synth.linear_rotor(levels, rng))
+    got = mgt.mgt_get_populations(mgt.mgt_model_create(m))
+    for half in (slice(0, n // 2), slice(n // 2, n)):
+        k = half.stop - half.start
+        nb = np.stack([np.arange(1, k + 1) % k, np.arange(-1, k - 1) % k], axis=1)
+        part = synth.Model("part", m.pos[half], m.vel[half], m.temp[half], m.vturb2[half], m.n_coll[half],
+                           m.n_spec[half], 2 * np.arange(k + 1, dtype=np.int64),
+                           np.sort(nb, axis=1).astype(np.int32).ravel(), np.array([0], np.int32), m.dirs, 3, m.lines)
+        np.testing.assert_array_equal(mgt.mgt_get_populations(mgt.mgt_model_create(part)), got[half])
