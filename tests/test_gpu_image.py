@@ -334,3 +334,30 @@ def test_anchors_of_a_small_cloud_far_away_with_a_rounded_direction(mgt):
     for scale in (1.0 - 4.9e-13, 1.0 + 4.9e-13):
         anchor, _, _ = mgt.mgt_image_rays(h, d * scale, 80, 80)
         assert np.array_equal(anchor, O.image_rays(m, d * scale, 80, 80).anchor)
+
+
+def test_held_view_read_on_two_streams(mgt):
+    # the kept pixel rays are read on a second stream while the first one asks
+    # for another view: its rays must not be written over those being read.
+    # The images of one stream alone, bit for bit
+    import torch
+    m = synth.sphere_model(3000, 5, 1, 5, seed=12)
+    lo, hi = _band(m)
+    views = [DIR, -DIR, np.array([0.0, 0.0, 1.0])]
+    px, nf = 96, 200
+    h = mgt.mgt_model_create(m)
+    out = [torch.empty((nf, px, px), dtype=torch.float32, device="cuda") for _ in range(6)]
+    for v, o in zip(views, out):
+        mgt.mgt_image(h, v, px, px, nf, lo, hi, out=o)
+    torch.cuda.synchronize()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(3):
+        for k in (0, 1):
+            for o in out[3:]:
+                o.zero_()
+            torch.cuda.synchronize()
+            mgt.mgt_image(h, views[k], px, px, nf, lo, hi, out=out[3], stream=s1)
+            mgt.mgt_image(h, views[k], px, px, nf, lo, hi, out=out[4], stream=s2)
+            mgt.mgt_image(h, views[k + 1], px, px, nf, lo, hi, out=out[5], stream=s1)
+            torch.cuda.synchronize()
+            assert torch.equal(out[3], out[k]) and torch.equal(out[4], out[k]) and torch.equal(out[5], out[k + 1])
