@@ -692,7 +692,8 @@ struct ImgWalkArgs {
 // L1.  Walk kernel, 100k shell points x 48 directions (1.9e8 steps): 36.9 ms
 // with 16 lanes per walk, records made inside, 64 registers; 16.0 ms with 4
 // lanes and the records left to k_walk_compact; 14.9 ms at 48 registers (ten
-// blocks of 128 threads per SM; 16.0 at eight, 18.8 at six, 17.5 at fourteen);
+// blocks of 128 threads per SM, and 32 to 44 bytes of spills; 16.0 at eight, 18.8
+// at six, 17.5 at fourteen);
 // 14.4 ms with 256-bit loads; 13.2 ms with the bounds above.  Before those, 8
 // lanes per walk took 18.7 ms, 2 lanes 16.2 ms.
 // Not kept: loading the next chunk ahead (16.8 ms, a quarter of the loads
